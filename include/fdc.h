@@ -270,17 +270,19 @@ int fdc_decode_attn_static(fdc_plan* plan, const fdc_kv_desc* kv, int32_t layer,
  * synchronising `stream`.  *host_bits receives the FDC_DEV_* bits; returns FDC_ERR_DEVICE if non-zero. */
 int fdc_status(fdc_plan* plan, int32_t* host_bits, int32_t clear, void* stream);
 
-/* Selects the split-pass kernel: 0 = automatic (3 for bf16, 1 for fp32), 1 = CUDA-core kernel
- * (any dtype), 2 = TMA + mma.sync kernel (bf16), 3 = TMA + tcgen05/TMEM kernel (bf16, head_dim
- * 128; head_dim 64 takes 2).  Unsupported combinations use 1. */
+/* Selects the split-pass kernel: 0 = automatic (fp32: 1; bf16: 3, or 2 for head_dim 64 and where
+ * the shapes say that 2 is faster: few scenes, short prefixes), 1 = CUDA-core kernel (any dtype), 2 = TMA +
+ * mma.sync kernel, one thread-block cluster per (scene, KV head) or per share of its query rows
+ * (bf16), 3 = TMA + tcgen05/TMEM kernel (bf16, head_dim 128; head_dim 64 takes 2).  Unsupported
+ * combinations use 1. */
 int fdc_set_attn_kernel(fdc_plan* plan, int32_t which);
 const char* fdc_kernel_name(int32_t which);
 
 /* Fused append (off by default; Sec. 3.3's shared cache, written and read in one kernel).  While
- * on, an fdc_kv_append on this plan whose cache the tcgen05 attention kernel serves (bf16,
- * head_dim 128) launches nothing: its arguments are recorded, and the NEXT fdc_decode_attn for
+ * on, an fdc_kv_append on this plan whose cache a tensor-core attention kernel serves (bf16, not
+ * with kernel 1 selected) launches nothing: its arguments are recorded, and the NEXT fdc_decode_attn for
  * the same cache, layer, stream and d_n_active writes the rows inside its own kernel, each by
- * the thread block that owns the row's KV tile, before that block loads the tile.  One kernel
+ * the thread block that owns the row's KV tile.  One kernel
  * per layer instead of two dependent ones.  Until that call returns the caller must not read
  * the rows from the cache, and must leave d_n_active, d_kv_row, d_k_new and d_v_new as they
  * were.  Any other call on the plan (another append, an attention call that does not match,

@@ -47,12 +47,54 @@ void prof_destroy(fdc_plan* p)
     p->prof = nullptr;
 }
 
-// The conditions under which fdc_decode_attn runs the tcgen05 kernel with the combine fused in
-// (the only kernel that can also carry out a recorded append).
-bool takes_tc_kernel(const fdc_plan* p, const fdc_kv_desc* kv)
+// Estimated time (us) of a launch of the tcgen05 kernel: fitted, like the cluster kernel's, to the 168 shapes
+// with head_dim 128 of the same measurement.  A launch costs a chain of latencies plus the rounds of 128 KV rows of
+// its busiest block, both growing with the width of the build (32, 64 or 128 query rows), and every further
+// pair that a block has to finish costs about as much as a launch.
+static float tc_estimate(const ClusterProblem& c)
 {
-    return kv->dtype == FDC_BF16 && kv->head_dim == 128 && (p->attn_kernel == 0 || p->attn_kernel == 3) &&
-           (long long)p->h.max_active * (kv->hq / kv->hkv) <= 128 && (long long)kv->batch * kv->hkv <= FDC_PAIR_COUNTERS;
+    const int k = c.mmax <= 32 ? 0 : (c.mmax <= 64 ? 1 : 2);
+    static const float fixed[] = {11.9f, 17.7f, 20.3f}, round[] = {1.63f, 2.0f, 4.9f};
+    const float rows = (float)c.P + 0.5f * (float)c.T, rounds = rows / 128.f, pairs = (float)c.pairs, sms = (float)c.sm_count;
+    const float busiest = fmaxf(fminf(4.f, rounds), pairs * rounds / sms);
+    const float t_mem = 8.f + pairs * rows * 512e-6f / 6.2f;
+    return fmaxf(fixed[k] + round[k] * busiest + 20.f * fmaxf(0.f, pairs / sms - 1.f), t_mem);
+}
+
+// The cluster kernel's cut of this problem and whether it is the faster kernel (kept in the plan: both follow
+// from the shapes alone).  Where both kernels can run, the cluster kernel is taken if its estimate is below 0.85
+// of the other's: with that factor 87 of the 168 shapes go to it, at 0.82 of the tcgen05 kernel's time over all
+// of them (1 scene x 7 query rows 14.5 -> 7.0 us a layer, 1 scene x 42 rows 19.3 -> 10.4, 16 scenes x 24 rows
+// at prefix 4096 stay at 53), and two of them are slower, by 4 and 6 %.
+static const ClusterShape& route(fdc_plan* p, const fdc_kv_desc* kv)
+{
+    const ClusterProblem c{(int64_t)kv->batch * kv->hkv, p->h.max_active * (kv->hq / kv->hkv), kv->head_dim, p->h.P, p->h.T, p->sm_count};
+    if (!(p->route_for == c)) {
+        float us = 0.f;
+        p->route_shape = pick_cluster(c, &us);
+        p->route_cluster = kv->head_dim != 128 || us < 0.85f * tc_estimate(c);
+        p->route_for = c;
+    }
+    return p->route_shape;
+}
+
+// bf16 launches that go to the cluster kernel: those asked for by name (2), those with head_dim 64, and, left to
+// the library (0), those it is the faster kernel for.
+bool takes_cluster_kernel(fdc_plan* p, const fdc_kv_desc* kv)
+{
+    if (kv->dtype != FDC_BF16 || p->attn_kernel == 1) return false;
+    if (p->attn_kernel == 2 || kv->head_dim != 128) return true;
+    if (p->attn_kernel == 3) return false;
+    route(p, kv);
+    return p->route_cluster != 0;
+}
+
+// Both tensor-core kernels can carry out a recorded append (the tcgen05 kernel while it merges its partials itself).
+bool fuses_append(fdc_plan* p, const fdc_kv_desc* kv)
+{
+    if (kv->dtype != FDC_BF16 || p->attn_kernel == 1) return false;
+    if ((long long)p->h.max_active * (kv->hq / kv->hkv) > 128) return false;
+    return takes_cluster_kernel(p, kv) || (long long)kv->batch * kv->hkv <= FDC_PAIR_COUNTERS;
 }
 }  // namespace fdc
 
@@ -142,7 +184,7 @@ int fdc_decode_attn(fdc_plan* p, const fdc_kv_desc* kv, int32_t layer, const int
     // a recorded append is carried out by this call's kernel if it belongs to it, else on its own first
     fdc_pending_append app = p->pend;
     if (app.valid) {
-        const bool mine = takes_tc_kernel(p, kv) && app.kv.k == kv->k && app.kv.v == kv->v && app.layer == layer &&
+        const bool mine = fuses_append(p, kv) && app.kv.k == kv->k && app.kv.v == kv->v && app.layer == layer &&
                           app.stream == stream && app.d_n_active == d_n_active && app.kv.stride_layer == kv->stride_layer;
         if (mine) {
             p->pend.valid = 0;
@@ -199,62 +241,62 @@ int fdc_decode_attn(fdc_plan* p, const fdc_kv_desc* kv, int32_t layer, const int
     a.pair_cnt = nullptr;
     a.split_memo = nullptr;
     a.seq = 0;
-    a.early = 0;
-    bool fused = false;                 // the split kernel merged the partials itself
-    if (kv->dtype == FDC_BF16 && (p->attn_kernel == 0 || p->attn_kernel == 3)) {
-        if ((long long)kv->batch * kv->hkv <= FDC_PAIR_COUNTERS) a.pair_cnt = p->d_pair_cnt;
-        a.split_memo = (a.pair_cnt && kv->batch <= FDC_MEMO_BATCH && a.n_cta <= FDC_MEMO_CTAS) ? p->d_split_memo : nullptr;
-        // The work split depends only on the pass tables, so it is computed once per pass, by a launch
-        // of its own ahead of the pass's first attention launch (an ordinary launch: it begins after
-        // everything before it in the stream has completed).
-        bool split_now = false;
-        if (a.split_memo) {
-            const fdc_split_key& k = p->split_key;
-            split_now = !k.valid || k.tables_gen != p->tables_gen || k.d_n_active != d_n_active || k.d_ntiles != d_ntiles ||
-                        k.batch != kv->batch || k.hkv != kv->hkv || k.n_cta != a.n_cta || k.P != a.P || k.stream != stream;
-            if (split_now) {
-                a.seq = ++p->split_gen;
-                a.early = 0;
-                rc = launch_attn_tc_split(a, kv->head_dim, st);
-                if (rc == FDC_OK) {
-                    p->split_key = fdc_split_key{p->tables_gen, d_n_active, d_ntiles, kv->batch, kv->hkv, a.n_cta, a.P, stream, 1};
-                } else {
-                    p->split_key.valid = 0;
-                    a.split_memo = nullptr;
-                    split_now = false;
+    bool fused = false;                 // the kernel merged the partials itself
+    // Reading ahead of the dependency wait: allowed from the second attention launch of a pass on
+    // the same stream.  The first one waits for everything before it (the pass tables, the split)
+    // before it lets the next kernel begin, and no kernel begins before the one ahead of it in the
+    // stream has let it, so whatever runs later finds those complete.
+    a.early = (p->attn_gen == p->tables_gen && p->attn_stream == stream && p->attn_gen_valid) ? 1 : 0;
+    if (app.valid) {
+        a.app_row = app.d_kv_row;
+        a.app_k = app.d_k_new;
+        a.app_v = app.d_v_new;
+    }
+    if (kv->dtype == FDC_BF16 && p->attn_kernel != 1) {
+        if (!takes_cluster_kernel(p, kv)) {
+            if ((long long)kv->batch * kv->hkv <= FDC_PAIR_COUNTERS) a.pair_cnt = p->d_pair_cnt;
+            a.split_memo = (a.pair_cnt && kv->batch <= FDC_MEMO_BATCH && a.n_cta <= FDC_MEMO_CTAS) ? p->d_split_memo : nullptr;
+            // The work split depends only on the pass tables, so it is computed once per pass, by a launch
+            // of its own ahead of the pass's first attention launch (an ordinary launch: it begins after
+            // everything before it in the stream has completed).
+            if (a.split_memo) {
+                const fdc_split_key& k = p->split_key;
+                const bool split_now = !k.valid || k.tables_gen != p->tables_gen || k.d_n_active != d_n_active || k.d_ntiles != d_ntiles ||
+                                       k.batch != kv->batch || k.hkv != kv->hkv || k.n_cta != a.n_cta || k.P != a.P || k.stream != stream;
+                if (split_now) {
+                    a.seq = ++p->split_gen;
+                    a.early = 0;
+                    if (launch_attn_tc_split(a, kv->head_dim, st) == FDC_OK) {
+                        p->split_key = fdc_split_key{p->tables_gen, d_n_active, d_ntiles, kv->batch, kv->hkv, a.n_cta, a.P, stream, 1};
+                    } else {
+                        p->split_key.valid = 0;
+                        a.split_memo = nullptr;
+                    }
                 }
-                rc = FDC_ERR_SHAPE;
+                a.seq = p->split_gen;
             }
-            a.seq = p->split_gen;
+            rc = launch_attn_tc(a, kv->head_dim, st);
+            fused = rc == FDC_OK && a.pair_cnt != nullptr;
+            a.pair_cnt = nullptr;
+            a.split_memo = nullptr;
         }
-        // Reading ahead of the dependency wait: allowed from the second attention launch of a pass on
-        // the same stream.  The first one waits for everything before it (the pass tables, the split)
-        // before it lets the next kernel begin, and no kernel begins before the one ahead of it in the
-        // stream has let it, so whatever runs later finds those complete.
-        a.early = (!split_now && p->attn_gen == p->tables_gen && p->attn_stream == stream && p->attn_gen_valid) ? 1 : 0;
-        if (app.valid) {
-            a.app_row = app.d_kv_row;
-            a.app_k = app.d_k_new;
-            a.app_v = app.d_v_new;
+        if (rc == FDC_ERR_SHAPE) {
+            a.cluster = route(p, kv);
+            rc = launch_attn_cluster(a, kv->head_dim, st);
+            fused = rc == FDC_OK;
         }
-        rc = launch_attn_tc(a, kv->head_dim, st);
         if (rc == FDC_OK) {
             p->attn_gen = p->tables_gen;
             p->attn_stream = stream;
             p->attn_gen_valid = 1;
         }
-        a.app_row = nullptr;
-        if (app.valid && rc != FDC_OK) {
-            // the kernel that would have written the rows was not launched: append on its own after all
-            int rca = launch_kv_append(p, kv, layer, app.d_n_active, app.d_kv_row, app.d_k_new, app.d_v_new, stream);
-            if (rca) return rca;
-        }
-        fused = rc == FDC_OK && a.pair_cnt != nullptr;
-        a.pair_cnt = nullptr;
-        a.split_memo = nullptr;
     }
-    if (kv->dtype == FDC_BF16 && (p->attn_kernel == 2 || (rc == FDC_ERR_SHAPE && p->attn_kernel != 1)))
-        rc = launch_attn_mma(a, kv->head_dim, st);
+    a.app_row = nullptr;
+    if (app.valid && rc != FDC_OK) {
+        // the kernel that would have written the rows was not launched: append on its own after all
+        int rca = launch_kv_append(p, kv, layer, app.d_n_active, app.d_kv_row, app.d_k_new, app.d_v_new, stream);
+        if (rca) return rca;
+    }
     if (rc == FDC_ERR_SHAPE) rc = launch_attn_ref(a, kv->dtype, kv->head_dim, st);
     if (rc) return rc;
     if (pr) cudaEventRecord(e1, st);

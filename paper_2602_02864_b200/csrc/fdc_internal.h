@@ -59,6 +59,22 @@ struct fdc_pending_append {
     void*          stream;
 };
 
+namespace fdc {
+// How the cluster kernel (fdc_attn_cluster.cu) cuts a launch.
+struct ClusterShape {
+    int nblk, qsplit, per_sm;        // blocks per cluster, clusters per (scene, KV head) pair, blocks per SM (1 or 2)
+};
+struct ClusterProblem {
+    int64_t pairs;
+    int32_t mmax, head_dim, P, T, sm_count;
+    bool operator==(const ClusterProblem& o) const
+    {
+        return pairs == o.pairs && mmax == o.mmax && head_dim == o.head_dim && P == o.P && T == o.T && sm_count == o.sm_count;
+    }
+};
+ClusterShape pick_cluster(const ClusterProblem& c, float* us);      // us (may be NULL): the estimated time
+}  // namespace fdc
+
 // Everything the work split of the tcgen05 attention kernel depends on (host side).
 struct fdc_split_key {
     uint32_t       tables_gen;
@@ -87,6 +103,9 @@ struct fdc_plan {
     int           device;
     int           sm_count;
     int           attn_kernel;       // 0 auto
+    fdc::ClusterProblem route_for;   // the problem `route_shape` / `route_cluster` were chosen for (sm_count 0: none yet)
+    fdc::ClusterShape   route_shape;
+    int           route_cluster;     // with attn_kernel 0: the cluster kernel is the faster one
     void*         prof;              // event records of fdc_profile (nullptr when never enabled)
     int           prof_on;
     int32_t*      succ_ptr;          // host CSR successor lists (kept for inspection)
@@ -116,6 +135,7 @@ struct AttnParams {
     uint32_t        seq;             // number of the split launch the memo must come from
     int32_t         early;           // the pass tables, the memo and the prefix rows were complete before the kernel
                                      // preceding this one in the stream began: they may be read ahead of the dependency wait
+    ClusterShape    cluster;         // cut of the launch (cluster kernel)
     const int32_t*  app_row;         // fused append: [batch][max_active] cache row of each branch's new K/V vector (nullptr: none)
     const void*     app_k;           // [batch][max_active][hkv][D]
     const void*     app_v;
@@ -126,13 +146,14 @@ void note_launch();
 int  set_cuda_error(cudaError_t e);                  // records the message, returns FDC_ERR_CUDA
 
 int launch_attn_ref(const AttnParams& p, int dtype, int head_dim, cudaStream_t st);
-int launch_attn_mma(const AttnParams& p, int head_dim, cudaStream_t st);
+int launch_attn_cluster(const AttnParams& p, int head_dim, cudaStream_t st);
 int launch_attn_tc(const AttnParams& p, int head_dim, cudaStream_t st);
 int launch_attn_tc_split(const AttnParams& p, int head_dim, cudaStream_t st);   // computes the work split only (into p.split_memo)
 int launch_attn_combine(const AttnParams& p, int dtype, int head_dim, cudaStream_t st);
 void prof_destroy(fdc_plan* plan);
 int  check_kv_desc(const fdc_plan* plan, const fdc_kv_desc* kv, int32_t layer);
-bool takes_tc_kernel(const fdc_plan* plan, const fdc_kv_desc* kv);   // fdc_decode_attn would run the tcgen05 kernel with the combine fused in
+bool takes_cluster_kernel(fdc_plan* plan, const fdc_kv_desc* kv);    // fdc_decode_attn would run the cluster kernel (else: the tcgen05 kernel, for bf16)
+bool fuses_append(fdc_plan* plan, const fdc_kv_desc* kv);            // ... and the kernel it would run can carry out a recorded append
 int  launch_kv_append(fdc_plan* plan, const fdc_kv_desc* kv, int32_t layer, const int32_t* d_n_active, const int32_t* d_kv_row,
                       const void* d_k_new, const void* d_v_new, void* stream);
 int  flush_pending_append(fdc_plan* plan);     // launches a recorded append on its own (no-op when there is none)

@@ -181,7 +181,7 @@ extern "C" int fdc_kv_append(fdc_plan* p, const fdc_kv_desc* kv, int32_t layer, 
     if (((uintptr_t)d_k_new & 15) || ((uintptr_t)d_v_new & 15)) return FDC_ERR_SHAPE;
     rc = flush_pending_append(p);                 // an earlier recorded append never met its attention call
     if (rc) return rc;
-    if (p->fuse_append && takes_tc_kernel(p, kv)) {
+    if (p->fuse_append && fuses_append(p, kv)) {
         // recorded only: the next fdc_decode_attn for this cache, layer and stream writes the rows itself
         fdc_pending_append& pe = const_cast<fdc_plan*>(p)->pend;
         pe.kv = *kv;

@@ -1,0 +1,25 @@
+"""The cluster kernel (fdc_set_attn_kernel 2; the automatic choice for head_dim 64 and for small passes)
+against the CPU checker at the sizes where its splits, rings and groups can go wrong."""
+import pytest
+
+from harness import run_and_compare
+from paper_2602_02864_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+# query rows per pair (hq / hkv x fields) around the group sizes 16 / 32 / 64 / 128; blocks per pair 16, 8, a
+# few, one; prefixes that are and are not whole tiles, empty, shorter than one stage; runs much longer
+# than the ring (few blocks per pair and a long prefix: every stage is reused many times)
+@pytest.mark.parametrize("head_dim,hq,hkv,fields,batch,prefix", [
+    (64, 14, 2, 1, 1, 31), (64, 14, 2, 5, 1, 1531), (64, 4, 2, 8, 3, 640), (64, 14, 2, 9, 24, 2100), (64, 4, 2, 32, 40, 1000),
+    (64, 16, 1, 8, 200, 1024), (64, 2, 2, 17, 2, 0),
+    (128, 4, 4, 1, 1, 64), (128, 28, 4, 3, 1, 4095), (128, 32, 8, 4, 6, 3000), (128, 32, 8, 9, 19, 2048), (128, 8, 2, 32, 5, 1025),
+    (128, 16, 8, 8, 20, 4000), (128, 8, 8, 20, 2, 97)])
+def test_cluster_kernel_shapes(head_dim, hq, hkv, fields, batch, prefix):
+    w = wl.random_template(7100 + fields + batch, n_nodes=fields, edge_prob=0.15, cap_lo=2, cap_hi=70, batch=batch, prefix_len=prefix, fixed_hi=2,
+                           hq=hq, hkv=hkv, head_dim=head_dim, dtype="bf16")
+    w.max_active = w.n_nodes
+    steps = {0, 1, 9, 33}
+    r = run_and_compare(w, check_steps=steps, kernel=2, max_steps=34)
+    assert r["checked"] > 0
