@@ -285,11 +285,15 @@ int fdc_decode_attn(fdc_plan* p, const fdc_kv_desc* kv, int32_t layer, const int
             rc = launch_attn_cluster(a, kv->head_dim, st);
             fused = rc == FDC_OK;
         }
-        if (rc == FDC_OK) {
-            p->attn_gen = p->tables_gen;
-            p->attn_stream = stream;
-            p->attn_gen_valid = 1;
-        }
+    }
+    if (kv->dtype == FDC_F32 && p->attn_kernel == 0) {
+        rc = launch_attn_f32(a, kv->head_dim, st);
+        fused = rc == FDC_OK;
+    }
+    if (rc == FDC_OK) {
+        p->attn_gen = p->tables_gen;
+        p->attn_stream = stream;
+        p->attn_gen_valid = 1;
     }
     a.app_row = nullptr;
     if (app.valid && rc != FDC_OK) {

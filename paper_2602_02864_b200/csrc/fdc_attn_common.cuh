@@ -133,8 +133,8 @@ __device__ __forceinline__ Segment decode_segment(long long u, long long hi, con
 }
 
 
-// Host: a cached 4-D tensor map (head_dim, rows, hkv, batch) of a bf16 cache with boxes of
-// 64 elements x box_rows rows and 128-byte swizzle.  out_map points to a CUtensorMap.
-int get_kv_tensor_map(const void* base, const AttnParams& p, int head_dim, int box_rows, void* out_map);
+// Host: a cached 4-D tensor map (head_dim, rows, hkv, batch) of a cache (dtype FDC_F32 or FDC_BF16) with
+// boxes of 128 bytes x box_rows rows and 128-byte swizzle.  out_map points to a CUtensorMap.
+int get_kv_tensor_map(const void* base, const AttnParams& p, int dtype, int head_dim, int box_rows, void* out_map);
 
 }  // namespace fdc

@@ -1816,9 +1816,9 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     const int nk = stages / 2, nv = stages - nk;
     const size_t smem = fixed + (size_t)stages * STAGE;
     alignas(64) CUtensorMap tk, tv;
-    int rc = get_kv_tensor_map(p.k, p, D, TILE, &tk);
+    int rc = get_kv_tensor_map(p.k, p, FDC_BF16, D, TILE, &tk);
     if (rc) return rc;
-    rc = get_kv_tensor_map(p.v, p, D, TILE, &tv);
+    rc = get_kv_tensor_map(p.v, p, FDC_BF16, D, TILE, &tv);
     if (rc) return rc;
     static size_t attr_smem[kMaxDevices] = {};
     rc = raise_dynamic_smem(reinterpret_cast<const void*>(FDC_TC_KERNEL), smem, attr_smem);

@@ -1,0 +1,630 @@
+// A (scene, KV head) pair's attention by thread-block clusters: what the bf16 kernel (fdc_attn_cluster.cu) and
+// the fp32 kernel (fdc_attn_f32.cu) share.  The blocks of a cluster take equal runs of the pair's tile parts (16
+// or 32 rows), a block's warps take the run's stages in turn, and the partial results meet in (distributed)
+// shared memory.  A kernel's arithmetic is its class `Math`:
+//   Elem, D                 cache element and head_dim
+//   NW                      warps of a block
+//   SROWS                   KV rows of a stage: a part of a 64-row tile (16 or 32)
+//   GROWS, GROUPS           query rows of a group; groups of a cluster at most (a power of two)
+//   ROWS, row(i)            query rows a thread needs visibility bits for
+//   STAGE_BYTES             SROWS rows of K, then of V, in panels of [SROWS rows][128 bytes] (128-byte swizzle)
+//   K_REUSED                stage() writes over the stage's K rows
+//   PREFIX_FIRST, FUSES     report a tile list that does not begin with the prefix; carry out recorded appends
+//   q_off                   place of a 16-byte chunk of a query row in shared memory
+//   stage(), write()        one stage for one warp (shared: other groups work on it too; k_read() is called by every warp once
+//                           it has read the stage's K rows for the last time and returns when all groups have); the warp's
+//                           accumulators and (m, l) to shared memory
+//   part_off, store         float offset of (row, column) of a partial; four results to the output
+#pragma once
+
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <atomic>
+#include <type_traits>
+
+#include "fdc_attn_common.cuh"
+
+namespace fdc {
+
+constexpr int MAX_STAGES = 16;
+constexpr int MASK_WORDS = 1024;              // (tile part, field) visibility words kept in shared memory
+constexpr int MASK_HALVES = 64;               // tile parts among them at most
+constexpr int ROW0S = 256;                    // tile parts of the run whose first row is kept in shared memory
+
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Byte offset of the 16-byte chunk `dc` (0 .. D/8-1) of row `r` of an operand in panels of `panel` bytes
+// ([rows][128 bytes], 64 bf16 columns each) with the 128-byte swizzle TMA applies: inside a panel the
+// chunk index is XORed with (row mod 8).
+__device__ __forceinline__ uint32_t swz(uint32_t panel, int r, int dc)
+{
+    return (uint32_t)(dc >> 3) * panel + (uint32_t)(r * 128 + (((dc & 7) ^ (r & 7)) << 4));
+}
+
+// 16-byte asynchronous copy global -> shared (zero fill when !valid).
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, bool valid)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+
+// Visibility of the SROWS rows row0.. for one field: prefix rows are all visible.
+template <int SROWS>
+__device__ __forceinline__ uint32_t part_bits(const uint64_t* __restrict__ words, int W, int P, int row0)
+{
+    constexpr uint32_t all = SROWS == 32 ? ~0u : (1u << (SROWS & 31)) - 1u;
+    const int npre = P - row0;
+    if (npre >= SROWS) return all;
+    return ((npre <= 0 ? 0u : ((1u << npre) - 1u)) | (uint32_t)extract64(words, W, row0 - P)) & all;
+}
+
+template <int N, class F, int I = 0>
+__device__ __forceinline__ void static_for(F&& f)
+{
+    if constexpr (I < N) {
+        f(std::integral_constant<int, I>{});
+        static_for<N, F, I + 1>(static_cast<F&&>(f));
+    }
+}
+
+// Waits until stage `slot` has been asked for at least `n` times.  The warps that use a slot in turn need
+// not be the same ones, and a parity wait tells only two consecutive phases of a barrier apart: a warp
+// that ran ahead would take the phase before the previous use for its own.  Once the n-th request has
+// been made the previous use is over, so the barrier is in the n-th phase or just past it.  Bounded
+// like every in-kernel wait.
+static __device__ __noinline__ bool wait_asked_slow(volatile int* asked, int n, volatile int* abort_flag, int32_t* status)
+{
+    for (uint32_t i = 0; i < SPIN_LIMIT * 16; ++i) {
+        if (*asked >= n) return true;
+        if ((i & 255u) == 255u && *abort_flag) return false;
+        __nanosleep(32);
+    }
+    *abort_flag = 1;
+    atomicOr(status, FDC_DEV_TIMEOUT);
+    return false;
+}
+__device__ __forceinline__ bool wait_asked(volatile int* asked, int n, volatile int* abort_flag, int32_t* status)
+{
+    return *asked >= n || wait_asked_slow(asked, n, abort_flag, status);
+}
+
+template <int NW, int GROWS>
+struct __align__(16) BlockState {
+    uint64_t full[MAX_STAGES];
+    uint64_t k_read[MAX_STAGES];              // all groups have read the stage's K rows (kernels that reuse their place)
+    int used[MAX_STAGES];                     // groups that have finished with the stage
+    int asked[MAX_STAGES];                    // requests made for the stage so far
+    int abort_flag;                           // a bounded wait ran out somewhere in the block
+    int first_beyond;                         // first part of the run that reaches beyond the prefix
+    int n_kept;                               // entries of kept[]
+    int pad;
+    float2 wml[NW * GROWS];                   // (m, l) per warp and row of its group ([lane][query row])
+    float2 cml[128];                          // (m, l) of the block per query row
+    int app_row[FDC_MAX_NODES];               // fused append: cache row of every field's new K/V vector, -1: not written
+    uint32_t newbits[2 * FDC_MAX_NODES];      // [new rows 0-31, 32-63][field] the new rows that the field sees
+    uint32_t seen[MASK_HALVES];               // rows of a tile part that some field sees
+    uint8_t kept[MASK_HALVES];                // those of them that hold a visible row, in order
+    uint32_t bits[MASK_WORDS];                // [part][field] the rows that the field sees
+    int row0[ROW0S];                          // first KV row of the run's parts
+};
+
+// The block's run of tile parts: positions [h0, h1) of the pair's list (each 64-row tile is two or four of them).
+// Positions p0 .. p0 + np - 1 have their visibility in shared memory; those of them that hold no
+// visible row are left out, so the i-th part that is loaded is not always position h0 + i.
+struct Run {
+    const int32_t* tiles;                     // the scene's tile list
+    const uint64_t* mask;                     // the scene's bitmaps
+    int h0, h1, p0, np;
+    int nx;                                   // stages of new rows, ahead of the tile parts
+    int total;                                // stages
+};
+template <int SROWS, class Block>
+__device__ __forceinline__ int part_row0(const Run& r, const Block& bs, int pos)
+{
+    const int i = pos - r.h0;
+    return i < ROW0S ? bs.row0[i] : r.tiles[pos / (FDC_TILE_ROWS / SROWS)] * FDC_TILE_ROWS + pos % (FDC_TILE_ROWS / SROWS) * SROWS;
+}
+template <class Block>
+__device__ __forceinline__ int stage_pos(const Run& r, const Block& bs, int it)
+{
+    const int i = it - r.nx - (r.p0 - r.h0);
+    if (i < 0) return r.h0 + it - r.nx;
+    return i < bs.n_kept ? r.p0 + bs.kept[i] : r.p0 + r.np + (i - bs.n_kept);
+}
+// Rows of the tile part that some field sees (whole warp).
+template <int SROWS>
+__device__ __noinline__ uint32_t part_seen_slow(const uint64_t* mask, int W, int P, int A, int row0)
+{
+    uint32_t x = 0u;
+    for (int b = threadIdx.x & 31; b < A; b += 32) x |= part_bits<SROWS>(mask + (size_t)b * W, W, P, row0);
+    return __reduce_or_sync(0xffffffffu, x);
+}
+
+// The new rows of this pass among the SROWS rows row0.. (their values come from the stage of new rows).
+template <int SROWS>
+__device__ __noinline__ uint32_t new_rows_of(const int* app_row, int A, int row0)
+{
+    uint32_t x = 0u;
+    for (int b = threadIdx.x & 31; b < A; b += 32) {
+        const int i = app_row[b] - row0;
+        if (i >= 0 && i < SROWS) x |= 1u << i;
+    }
+    return __reduce_or_sync(0xffffffffu, x);
+}
+
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ float2 ld_cluster2(uint32_t addr)
+{
+    float2 v;
+    asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(uint32_t addr)
+{
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+// Merge over the lanes of a block, for every (query row, 4 columns): `rows` = query rows of a lane's partial;
+// `done(row, column, m, l, sum)` takes the result.
+template <class Math, int L, class F>
+__device__ __forceinline__ void merge_lanes_n(int tid, int M, int rows, const float2* ml, const float* part, F&& done)
+{
+    constexpr int D = Math::D;
+    for (int idx = tid; idx < M * (D / 4); idx += Math::NW * 32) {
+        const int mm = idx / (D / 4), c4 = (idx - mm * (D / 4)) * 4;
+        float4 x[L];
+        float2 v[L];
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            v[k] = ml[mm + k * rows];
+            x[k] = *reinterpret_cast<const float4*>(part + k * rows * D + Math::part_off(mm, c4));
+        }
+        float mx = v[0].x;
+#pragma unroll
+        for (int k = 1; k < L; ++k) mx = fmaxf(mx, v[k].x);
+        const float ms = mx == -INFINITY ? 0.f : mx;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float lt = 0.f;
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            const float w = fast_exp2(v[k].x - ms);
+            lt = fmaf(v[k].y, w, lt);
+            acc.x = fmaf(x[k].x, w, acc.x);
+            acc.y = fmaf(x[k].y, w, acc.y);
+            acc.z = fmaf(x[k].z, w, acc.z);
+            acc.w = fmaf(x[k].w, w, acc.w);
+        }
+        done(mm, c4, mx, lt, acc);
+    }
+}
+template <class Math, class F>
+__device__ __forceinline__ void merge_lanes(int lanes, int tid, int M, int rows, const float2* ml, const float* part, F&& done)
+{
+    if constexpr (Math::NW == 8) {
+        switch (lanes) {
+            case 1: return merge_lanes_n<Math, 1>(tid, M, rows, ml, part, done);
+            case 2: return merge_lanes_n<Math, 2>(tid, M, rows, ml, part, done);
+            case 4: return merge_lanes_n<Math, 4>(tid, M, rows, ml, part, done);
+            default: return merge_lanes_n<Math, 8>(tid, M, rows, ml, part, done);
+        }
+    } else {
+        static_assert(Math::NW == 12 && Math::GROUPS <= 2, "lanes of a group");
+        if (lanes == 6) merge_lanes_n<Math, 6>(tid, M, rows, ml, part, done);
+        else merge_lanes_n<Math, 12>(tid, M, rows, ml, part, done);
+    }
+}
+
+// The kernel (two blocks' worth of arguments beyond AttnParams: ring slots, blocks per cluster, clusters per
+// pair, query rows per cluster).
+template <class Math>
+__device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const int nstage, const int nblk,
+                                                  const int qsplit, const int qrows)
+{
+    constexpr int D = Math::D, GROWS = Math::GROWS, STAGE_BYTES = Math::STAGE_BYTES, NW = Math::NW, THREADS = NW * 32, SROWS = Math::SROWS;
+    constexpr int PARTS = FDC_TILE_ROWS / SROWS;           // stages of a tile
+    constexpr int CHUNK = 16 / sizeof(typename Math::Elem);         // elements of a 16-byte chunk
+    extern __shared__ unsigned char smem_dyn[];
+    unsigned char* ring = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
+    unsigned char* qs = ring + (size_t)nstage * STAGE_BYTES;
+    float* part = reinterpret_cast<float*>(ring);          // after the last stage: [warp][GROWS][D] partials
+    __shared__ BlockState<NW, GROWS> bs;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x % nblk;                    // = rank in the cluster (the grid is cut into runs of nblk blocks)
+    const int cluster = blockIdx.x / nblk;
+    const int pair = cluster / qsplit, m0 = (cluster - pair * qsplit) * qrows;      // this cluster: query rows m0 .. m0 + qrows - 1 of the pair
+    const int s = pair / p.hkv, g = pair - s * p.hkv;
+    // Programmatic dependent launch: as in the tcgen05 kernel (fdc_attn_tc_kernel.cuh).  With p.early the pass
+    // tables and the prefix rows may be read ahead of the wait; every thread passes the wait.
+    if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int A = p.n_active[s], nt = p.ntiles[s];
+    if (A * p.group <= m0 || nt <= 0) {                    // nothing to do (all blocks of the cluster agree)
+        if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+        return;
+    }
+    const int M = A * p.group - m0 < qrows ? A * p.group - m0 : qrows;
+    const int groups = Math::GROUPS == 1 || M <= GROWS ? 1 : (Math::GROUPS == 2 || M <= 2 * GROWS ? 2 : (M <= 4 * GROWS ? 4 : 8)), lanes = NW / groups;
+    Run r;
+    r.tiles = p.tiles + (size_t)s * p.ntile_max;
+    r.mask = p.mask + (size_t)s * p.max_active * p.W;
+    r.h0 = (int)((long long)rank * PARTS * nt / nblk);
+    r.h1 = (int)((long long)(rank + 1) * PARTS * nt / nblk);
+    r.p0 = PARTS * (p.P / FDC_TILE_ROWS);                      // the whole tiles of the prefix come first in a list
+    if (r.p0 < r.h0) r.p0 = r.h0;
+    if (r.p0 > r.h1) r.p0 = r.h1;
+    r.np = r.h1 - r.p0;
+    if (r.np > MASK_WORDS / A) r.np = MASK_WORDS / A;
+    if (r.np > MASK_HALVES) r.np = MASK_HALVES;
+    // ---- set-up: barriers, the run's rows, the fields' visibility beyond the prefix
+    r.nx = p.app_row && rank == 0 ? (A + SROWS - 1) / SROWS : 0;
+    if (tid == 0) {
+        bs.abort_flag = 0;
+        bs.first_beyond = r.h1 - r.h0;
+        for (int i = 0; i < nstage; ++i) {
+            bs.used[i] = 0;
+            bs.asked[i] = i < r.nx ? 1 : 0;
+            mbar_init(smem_u32(&bs.full[i]), 1);
+            if (Math::K_REUSED) mbar_init(smem_u32(&bs.k_read[i]), groups);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_smem();
+        for (int i = 0; i < r.nx; ++i) mbar_arrive(smem_u32(&bs.full[i]));      // filled by this block itself, ahead of the main loop
+    }
+    if (tid < MASK_HALVES) bs.seen[tid] = 0u;
+    bool off_list = false;
+    int beyond = 0x7fffffff;                               // first part of this thread's that reaches beyond the prefix
+    for (int i = tid; i < r.h1 - r.h0; i += THREADS) {
+        const int pos = r.h0 + i, row0 = r.tiles[pos / (FDC_TILE_ROWS / SROWS)] * FDC_TILE_ROWS + pos % (FDC_TILE_ROWS / SROWS) * SROWS;
+        if (i < ROW0S) bs.row0[i] = row0;
+        if (row0 + SROWS > p.P && beyond == 0x7fffffff) beyond = i;
+        off_list |= pos < PARTS * (p.P / FDC_TILE_ROWS) && row0 != pos * SROWS;
+    }
+    __syncthreads();
+    if (beyond != 0x7fffffff) atomicMin(&bs.first_beyond, beyond);
+    auto cache_bits = [&]() {
+        for (int i = tid; i < r.np * A; i += THREADS) {
+            const int h = i / A, b = i - h * A;
+            const uint32_t x = part_bits<SROWS>(r.mask + (size_t)b * p.W, p.W, p.P, part_row0<SROWS>(r, bs, r.p0 + h));
+            bs.bits[i] = x;
+            if (x) atomicOr(&bs.seen[h], x);
+        }
+    };
+    // Fused append, from the new rows' places (bs.app_row): which of them every field sees, and their rows
+    // taken out of the tables of the cache's tile parts.
+    auto new_bits = [&]() {
+        for (int i = tid; i < r.np * A; i += THREADS) {
+            const int h = i / A, b = i - h * A, x = bs.app_row[b] - part_row0<SROWS>(r, bs, r.p0 + h);
+            if (x >= 0 && x < SROWS) {
+                atomicAnd(&bs.seen[h], ~(1u << x));
+                for (int b2 = 0; b2 < A; ++b2) atomicAnd(&bs.bits[h * A + b2], ~(1u << x));
+            }
+        }
+        for (int i = warp; i < r.nx * A; i += NW) {
+            const int x = i / A, b = i - x * A, j = x * SROWS + lane;
+            const int ar = j < A ? bs.app_row[j] : -1, t = ar - p.P;
+            const bool on = ar >= 0 && (t >> 6) < p.W && ((r.mask[(size_t)b * p.W + (t >> 6)] >> (t & 63)) & 1ull);
+            const uint32_t bits = __ballot_sync(0xffffffffu, on);
+            if (lane == 0) bs.newbits[x * FDC_MAX_NODES + b] = bits;
+        }
+    };
+    // (the launch may be ahead of whatever writes the row numbers: what is read here is checked after the wait)
+    int ar0 = p.app_row && tid < A ? p.app_row[(size_t)s * p.max_active + tid] : -1;
+    if (tid < A) bs.app_row[tid] = ar0 >= p.P && ar0 < p.rows ? ar0 : -1;
+    cache_bits();
+    __syncthreads();
+    if (warp == 0) {
+        // the parts that hold a visible row, in order
+        int n = 0;
+        for (int h0 = 0; h0 < r.np; h0 += 32) {
+            const bool keep = h0 + lane < r.np && bs.seen[h0 + lane] != 0u;
+            const uint32_t ball = __ballot_sync(0xffffffffu, keep);
+            if (keep) bs.kept[n + __popc(ball & ((1u << lane) - 1u))] = (uint8_t)(h0 + lane);
+            n += __popc(ball);
+        }
+        if (lane == 0) bs.n_kept = n;
+    }
+    __syncthreads();
+    if (p.app_row) new_bits();                             // (read after the block's next barrier)
+    r.total = r.nx + (r.h1 - r.h0) - (r.np - bs.n_kept);
+    // stages fb.. may hold rows beyond the prefix (parts ahead of p0 are never left out)
+    const int fb = r.nx + (bs.first_beyond < r.p0 - r.h0 ? bs.first_beyond : r.p0 - r.h0);
+    volatile int* abortp = &bs.abort_flag;
+    const uint32_t full0 = smem_u32(bs.full), ring0 = smem_u32(ring);
+    auto request = [&](int it, int st, int n) {            // one thread: the copies of stage `it`, the n-th to use slot st
+        const uint32_t bar = full0 + 8 * st, dst = ring0 + (uint32_t)st * STAGE_BYTES;
+        const int row0 = part_row0<SROWS>(r, bs, stage_pos(r, bs, it));
+        mbar_expect_tx(bar, STAGE_BYTES);
+#pragma unroll
+        for (int h = 0; h < STAGE_BYTES / (2 * SROWS * 128); ++h) {
+            tma_load_4d(dst + h * (SROWS * 128), &tm_k, bar, h * 8 * CHUNK, row0, g, s);
+            tma_load_4d(dst + STAGE_BYTES / 2 + h * (SROWS * 128), &tm_v, bar, h * 8 * CHUNK, row0, g, s);
+        }
+        __threadfence_block();
+        *(volatile int*)&bs.asked[st] = n;
+    };
+    // the first stages: warp w requests w and w + 8; those of the prefix ahead of the dependency wait
+    if (lane == 0) {
+        for (int it = warp; it < nstage && it < fb; it += NW)
+            if (it >= r.nx) request(it, it, 1);
+    }
+    __syncwarp();
+    if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (lane == 0) {
+        for (int it = warp; it < nstage && it < r.total; it += NW)
+            if (it >= fb) request(it, it, 1);
+    }
+    __syncwarp();
+    // queries of the pair: row m = field * group + head-in-group; rows M.. up to a whole group are zero
+    for (int i = tid; i < (M + GROWS - 1) / GROWS * GROWS * (D / CHUNK); i += THREADS) {
+        const int m = i / (D / CHUNK), dc = i - m * (D / CHUNK);
+        const int b = m < M ? (m0 + m) / p.group : 0, hg = m < M ? m0 + m - b * p.group : 0;
+        cp_async16(qs + Math::q_off(qrows, m, dc),
+                   reinterpret_cast<const uint4*>(p.q) + ((((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * D) / CHUNK + dc, m < M);
+    }
+    // the stages of new rows: row i of stage x = the new vectors of field 32 x + i (rows past the last field: zero)
+    for (int i = tid; i < r.nx * SROWS * (D / CHUNK); i += THREADS) {
+        const int b = i / (D / CHUNK), dc = i - b * (D / CHUNK);
+        const size_t src = ((size_t)s * p.max_active * p.hkv + g + (size_t)(b < A ? b : 0) * p.hkv) * (D / CHUNK) + dc;
+        unsigned char* ks = ring + (size_t)(b / SROWS) * STAGE_BYTES + swz(SROWS * 128, b % SROWS, dc);
+        cp_async16(ks, reinterpret_cast<const uint4*>(p.app_k) + src, b < A);
+        cp_async16(ks + STAGE_BYTES / 2, reinterpret_cast<const uint4*>(p.app_v) + src, b < A);
+    }
+    // (kernels for other caches have never asked for the prefix tiles to come first)
+    if (Math::PREFIX_FIRST && off_list) atomicOr(p.status, FDC_DEV_TILE_LIST);
+    int moved = 0;
+    if (p.app_row && tid < A) {
+        const int ar = __ldcg(p.app_row + (size_t)s * p.max_active + tid);
+        if ((ar < p.P || ar >= p.rows) && cluster == s * p.hkv * qsplit && rank == 0) atomicOr(p.status, FDC_DEV_ROW_RANGE);     // skipped and flagged
+        moved = ar != ar0;
+        ar0 = ar;
+    }
+    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+    fence_async_smem();                                    // (the next copy into the new rows' slots goes through the asynchronous proxy)
+    if (__syncthreads_or(moved)) {
+        // the row numbers were written by the kernel ahead: the tables once more
+        if (tid < A) bs.app_row[tid] = ar0 >= p.P && ar0 < p.rows ? ar0 : -1;
+        if (tid < MASK_HALVES) bs.seen[tid] = 0u;
+        __syncthreads();
+        cache_bits();
+        __syncthreads();
+        new_bits();
+        __syncthreads();
+    }
+    const int mg = warp % groups, kl = warp / groups;
+    const int left = M - mg * GROWS;                       // rows of this warp's group that exist (<= 0: none)
+    Math math(p, qs, qrows, left > 0 ? mg * GROWS : 0, lane);
+    int fld[Math::ROWS];                                   // fields of the thread's query rows
+#pragma unroll
+    for (int i = 0; i < Math::ROWS; ++i) fld[i] = math.row(i) < left ? (m0 + mg * GROWS + math.row(i)) / p.group : -1;
+    bool alive = true;
+    int st = kl, use = 1;                                  // slot of stage `it`, and how many stages (this one included) have used it
+    while (st >= nstage) {
+        st -= nstage;
+        ++use;
+    }
+    for (int it = kl; it < r.total; it += lanes) {
+        alive = wait_asked(&bs.asked[st], use, abortp, p.status) && mbar_wait(full0 + 8 * st, (uint32_t)(use - 1) & 1, abortp, p.status);
+        if (!__all_sync(0xffffffffu, alive)) break;
+        if (left > 0) {
+            bool masked = false;
+            uint32_t mk[Math::ROWS], seen = ~0u, any = ~0u;
+#pragma unroll
+            for (int i = 0; i < Math::ROWS; ++i) mk[i] = ~0u;
+            if (it < r.nx) {
+                masked = true;
+#pragma unroll
+                for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[i] < 0 ? 0u : bs.newbits[it * FDC_MAX_NODES + fld[i]];
+                for (int b = 0; b < SROWS && it * SROWS + b < A; ++b)     // (values of rows that are not written do not count either)
+                    if (bs.app_row[it * SROWS + b] < 0) seen &= ~(1u << b);
+            } else if (it >= fb) {
+                const int pos = stage_pos(r, bs, it), row0 = part_row0<SROWS>(r, bs, pos), h = pos - r.p0;
+                if (row0 + SROWS > p.P) {
+                    masked = true;
+                    if (h >= 0 && h < r.np) {
+#pragma unroll
+                        for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[i] < 0 ? 0u : bs.bits[h * A + fld[i]];
+                        seen = bs.seen[h];
+                    } else {
+                        const uint32_t fresh = p.app_row ? new_rows_of<SROWS>(bs.app_row, A, row0) : 0u;
+#pragma unroll
+                        for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[i] < 0 ? 0u : part_bits<SROWS>(r.mask + (size_t)fld[i] * p.W, p.W, p.P, row0) & ~fresh;
+                        seen = part_seen_slow<SROWS>(r.mask, p.W, p.P, A, row0) & ~fresh;
+                    }
+                }
+            }
+            if (masked) {
+                any = 0u;
+#pragma unroll
+                for (int i = 0; i < Math::ROWS; ++i) any |= mk[i];
+            }
+            auto k_read = [&]() {
+                if constexpr (Math::K_REUSED) {
+                    __syncwarp();
+                    if (groups == 1) return;
+                    if (lane == 0) mbar_arrive(smem_u32(&bs.k_read[st]));
+                    alive = mbar_wait(smem_u32(&bs.k_read[st]), (uint32_t)(use - 1) & 1, abortp, p.status);
+                }
+            };
+            if (__any_sync(0xffffffffu, any != 0u)) math.stage(ring0 + (uint32_t)st * STAGE_BYTES, masked, mk, seen, k_read);
+            else k_read();                                 // (a part that only other groups' fields see)
+            if (Math::K_REUSED && !__all_sync(0xffffffffu, alive)) break;
+        } else if (Math::K_REUSED && groups > 1 && lane == 0) {
+            mbar_arrive(smem_u32(&bs.k_read[st]));
+        }
+        // the last group to finish with the stage requests its next rows
+        __syncwarp();
+        if (lane == 0 && it + nstage < r.total) {
+            bool mine = groups == 1;
+            if (!mine) {
+                __threadfence_block();
+                mine = atomicAdd(&bs.used[st], 1) == groups - 1;
+                __threadfence_block();
+                if (mine) bs.used[st] = 0;
+            }
+            if (mine) request(it + nstage, st, use + 1);
+        }
+        st += lanes;
+        while (st >= nstage) {
+            st -= nstage;
+            ++use;
+        }
+    }
+    // a wait that ran out: give the copies already in flight a bounded chance to land before the ring is reused
+    if (*abortp) {
+        for (int i = 0; i < 100; ++i) __nanosleep(1000);
+    }
+    // ---- the warps' results meet in shared memory (the ring is free: every stage has been consumed)
+    __syncthreads();
+    if (left > 0) math.write(part + warp * (GROWS * D), bs.wml + warp * GROWS);
+    __syncthreads();
+    auto store_out = [&](int mm, int c4, const float4& acc, float lt) {
+        const float inv = 1.f / lt;
+        const int b = (m0 + mm) / p.group, hg = m0 + mm - b * p.group;
+        Math::store(reinterpret_cast<typename Math::Elem*>(p.out) + (((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * D + c4,
+                    make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
+    };
+    // block: merge over the warps of a group; with one block per pair that is the result
+    merge_lanes<Math>(lanes, tid, M, groups * GROWS, bs.wml, part, [&](int mm, int c4, float mx, float lt, const float4& acc) {
+        if (nblk == 1) {
+            store_out(mm, c4, acc, lt);
+        } else {
+            *reinterpret_cast<float4*>(part + Math::part_off(mm, c4)) = acc;          // in place of the first lane's partial (one thread reads and writes it)
+            if (c4 == 0) bs.cml[mm] = make_float2(mx, lt);
+        }
+    });
+    if (nblk > 1) {
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    }
+    // fused append: the new rows whose tile parts are in this block's run go to the cache (this block's copies
+    // from there have landed; clusters with the pair's other query rows may still be reading the
+    // part, but to them, too, the row counts as unseen: its bytes there do not matter)
+    if (Math::FUSES && p.app_row && m0 == 0 && bs.first_beyond < r.h1 - r.h0)
+        for (int b = warp; b < A; b += NW) {
+            const int ar = bs.app_row[b];
+            bool here = false;
+            for (int i = bs.first_beyond + lane; i < r.h1 - r.h0; i += 32) {
+                const int x = ar - part_row0<SROWS>(r, bs, r.h0 + i);
+                here |= x >= 0 && x < SROWS;
+            }
+            here = __any_sync(0xffffffffu, here && ar >= 0);
+            const int dc = lane & 15;
+            if (here && dc < D / CHUNK) {
+                // lanes 0-15: the K row, lanes 16-31: the V row
+                const uint4 x = reinterpret_cast<const uint4*>(lane < 16 ? p.app_k : p.app_v)[((((size_t)s * p.max_active + b) * p.hkv + g) * D) / CHUNK + dc];
+                auto* cache = const_cast<typename Math::Elem*>(reinterpret_cast<const typename Math::Elem*>(lane < 16 ? p.k : p.v));
+                *reinterpret_cast<uint4*>(cache + (size_t)s * p.stride_scene + (size_t)g * p.stride_head + (size_t)ar * p.stride_row + dc * CHUNK) = x;
+            }
+        }
+    if (nblk == 1) return;
+    // ---- cluster: every block merges its share of the (query row, 4 columns) items over all blocks
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    {
+        // Four threads per item, each with every fourth block (at most four: one trip), summed by shuffles.
+        const uint32_t ml0 = smem_u32(bs.cml), part0 = smem_u32(part);
+        const int q = tid & 3, items = M * (D / 4);
+        for (int i0 = (tid >> 2) * nblk + rank; __any_sync(0xffffffffu, i0 < items); i0 += (THREADS / 4) * nblk) {
+            const bool on = i0 < items;
+            const int mm = on ? i0 / (D / 4) : 0, c4 = on ? (i0 - mm * (D / 4)) * 4 : 0;
+            const uint32_t a_ml = ml0 + mm * 8, a_o = part0 + 4 * Math::part_off(mm, c4);
+            float2 v[4];
+            float4 x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[j] = make_float2(-INFINITY, 0.f);
+                x[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (on && q + 4 * j < nblk) {
+                    v[j] = ld_cluster2(map_rank(a_ml, q + 4 * j));
+                    x[j] = ld_cluster4(map_rank(a_o, q + 4 * j));
+                }
+            }
+            float mx = fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            const float ms = mx == -INFINITY ? 0.f : mx;
+            float lt = 0.f;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float w = fast_exp2(v[j].x - ms);    // a block that saw nothing: 0
+                lt = fmaf(v[j].y, w, lt);
+                acc.x = fmaf(x[j].x, w, acc.x);
+                acc.y = fmaf(x[j].y, w, acc.y);
+                acc.z = fmaf(x[j].z, w, acc.z);
+                acc.w = fmaf(x[j].w, w, acc.w);
+            }
+#pragma unroll
+            for (int d = 1; d < 4; d <<= 1) {
+                lt += __shfl_xor_sync(0xffffffffu, lt, d);
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, d);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, d);
+                acc.z += __shfl_xor_sync(0xffffffffu, acc.z, d);
+                acc.w += __shfl_xor_sync(0xffffffffu, acc.w, d);
+            }
+            if (on && q == 0) store_out(mm, c4, acc, lt);
+        }
+    }
+    __syncwarp();
+    // nobody leaves while its shared memory is still being read
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Host: shared memory of a launch, tensor maps, launch attributes.  `room`: bytes a block may use.
+template <class Math, class Kernel>
+int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const ClusterShape& h, cudaStream_t st)
+{
+    const int qrows = ((p.mmax + Math::GROWS - 1) / Math::GROWS + h.qsplit - 1) / h.qsplit * Math::GROWS;
+    const size_t fixed = 1024 + Math::q_bytes(qrows);
+    int nstage = (int)((room - sizeof(BlockState<Math::NW, Math::GROWS>) - 256 - fixed) / Math::STAGE_BYTES);
+    if (nstage > MAX_STAGES) nstage = MAX_STAGES;
+    if ((size_t)nstage * Math::STAGE_BYTES < (size_t)Math::NW * Math::GROWS * Math::D * 4) return FDC_ERR_SHAPE;      // the partials take the ring's place
+    size_t smem = fixed + (size_t)nstage * Math::STAGE_BYTES;
+    if (h.per_sm <= 1 && smem < 120 * 1024) smem = 120 * 1024;        // (more than half of an SM's: no second block beside this one)
+    static size_t attr_smem[kMaxDevices] = {};
+    int rc = raise_dynamic_smem(reinterpret_cast<const void*>(kernel), smem, attr_smem);
+    if (rc) return rc;
+    if (h.nblk > 8) {
+        static std::atomic<uint64_t> wide_ok{0};           // devices on which clusters of 16 have been asked for
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return FDC_ERR_CUDA;
+        if (dev > 63 || !((wide_ok.load() >> dev) & 1)) {
+            cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e != cudaSuccess) return set_cuda_error(e);
+            if (dev <= 63) wide_ok.fetch_or(1ull << dev);
+        }
+    }
+    alignas(64) CUtensorMap tk, tv;
+    const int dtype = sizeof(typename Math::Elem) == 4 ? FDC_F32 : FDC_BF16;
+    rc = get_kv_tensor_map(p.k, p, dtype, Math::D, Math::SROWS, &tk);
+    if (rc) return rc;
+    rc = get_kv_tensor_map(p.v, p, dtype, Math::D, Math::SROWS, &tv);
+    if (rc) return rc;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((long long)p.batch * p.hkv * h.qsplit * h.nblk));
+    cfg.blockDim = dim3(Math::NW * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)h.nblk;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, tk, tv, nstage, h.nblk, h.qsplit, qrows);
+    if (e != cudaSuccess) return set_cuda_error(e);
+    note_launch();
+    return FDC_OK;
+}
+
+}  // namespace fdc

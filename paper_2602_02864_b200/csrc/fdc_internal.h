@@ -146,6 +146,7 @@ void note_launch();
 int  set_cuda_error(cudaError_t e);                  // records the message, returns FDC_ERR_CUDA
 
 int launch_attn_ref(const AttnParams& p, int dtype, int head_dim, cudaStream_t st);
+int launch_attn_f32(const AttnParams& p, int head_dim, cudaStream_t st);
 int launch_attn_cluster(const AttnParams& p, int head_dim, cudaStream_t st);
 int launch_attn_tc(const AttnParams& p, int head_dim, cudaStream_t st);
 int launch_attn_tc_split(const AttnParams& p, int head_dim, cudaStream_t st);   // computes the work split only (into p.split_memo)

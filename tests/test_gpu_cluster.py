@@ -1,5 +1,5 @@
-"""The cluster kernel (fdc_set_attn_kernel 2; the automatic choice for head_dim 64 and for small passes)
-against the CPU checker at the sizes where its splits, rings and groups can go wrong."""
+"""The cluster kernels (bf16: fdc_set_attn_kernel 2, the automatic choice for head_dim 64 and for small passes;
+fp32: the automatic choice) against the CPU checker at the sizes where its splits, rings and groups can go wrong."""
 import pytest
 
 from harness import run_and_compare
@@ -22,4 +22,17 @@ def test_cluster_kernel_shapes(head_dim, hq, hkv, fields, batch, prefix):
     w.max_active = w.n_nodes
     steps = {0, 1, 9, 33}
     r = run_and_compare(w, check_steps=steps, kernel=2, max_steps=34)
+    assert r["checked"] > 0
+
+
+# fp32: query rows per pair around what a lane's tile holds (8 / 16 / 24 / 32 rows) and wider pairs, which are cut
+# over several clusters; one block per pair (many pairs) up to eight
+@pytest.mark.parametrize("head_dim,hq,hkv,fields,batch,prefix", [
+    (64, 4, 2, 1, 1, 33), (64, 14, 2, 2, 3, 200), (64, 4, 2, 9, 30, 1000), (64, 16, 8, 16, 2, 700), (64, 2, 2, 33, 1, 0),
+    (128, 32, 8, 2, 1, 2048), (128, 28, 4, 3, 2, 1531), (128, 32, 8, 6, 12, 600), (128, 32, 8, 9, 2, 129), (128, 8, 2, 32, 3, 500)])
+def test_fp32_cluster_kernel_shapes(head_dim, hq, hkv, fields, batch, prefix):
+    w = wl.random_template(8100 + fields + batch, n_nodes=fields, edge_prob=0.15, cap_lo=2, cap_hi=70, batch=batch, prefix_len=prefix, fixed_hi=2,
+                           hq=hq, hkv=hkv, head_dim=head_dim, dtype="f32")
+    w.max_active = w.n_nodes
+    r = run_and_compare(w, check_steps={0, 1, 9, 33}, max_steps=34)
     assert r["checked"] > 0
