@@ -47,14 +47,14 @@ void prof_destroy(fdc_plan* p)
     p->prof = nullptr;
 }
 
-// Estimated time (us) of a launch of the tcgen05 kernel: fitted, like the cluster kernel's, to the 168 shapes
-// with head_dim 128 of the same measurement.  A launch costs a chain of latencies plus the rounds of 128 KV rows of
-// its busiest block, both growing with the width of the build (32, 64 or 128 query rows), and every further
-// pair that a block has to finish costs about as much as a launch.
+// Estimated time (us) of a launch of the tcgen05 kernels: fitted, like the cluster kernel's, to the 168 shapes
+// with head_dim 128 of the same measurement (more than 64 query rows: to six shapes of the row form).  A launch costs
+// a chain of latencies plus the rounds of 128 KV rows of its busiest block, by kernel (up to 32, 64 and 128 query rows),
+// and every further pair that a block has to finish costs about as much as a launch.
 static float tc_estimate(const ClusterProblem& c)
 {
     const int k = c.mmax <= 32 ? 0 : (c.mmax <= 64 ? 1 : 2);
-    static const float fixed[] = {11.9f, 17.7f, 20.3f}, round[] = {1.63f, 2.0f, 4.9f};
+    static const float fixed[] = {11.9f, 17.7f, 29.f}, round[] = {1.63f, 2.0f, 1.6f};
     const float rows = (float)c.P + 0.5f * (float)c.T, rounds = rows / 128.f, pairs = (float)c.pairs, sms = (float)c.sm_count;
     const float busiest = fmaxf(fminf(4.f, rounds), pairs * rounds / sms);
     const float t_mem = 8.f + pairs * rows * 512e-6f / 6.2f;

@@ -4,5 +4,4 @@
 #define FDC_TC_NPMAX 64
 #define FDC_TC_KERNEL attn_tc_kernel_g2
 #define FDC_TC_LAUNCH launch_tc_np64
-#define FDC_TC_TRACE_READ fdc_tr_read_g2
 #include "fdc_attn_tc_kernel.cuh"
