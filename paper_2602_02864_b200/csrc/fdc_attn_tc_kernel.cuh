@@ -173,7 +173,10 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, bool vali
 // One elected thread: S^T[g mod ns] = K(stage) Q^T for every round g.  A score buffer is free again
 // once the softmax threads have read round g - ns (s_free); with four buffers K Q^T runs well ahead of
 // the softmax, so a K stage is released soon after it landed and the K ring stays in flight.
-__device__ __forceinline__ void qk_loop(const AttnParams& p, const Ctx& cx, long long lo, long long hi, int lane)
+// The whole warp goes round this loop (and those of the other two issuing warps) and one elected thread issues: a
+// round's issue is on the path from its K rows to its weights, and with the loops inside "lane 0" it took longer (us a
+// layer, lane 0 / elected: 8 scenes x 4 heads, 64 rows, prefix 8192: 61.5 / 59.1; 16 scenes, 24 rows, prefix 4096: 53.3 / 52.2).
+__device__ __forceinline__ void qk_loop(const AttnParams& p, const Ctx& cx, long long lo, long long hi)
 {
     const uint64_t q_desc = smem_desc(smem_u32(cx.qs), 16, 1024);
     const uint64_t k_desc0 = smem_desc(smem_u32(cx.kring), 16, 1024);
@@ -184,21 +187,22 @@ __device__ __forceinline__ void qk_loop(const AttnParams& p, const Ctx& cx, long
     int st = 0;
     uint32_t kph = 0;                               // ring position and phase of the K stage of round g
     long long u = lo;
-    int ok = 1;
+    bool ok = true;
     while (u < hi && ok) {
         const Segment sg = decode_segment(u, hi, cx.pre, p.hkv, s);
         const int nr = (sg.j1 - sg.j0 + 1) >> 1;
-        if (lane == 0) {
-            const int M = cx.nact[sg.s] * p.group;
-            const int NP = (NP_MAX == 32 || M <= 32) ? 32 : 64;
-            const uint32_t idesc_qk = instr_desc(RROWS, NP, 0);
-            bool good = mbar_wait(cx.q_ready(), seg & 1, cx.abortp, p.status);
-            for (int t = 0; t < nr && good; ++t, ++g) {
-                good = mbar_wait(cx.k_full() + 8 * st, kph, cx.abortp, p.status);
-                const uint32_t sb = g & (cx.ns - 1);                  // score buffer of the round
-                if (good && g >= (uint32_t)cx.ns) good = mbar_wait(cx.s_free() + 8 * sb, ((g / cx.ns) - 1) & 1, cx.abortp, p.status);
-                if (!good) break;
-                tc_fence_after();
+        const int M = cx.nact[sg.s] * p.group;
+        const int NP = (NP_MAX == 32 || M <= 32) ? 32 : 64;
+        const uint32_t idesc_qk = instr_desc(RROWS, NP, 0);
+        bool good = ok && mbar_wait(cx.q_ready(), seg & 1, cx.abortp, p.status);
+        for (int t = 0; t < nr && good; ++t, ++g) {
+            good = mbar_wait(cx.k_full() + 8 * st, kph, cx.abortp, p.status);
+            const uint32_t sb = g & (cx.ns - 1);                  // score buffer of the round
+            if (good && g >= (uint32_t)cx.ns) good = mbar_wait(cx.s_free() + 8 * sb, ((g / cx.ns) - 1) & 1, cx.abortp, p.status);
+            good = __all_sync(0xffffffffu, good);
+            if (!good) break;
+            tc_fence_after();
+            if (elect_one()) {
                 const uint32_t kd = k_lo0 + (uint32_t)((st * STAGE) >> 4);
                 const uint32_t d = cx.tmem + sb * cx.s_stride;
 #pragma unroll
@@ -207,17 +211,14 @@ __device__ __forceinline__ void qk_loop(const AttnParams& p, const Ctx& cx, long
                           idesc_qk, ks > 0);
                 umma_commit(cx.k_empty() + 8 * st);
                 umma_commit(cx.s_full() + 8 * sb);
-                if (++st == cx.nk) {
-                    st = 0;
-                    kph ^= 1;
-                }
             }
-            ok = good;
+            __syncwarp();
+            if (++st == cx.nk) {
+                st = 0;
+                kph ^= 1;
+            }
         }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        g = __shfl_sync(0xffffffffu, g, 0);
-        st = __shfl_sync(0xffffffffu, st, 0);
-        kph = __shfl_sync(0xffffffffu, kph, 0);
+        ok = good;
         ++seg;
         u = sg.next_u;
     }
@@ -250,19 +251,20 @@ __device__ __forceinline__ void aux_loop(const AttnParams& p, const Ctx& cx, lon
     int s = 0;
     uint32_t g = 0, seg = 0;
     long long u = lo;
-    int ok = 1;
+    bool ok = true;
     while (u < hi && ok) {
         const Segment sg = decode_segment(u, hi, cx.pre, p.hkv, s);
-        if (lane == 0) {
-            const uint32_t idesc_sum = instr_desc(128, 16, 1);
-            const int ntile = sg.j1 - sg.j0;
-            bool good = true;
-            for (int t = 0; 2 * t < ntile && good; ++t, ++g) {
-                good = mbar_wait(cx.p_full() + 8 * (g & 1), (g >> 1) & 1, cx.abortp, p.status);
-                if (good && t == 0 && seg > 0) good = mbar_wait(cx.o_free(), (seg - 1) & 1, cx.abortp, p.status);
-                if (!good) break;
-                const uint32_t steps = (uint32_t)cx.v_steps[(g & 1) * 2] | ((uint32_t)cx.v_steps[(g & 1) * 2 + 1] << 4);
-                tc_fence_after();
+        const uint32_t idesc_sum = instr_desc(128, 16, 1);
+        const int ntile = sg.j1 - sg.j0;
+        bool good = ok;
+        for (int t = 0; 2 * t < ntile && good; ++t, ++g) {
+            good = mbar_wait(cx.p_full() + 8 * (g & 1), (g >> 1) & 1, cx.abortp, p.status);
+            if (good && t == 0 && seg > 0) good = mbar_wait(cx.o_free(), (seg - 1) & 1, cx.abortp, p.status);
+            good = __all_sync(0xffffffffu, good);
+            if (!good) break;
+            const uint32_t steps = (uint32_t)cx.v_steps[(g & 1) * 2] | ((uint32_t)cx.v_steps[(g & 1) * 2 + 1] << 4);
+            tc_fence_after();
+            if (elect_one()) {
                 const uint32_t pd = p_lo0 + (uint32_t)((((g & 1) & (cx.npb - 1)) * cx.p_buf) >> 4);
                 uint32_t acc = t > 0 ? 1u : 0u;
 #pragma unroll 1
@@ -273,10 +275,9 @@ __device__ __forceinline__ void aux_loop(const AttnParams& p, const Ctx& cx, lon
                     }
                 umma_commit(cx.pv_done() + 8 * (g & 1));
             }
-            ok = good;
+            __syncwarp();
         }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        g = __shfl_sync(0xffffffffu, g, 0);
+        ok = good;
         ++seg;
         u = sg.next_u;
     }
@@ -286,7 +287,7 @@ __device__ __forceinline__ void aux_loop(const AttnParams& p, const Ctx& cx, lon
 // the softmax warps have delivered P^T (and, beyond the prefix, cleared the stage's unseen rows).
 // The multiplication runs in steps of 16 KV rows; the softmax warps say which steps hold a visible
 // row (all of them inside the prefix), the others are left out.
-__device__ __forceinline__ void pv_loop(const AttnParams& p, const Ctx& cx, long long lo, long long hi, int lane)
+__device__ __forceinline__ void pv_loop(const AttnParams& p, const Ctx& cx, long long lo, long long hi)
 {
     const uint64_t v_desc0 = smem_desc(smem_u32(cx.vring), PANEL, 1024);
     const uint64_t p_desc0 = smem_desc(smem_u32(cx.ps), PANEL, 1024);
@@ -297,22 +298,23 @@ __device__ __forceinline__ void pv_loop(const AttnParams& p, const Ctx& cx, long
     int st = 0;
     uint32_t vph = 0;
     long long u = lo;
-    int ok = 1;
+    bool ok = true;
     while (u < hi && ok) {
         const Segment sg = decode_segment(u, hi, cx.pre, p.hkv, s);
-        if (lane == 0) {
-            const int M = cx.nact[sg.s] * p.group;
-            const int NP = (NP_MAX == 32 || M <= 32) ? 32 : 64;
-            const uint32_t idesc_pv = instr_desc(D, NP, 1);
-            const int ntile = sg.j1 - sg.j0;
-            bool good = true;
-            for (int t = 0; 2 * t < ntile && good; ++t, ++g) {
-                good = mbar_wait(cx.v_full() + 8 * st, vph, cx.abortp, p.status);
-                if (good) good = mbar_wait(cx.p_full() + 8 * (g & 1), (g >> 1) & 1, cx.abortp, p.status);
-                if (good && t == 0 && seg > 0) good = mbar_wait(cx.o_free(), (seg - 1) & 1, cx.abortp, p.status);
-                if (!good) break;
-                const uint32_t steps = (uint32_t)cx.v_steps[(g & 1) * 2] | ((uint32_t)cx.v_steps[(g & 1) * 2 + 1] << 4);
-                tc_fence_after();
+        const int M = cx.nact[sg.s] * p.group;
+        const int NP = (NP_MAX == 32 || M <= 32) ? 32 : 64;
+        const uint32_t idesc_pv = instr_desc(D, NP, 1);
+        const int ntile = sg.j1 - sg.j0;
+        bool good = ok;
+        for (int t = 0; 2 * t < ntile && good; ++t, ++g) {
+            good = mbar_wait(cx.v_full() + 8 * st, vph, cx.abortp, p.status);
+            if (good) good = mbar_wait(cx.p_full() + 8 * (g & 1), (g >> 1) & 1, cx.abortp, p.status);
+            if (good && t == 0 && seg > 0) good = mbar_wait(cx.o_free(), (seg - 1) & 1, cx.abortp, p.status);
+            good = __all_sync(0xffffffffu, good);
+            if (!good) break;
+            const uint32_t steps = (uint32_t)cx.v_steps[(g & 1) * 2] | ((uint32_t)cx.v_steps[(g & 1) * 2 + 1] << 4);
+            tc_fence_after();
+            if (elect_one()) {
                 const uint32_t vd = v_lo0 + (uint32_t)((st * STAGE) >> 4);
                 const uint32_t pd = p_lo0 + (uint32_t)((((g & 1) & (cx.npb - 1)) * cx.p_buf) >> 4);
                 if (steps == 0xffu) {
@@ -331,17 +333,14 @@ __device__ __forceinline__ void pv_loop(const AttnParams& p, const Ctx& cx, long
                 }
                 umma_commit(cx.v_empty() + 8 * st);
                 umma_commit(cx.pv_done() + 8 * (g & 1));
-                if (++st == cx.nv) {
-                    st = 0;
-                    vph ^= 1;
-                }
             }
-            ok = good;
+            __syncwarp();
+            if (++st == cx.nv) {
+                st = 0;
+                vph ^= 1;
+            }
         }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        g = __shfl_sync(0xffffffffu, g, 0);
-        st = __shfl_sync(0xffffffffu, st, 0);
-        vph = __shfl_sync(0xffffffffu, vph, 0);
+        ok = good;
         ++seg;
         u = sg.next_u;
     }
@@ -1097,9 +1096,9 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
     } else if (warp == W_AUX) {
         aux_loop(p, cx, lo, hi, lane);
     } else if (warp == W_PV) {
-        pv_loop(p, cx, lo, hi, lane);
+        pv_loop(p, cx, lo, hi);
     } else if (warp == W_QK) {
-        qk_loop(p, cx, lo, hi, lane);
+        qk_loop(p, cx, lo, hi);
     } else {
         int s = 0;
         uint32_t g = 0, seg = 0;

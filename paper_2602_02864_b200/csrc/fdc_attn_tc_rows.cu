@@ -55,14 +55,6 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32
         ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// True in one thread of the (converged) warp.  A region entered by this predicate issues the multiplications faster than
-// one behind "lane == 0" (measured: about 60 cycles each against 110).
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t r;
-    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
-    return r != 0;
-}
 // Barrier of the softmax warps (a named barrier).  Every call site is reached by all sixteen warps
 // the same number of times whatever happens: a warp whose bounded wait ran out goes on without
 // waiting but still takes every one of these.
