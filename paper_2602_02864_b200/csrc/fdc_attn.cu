@@ -47,32 +47,34 @@ void prof_destroy(fdc_plan* p)
     p->prof = nullptr;
 }
 
-// Estimated time (us) of a launch of the tcgen05 kernels: fitted, like the cluster kernel's, to the 168 shapes
-// with head_dim 128 of the same measurement (more than 64 query rows: to six shapes of the row form).  A launch costs
-// a chain of latencies plus the rounds of 128 KV rows of its busiest block, by kernel (up to 32, 64 and 128 query rows),
-// and every further pair that a block has to finish costs about as much as a launch.
+// Estimated time (us) of a launch of the tcgen05 kernels, fitted (least absolute deviation of the logarithm) to 150
+// shapes with head_dim 128 drawn over 1 to 64 scenes, prefix 256 to 8800 and 4 to 128 query rows: the middle error is
+// 6 %.  A launch costs a chain of latencies plus the rounds of 128 KV rows of its busiest block, by kernel (up to 32, 64
+// and 128 query rows), and more where a block has further pairs to finish.
 static float tc_estimate(const ClusterProblem& c)
 {
     const int k = c.mmax <= 32 ? 0 : (c.mmax <= 64 ? 1 : 2);
-    static const float fixed[] = {11.9f, 17.7f, 29.f}, round[] = {1.63f, 2.0f, 1.6f};
-    const float rows = (float)c.P + 0.5f * (float)c.T, rounds = rows / 128.f, pairs = (float)c.pairs, sms = (float)c.sm_count;
-    const float busiest = fmaxf(fminf(4.f, rounds), pairs * rounds / sms);
-    const float t_mem = 8.f + pairs * rows * 512e-6f / 6.2f;
-    return fmaxf(fixed[k] + round[k] * busiest + 20.f * fmaxf(0.f, pairs / sms - 1.f), t_mem);
+    static const float fixed[] = {13.1f, 12.9f, 17.5f}, round[] = {1.12f, 1.9f, 1.63f};
+    const float rounds = (float)(c.P + c.T) / 128.f, pairs = (float)c.pairs, sms = (float)c.sm_count;
+    const float busiest = fmaxf(fminf(1.28f, rounds), pairs * rounds / sms);
+    const float t_mem = 8.f + pairs * ((float)c.P + 0.5f * (float)c.T) * 512e-6f / 6.2f;
+    return fmaxf(fixed[k] + round[k] * busiest + 11.2f * fmaxf(0.f, pairs / sms - 1.f), t_mem);
 }
 
 // The cluster kernel's cut of this problem and whether it is the faster kernel (kept in the plan: both follow
-// from the shapes alone).  Where both kernels can run, the cluster kernel is taken if its estimate is below 0.85
-// of the other's: with that factor 87 of the 168 shapes go to it, at 0.82 of the tcgen05 kernel's time over all
-// of them (1 scene x 7 query rows 14.5 -> 7.0 us a layer, 1 scene x 42 rows 19.3 -> 10.4, 16 scenes x 24 rows
-// at prefix 4096 stay at 53), and two of them are slower, by 4 and 6 %.
+// from the shapes alone).  Where both kernels can run, the cluster kernel is taken if its estimate is below 0.82
+// of the other's.  How long either takes also depends on how many of the dependencies are met, which the shapes do not
+// tell, so the line lies on the side of the tcgen05 kernel: 59 of the 150 shapes go to the cluster kernel, and three of
+// them are slower there (by 2, 5 and 16 %; with 0.9 it would be 77 and ten, up to 20 %; of 110 others, 53 and four).  Cluster / tcgen05 kernel, us a
+// layer: 1 scene x 7 query rows, prefix 2048 8.0 / 14.5, 1 scene x 42 rows 11.9 / 17.7; 13 scenes x 49 rows, prefix 529
+// 21.6 / 18.3; 16 scenes x 24 rows, prefix 4096 59 / 52.
 static const ClusterShape& route(fdc_plan* p, const fdc_kv_desc* kv)
 {
     const ClusterProblem c{(int64_t)kv->batch * kv->hkv, p->h.max_active * (kv->hq / kv->hkv), kv->head_dim, p->h.P, p->h.T, p->sm_count};
     if (!(p->route_for == c)) {
         float us = 0.f;
         p->route_shape = pick_cluster(c, &us);
-        p->route_cluster = kv->head_dim != 128 || us < 0.85f * tc_estimate(c);
+        p->route_cluster = kv->head_dim != 128 || us < 0.82f * tc_estimate(c);
         p->route_for = c;
     }
     return p->route_shape;
