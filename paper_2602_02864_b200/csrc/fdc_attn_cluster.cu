@@ -266,6 +266,8 @@ int get_map(const void* base, const AttnParams& p, int dtype, int d, int box_row
             *out = it.second;
             return FDC_OK;
         }
+    // A cache expanded over scenes or heads (stride 0, extent > 1) is nothing that a tensor map describes.
+    if ((p.batch > 1 && p.stride_scene == 0) || (p.hkv > 1 && p.stride_head == 0)) return FDC_ERR_SHAPE;
     PFN_cuTensorMapEncodeTiled enc = get_encode();
     if (!enc) return FDC_ERR_CUDA;
     cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)p.rows, (cuuint64_t)p.hkv, (cuuint64_t)p.batch};
