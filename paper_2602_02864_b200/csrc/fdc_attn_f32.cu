@@ -94,10 +94,13 @@ struct MathF32 {
 #pragma unroll
             for (int h = 0; h < D / 32; ++h) lds4(a + (uint32_t)(h * (SROWS * 128)), v[h][0], v[h][1]);
         }
-        __device__ __forceinline__ void fma(uint64_t (&o)[QL][D / 32][2]) const
+        // SOME: only for the query rows that see the KV row, r (a weight of 0 is no help against an infinite or NaN value)
+        template <bool SOME>
+        __device__ __forceinline__ void fma(uint64_t (&o)[QL][D / 32][2], const uint32_t (&mk)[ROWS], int r) const
         {
 #pragma unroll
             for (int i = 0; i < QL; ++i) {
+                if (SOME && !((mk[i] >> r) & 1u)) continue;
                 const uint64_t w2 = pair(w[i], w[i]);
 #pragma unroll
                 for (int h = 0; h < D / 32; ++h) {
@@ -108,7 +111,7 @@ struct MathF32 {
         }
     };
     template <class F>
-    __device__ __forceinline__ void stage(uint32_t kb, bool masked, const uint32_t (&mk)[ROWS], uint32_t seen, F&& k_read)
+    __device__ __forceinline__ void stage(uint32_t kb, bool masked, const uint32_t (&mk)[ROWS], uint32_t, F&& k_read)
     {
         uint64_t s2[QL][JR];                               // (sum over even columns, sum over odd columns)
 #pragma unroll
@@ -184,27 +187,26 @@ struct MathF32 {
             for (int i = 0; i < QP; i += 2)
                 asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(pw + (uint32_t)(j * 8 * PROW + i * 4)), "f"(s[i][j]), "f"(i + 1 < QL ? s[i + 1 < QL ? i + 1 : 0][j] : 0.f) : "memory");
         const uint32_t vb = kb + STAGE_BYTES / 2, pr = kb + p_off + (uint32_t)qg * (QP * 4);
-        if (masked) {
-            // V rows that nobody sees can hold anything (NaN included), and 0 * NaN must not reach the accumulator
-            const int lane = qg * 8 + rg;
-            for (uint32_t z = ~seen & ((1u << SROWS) - 1u); z; z &= z - 1) {
-                const uint32_t r = (uint32_t)(__ffs(z) - 1);
-                if (lane < D / 4)
-                    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(vb + (uint32_t)(lane >> 3) * (SROWS * 128) + r * 128 + (uint32_t)(lane & 7) * 16), "r"(0u)
-                                 : "memory");
-            }
-        }
         __syncwarp();
-        // O += P V, a KV row a step, the next row's operands read while this one's FMAs run
-        {
+        // O += P V, a KV row a step.  Rows that a query row does not see can hold anything, a sibling field's infinities
+        // and NaN among them: a stage that reaches beyond the prefix goes by the query rows' bits.
+        if (masked) {
+            Row x;
+#pragma unroll 1
+            for (int r = 0; r < SROWS; ++r) {
+                x.load(pr, vb, rg, r);
+                x.template fma<true>(o, mk, r);
+            }
+        } else {
+            // the next row's operands are read while this one's FMAs run
             Row x, y;
             x.load(pr, vb, rg, 0);
 #pragma unroll 1
             for (int r = 0; r < SROWS; r += 2) {
                 y.load(pr, vb, rg, r + 1);
-                x.fma(o);
+                x.template fma<false>(o, mk, r);
                 if (r + 2 < SROWS) x.load(pr, vb, rg, r + 2);
-                y.fma(o);
+                y.template fma<false>(o, mk, r + 1);
             }
         }
         __syncwarp();

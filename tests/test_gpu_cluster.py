@@ -1,6 +1,7 @@
 """The cluster kernels (bf16: fdc_set_attn_kernel 2, the automatic choice for head_dim 64 and for small passes;
 fp32: the automatic choice) against the CPU checker at the sizes where its splits, rings and groups can go wrong."""
 import pytest
+import torch
 
 from harness import run_and_compare
 from paper_2602_02864_b200 import workloads as wl
@@ -36,3 +37,41 @@ def test_fp32_cluster_kernel_shapes(head_dim, hq, hkv, fields, batch, prefix):
     w.max_active = w.n_nodes
     r = run_and_compare(w, check_steps={0, 1, 9, 33}, max_steps=34)
     assert r["checked"] > 0
+
+
+# fp32: what a field's rows hold is nobody's business but the fields' that see them.  Infinities and NaN in one field's K and V
+# rows (new ones and earlier ones, a tile shared with its neighbours among them) leave the other fields' results as they are, bit
+# for bit.  Query rows per pair for all tile heights of the kernel (8 / 16 / 24 / 32 rows, more than one cluster).
+@pytest.mark.parametrize("head_dim,hq,hkv,fields,batch,prefix", [
+    (64, 4, 2, 3, 2, 70), (64, 16, 2, 3, 1, 600), (128, 16, 4, 4, 1, 33), (128, 28, 4, 3, 2, 200), (128, 32, 8, 8, 9, 129), (64, 8, 2, 16, 1, 0)])
+def test_fp32_siblings_are_independent(head_dim, hq, hkv, fields, batch, prefix):
+    from paper_2602_02864_b200 import fdc
+    passes, bad = 5, 1
+    cap = [9 + 5 * (v % 4) for v in range(fields)]
+    sess = fdc.DecodeSession(fields, [], cap, None, prefix, fields, batch)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    shape = (batch, 1, hkv, prefix + sum(cap), head_dim)
+    k, v = (torch.randn(shape, generator=g, device="cuda") for _ in range(2))
+    q = torch.randn(batch, fields, hq, head_dim, generator=g, device="cuda")
+    sess.bind_cache(k, v, hq)
+    sess.init(None)
+    for _ in range(passes):
+        sess.frontier()
+    sess.build_masks()
+    r0 = prefix + sum(cap[:bad])
+
+    def attend(rows):
+        k[:, :, :, r0:r0 + passes], v[:, :, :, r0:r0 + passes] = rows
+        out = torch.zeros_like(q)
+        sess.decode_attn(0, q, out, head_dim ** -0.5)
+        return out
+
+    clean = attend((k[:, :, :, r0:r0 + passes].clone(), v[:, :, :, r0:r0 + passes].clone()))
+    assert torch.isfinite(clean).all()
+    others = [b for b in range(fields) if b != bad]
+    for kx, vx in ((0.5, float("inf")), (float("nan"), float("nan")), (float("inf"), -float("inf")), (float("nan"), 1.0)):
+        out = attend((torch.full((), kx, device="cuda"), torch.full((), vx, device="cuda")))
+        assert not torch.isfinite(out[:, bad]).all()
+        assert torch.equal(out[:, others], clean[:, others])
+    assert sess.status() == 0
+    sess.close()
