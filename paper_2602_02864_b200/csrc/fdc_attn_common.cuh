@@ -56,6 +56,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, abort_flag, status);
 }
+// The same for a warp that goes on as one: near the limit the wait can run out in some lanes and end in others, and what
+// follows (votes, elect.sync) needs all of them on the same side.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
+}
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2, int c3)
 {
     asm volatile(

@@ -194,7 +194,7 @@ __device__ __forceinline__ void qk_loop(const AttnParams& p, const Ctx& cx, long
         const int M = cx.nact[sg.s] * p.group;
         const int NP = (NP_MAX == 32 || M <= 32) ? 32 : 64;
         const uint32_t idesc_qk = instr_desc(RROWS, NP, 0);
-        bool good = ok && mbar_wait(cx.q_ready(), seg & 1, cx.abortp, p.status);
+        bool good = ok && mbar_wait_warp(cx.q_ready(), seg & 1, cx.abortp, p.status);
         for (int t = 0; t < nr && good; ++t, ++g) {
             good = mbar_wait(cx.k_full() + 8 * st, kph, cx.abortp, p.status);
             const uint32_t sb = g & (cx.ns - 1);                  // score buffer of the round

@@ -117,7 +117,7 @@ __device__ __forceinline__ void qk_loop(const AttnParams& p, const Ctx& cx, long
     while (u < hi && good) {
         const Segment sg = decode_segment(u, hi, cx.pre, p.hkv, s);
         const int ntile = sg.j1 - sg.j0;
-        good = mbar_wait(cx.q_ready(), seg & 1, cx.abortp, p.status);
+        good = mbar_wait_warp(cx.q_ready(), seg & 1, cx.abortp, p.status);
         for (int t = 0; t < ntile && good; ++t, ++g) {
             good = mbar_wait(cx.k_full() + 8 * st, kph, cx.abortp, p.status);
             if (good && g >= NBUF) good = mbar_wait(cx.pv_done() + 8 * ((g - NBUF) % NBAR), ((g - NBUF) / NBAR) & 1, cx.abortp, p.status);

@@ -478,3 +478,16 @@ def test_random_templates_larger_shapes(case):
     n = max(len(sch.simulate(w.n_nodes, w.edges, w.lens[s].tolist(), w.n_fixed)) for s in range(w.batch))
     r = run_and_compare(w, check_steps={0, 1, 2, n // 3, n // 2, n - 2, n - 1}, fused_append=bool(rng.integers(2)), kernel=3)
     assert r["steps"] == n and r["checked"] > 0
+
+
+def test_a_wait_of_a_whole_warp_gives_up_as_one():
+    """The issuing warps of the tcgen05 kernels wait with all lanes and then vote and elect: lanes that came back from a wait
+    with different answers would part there for good.  In the self-test's second warp every other lane's barrier is
+    complete; all 32 lanes must report the wait as given up all the same (64 with the first warp's, 48 without the vote)."""
+    from paper_2602_02864_b200 import fdc
+    plan = fdc.fdc_plan_graph(1, [], [4], None, 0, 1)
+    outcome = torch.zeros(1, dtype=torch.int32, device="cuda")
+    fdc.fdc_selftest_bounded_wait(plan, outcome)
+    assert fdc.fdc_status(plan, clear=True) == fdc.FDC_DEV_TIMEOUT
+    assert int(outcome.item()) == 64
+    fdc.fdc_plan_destroy(plan)
