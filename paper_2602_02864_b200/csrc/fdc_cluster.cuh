@@ -577,6 +577,30 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// Host: which cluster sizes of one kernel the devices have been asked about and can place: bit n of a device's word for
+// clusters of n blocks with one block per SM, bit 16 + n with two (with either, the SMs of a GPC decide, not the
+// launch's exact shared memory).
+struct PlaceableClusters {
+    std::atomic<uint64_t> asked[kMaxDevices] = {}, yes[kMaxDevices] = {};
+};
+inline bool cluster_placeable(const void* kernel, const cudaLaunchConfig_t& cfg, int n, bool two, PlaceableClusters& known)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return n <= 8;
+    const uint64_t bit = 1ull << (n + (two ? 16 : 0));
+    if (known.asked[dev].load(std::memory_order_acquire) & bit) return (known.yes[dev].load(std::memory_order_relaxed) & bit) != 0;
+    int clusters = 0;
+    cudaError_t e = n > 8 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : cudaSuccess;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg);
+    if (e != cudaSuccess) {
+        cudaGetLastError();                                // (no answer: left to the launch, the portable sizes only)
+        return n <= 8;
+    }
+    if (clusters > 0) known.yes[dev].fetch_or(bit, std::memory_order_relaxed);
+    known.asked[dev].fetch_or(bit, std::memory_order_release);
+    return clusters > 0;
+}
+
 // Host: shared memory of a launch, tensor maps, launch attributes.  `room`: bytes a block may use.
 template <class Math, class Kernel>
 int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const ClusterShape& h, cudaStream_t st)
@@ -591,16 +615,7 @@ int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const Cluste
     static size_t attr_smem[kMaxDevices] = {};
     int rc = raise_dynamic_smem(reinterpret_cast<const void*>(kernel), smem, attr_smem);
     if (rc) return rc;
-    if (h.nblk > 8) {
-        static std::atomic<uint64_t> wide_ok{0};           // devices on which clusters of 16 have been asked for
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return FDC_ERR_CUDA;
-        if (dev > 63 || !((wide_ok.load() >> dev) & 1)) {
-            cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-            if (e != cudaSuccess) return set_cuda_error(e);
-            if (dev <= 63) wide_ok.fetch_or(1ull << dev);
-        }
-    }
+    static PlaceableClusters known;
     alignas(64) CUtensorMap tk, tv;
     const int dtype = sizeof(typename Math::Elem) == 4 ? FDC_F32 : FDC_BF16;
     rc = get_kv_tensor_map(p.k, p, dtype, Math::D, Math::SROWS, &tk);
@@ -608,7 +623,6 @@ int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const Cluste
     rc = get_kv_tensor_map(p.v, p, dtype, Math::D, Math::SROWS, &tv);
     if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((long long)p.batch * p.hkv * h.qsplit * h.nblk));
     cfg.blockDim = dim3(Math::NW * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -616,12 +630,23 @@ int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const Cluste
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = (unsigned)h.nblk;
     at[1].val.clusterDim.y = 1;
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, tk, tv, nstage, h.nblk, h.qsplit, qrows);
+    // The cuts are made for a whole B200.  What a device cannot place (a part of one, or GPCs with fewer SMs) is
+    // launched as the next smaller clusters that it can; any size is right.
+    const int nblk = largest_placeable(h.nblk, [&](int n) {
+        cudaLaunchConfig_t one = cfg;
+        at[1].val.clusterDim.x = (unsigned)n;
+        one.gridDim = dim3((unsigned)n);
+        one.attrs = &at[1];
+        one.numAttrs = 1;
+        return cluster_placeable(reinterpret_cast<const void*>(kernel), one, n, h.per_sm > 1, known);
+    });
+    at[1].val.clusterDim.x = (unsigned)nblk;
+    cfg.gridDim = dim3((unsigned)((long long)p.batch * p.hkv * h.qsplit * nblk));
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, tk, tv, nstage, nblk, h.qsplit, qrows);
     if (e != cudaSuccess) return set_cuda_error(e);
     note_launch();
     return FDC_OK;

@@ -73,6 +73,13 @@ struct ClusterProblem {
     }
 };
 ClusterShape pick_cluster(const ClusterProblem& c, float* us);      // us (may be NULL): the estimated time
+// The largest cluster of at most `nblk` blocks that the device can place (a single block always can).
+template <class F>
+int largest_placeable(int nblk, F&& placeable)
+{
+    while (nblk > 1 && !placeable(nblk)) --nblk;
+    return nblk;
+}
 }  // namespace fdc
 
 // Everything the work split of the tcgen05 attention kernel depends on (host side).

@@ -59,3 +59,26 @@ def test_plan_rejects_bad_templates_on_host(lib):
     assert "cycle" in lib.fdc_strerror(lib.FDC_ERR_CYCLE)
     assert lib.fdc_kernel_name(1) == "ref_cuda_core"
     assert lib.fdc_launch_count() >= 0
+
+
+def test_cluster_size_that_a_device_cannot_place(tmp_path):
+    """The cut of a launch is made for a whole B200; a device that cannot place clusters of that size gets the next
+    smaller one it can, down to single blocks."""
+    import subprocess
+    src = tmp_path / "fit.cpp"
+    src.write_text('#include "fdc_internal.h"\n#include <cstdio>\n#include <cstdlib>\n'
+                   'int main(int, char** v) { const unsigned long fits = strtoul(v[2], nullptr, 0); int asked = 0;\n'
+                   'const int n = fdc::largest_placeable(atoi(v[1]), [&](int k) { ++asked; return ((fits >> k) & 1) != 0; });\n'
+                   'printf("%d %d\\n", n, asked); return 0; }\n')
+    exe = tmp_path / "fit"
+    subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2602_02864_b200", "csrc"),
+                           "-I", "/usr/local/cuda/include", str(src), "-o", str(exe)])
+
+    def largest(nblk, sizes):
+        return [int(x) for x in subprocess.check_output([str(exe), str(nblk), str(sum(1 << k for k in sizes))]).split()]
+    assert largest(16, range(1, 17)) == [16, 1]               # a whole B200: what was asked for, one look
+    assert largest(16, range(1, 13))[0] == 12
+    assert largest(16, [1, 2, 4, 8])[0] == 8
+    assert largest(6, [1, 2, 4, 8])[0] == 4
+    assert largest(8, [])[0] == 1                             # (single blocks are not asked about)
+    assert largest(1, [])[0] == 1
