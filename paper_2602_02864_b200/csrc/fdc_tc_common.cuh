@@ -312,16 +312,19 @@ struct SplitFinder {
             if (one_part && threadIdx.x == 0) {
                 // One part per CTA leaves CTAs idle when the parts per pair do not divide the CTAs evenly
                 // (64 pairs on 148 CTAs: 2 or 3 parts, a CTA carries up to 16 % more than the average).  Where the
-                // shares are long enough for a pair boundary inside a CTA to cost less than that (measured:
-                // from about 200 prefix tiles per CTA, half of that with 128 query rows, whose rounds take twice
-                // as long), equal shares of the weighted length win after all.
+                // shares are long enough for a pair boundary inside a CTA to cost less than that, equal shares of the
+                // weighted length win after all: from about 200 prefix tiles per CTA, half of that with more than 64 query
+                // rows (the row form), whose tiles take longer.  Measured there, us a layer one part / equal shares, 32 / 8
+                // heads x 128, 32 fields: 26 tiles per CTA (8 scenes, prefix 3840) 57 / 65, 60 tiles 85.9 / 85.1, 100 tiles
+                // 121 / 116, 150 tiles 165 / 158; 100 tiles in 5 scenes (40 pairs) 124 / 116, in 12 scenes (96 pairs) 153 /
+                // 125; where the parts divide well (48 pairs in 144 parts) 103 / 107.
                 long long tot = 0;
                 for (int i = 0; i < p.batch; ++i) {
                     const int nt = cx.pre[i + 1] - cx.pre[i];
                     if (nt > 0) tot += vt_of(cx, nt, nt) + W_PAIR;
                 }
                 const long long avg = tot * p.hkv / p.n_cta;
-                if (avg >= 200 * W_PREFIX && (long long)split_tpart * 100 > avg * 108) split_tpart = 0;
+                if (avg * (p.mmax > 64 ? 2 : 1) >= 200 * W_PREFIX && (long long)split_tpart * 100 > avg * 108) split_tpart = 0;
             }
             __syncthreads();
             if (threadIdx.x < 32) {

@@ -2,8 +2,10 @@
 widths around its row quadrants, segments of one and of a few tiles, prefixes that are and are not whole tiles (and
 none), more pairs than thread blocks, both ways of appending."""
 import pytest
+import torch
 
-from harness import run_and_compare
+from harness import check_close, f32, run_and_compare
+from oracle import attention as oatt
 from paper_2602_02864_b200 import workloads as wl
 
 pytestmark = pytest.mark.gpu
@@ -20,3 +22,39 @@ def test_row_form_shapes(hq, hkv, fields, batch, prefix, fused):
     assert 64 < w.max_active * (hq // hkv) <= 128
     r = run_and_compare(w, check_steps={0, 1, 9, 33}, kernel=3, max_steps=34, fused_append=fused)
     assert r["checked"] > 0
+
+
+@pytest.mark.parametrize("tiles_per_block,equal_shares", [(70, False), (112, True)])
+def test_row_form_split_of_long_prefixes(tiles_per_block, equal_shares):
+    """64 pairs on 148 blocks: one part per block leaves 20 blocks idle; from 100 prefix tiles per block every block gets an
+    equal share (seen in the scratch: block c's partial of pair i lies in slot c + i).  A sampled scene's and KV head's
+    output against the CPU checker."""
+    from paper_2602_02864_b200 import fdc
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    pairs, fields, batch, hkv, D = 64, 32, 8, 8, 128
+    prefix = tiles_per_block * sms // pairs * 64
+    sess = fdc.DecodeSession(fields, [], [64] * fields, None, prefix, fields, batch)
+    fdc.fdc_set_attn_kernel(sess.plan, 3)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    k, v = (torch.empty(batch, 1, hkv, prefix + 64 * fields, D, dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.5, generator=g) for _ in range(2))
+    q = torch.empty(batch, fields, 4 * hkv, D, dtype=torch.bfloat16, device="cuda").normal_(generator=g)
+    out = torch.zeros_like(q)
+    sess.bind_cache(k, v, 4 * hkv)
+    sess.init(None)
+    sess.frontier()
+    sess.build_masks()
+    sess.workspace.view(torch.float32).fill_(float("nan"))
+    sess.decode_attn(0, q, out, D ** -0.5)
+    assert sess.status() == 0
+    slots = 2 * sms + pairs
+    partials = sess.workspace.view(torch.float32)[:slots * 128 * D].view(slots, 128 * D)
+    written = int((~partials.isnan()).any(dim=1).nonzero().max())
+    last = sms // pairs * pairs - 1 + pairs - 1            # last block of the one-part split, last pair
+    assert written > last if equal_shares else written <= last
+    sess.close()
+    s, h = 5, 3
+    vis = torch.zeros(fields, prefix + 64 * fields, dtype=torch.bool)
+    vis[:, :prefix] = True
+    vis[torch.arange(fields), prefix + 64 * torch.arange(fields)] = True
+    ref = oatt.attention(f32(q[s, :, 4 * h:4 * h + 4]), f32(k[s, 0, h:h + 1]), f32(v[s, 0, h:h + 1]), vis.numpy(), D ** -0.5)
+    check_close(f32(out[s, :, 4 * h:4 * h + 4]), ref, "bf16")
