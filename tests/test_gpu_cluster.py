@@ -75,3 +75,29 @@ def test_fp32_siblings_are_independent(head_dim, hq, hkv, fields, batch, prefix)
         assert torch.equal(out[:, others], clean[:, others])
     assert sess.status() == 0
     sess.close()
+
+
+# The same kernel with several layers a pass (launches after the first read ahead of the dependency wait), whole schedules (the
+# cache is compared bit for bit at the end) and both ways of appending: few fields and query rows cut over several clusters;
+# more than 32 fields (two stages of new rows), cut and uncut; more parts beyond the prefix in one block than have their
+# visibility in shared memory (32 fields: 32 parts; 50: 20); a field's rows past the table that new rows are taken out of.
+@pytest.mark.parametrize("fused", [False, True], ids=["append_kernel", "append_inside_attention"])
+@pytest.mark.parametrize("head_dim,hq,hkv,fields,cap_hi,batch,prefix", [
+    (64, 14, 2, 6, 40, 2, 700), (64, 2, 2, 40, 12, 1, 200), (64, 8, 8, 32, 60, 20, 100), (128, 28, 4, 6, 40, 1, 2048), (128, 4, 2, 50, 24, 2, 300),
+    (128, 8, 8, 50, 40, 12, 20)])
+def test_cluster_kernel_whole_schedules(head_dim, hq, hkv, fields, cap_hi, batch, prefix, fused):
+    w = wl.random_template(7300 + fields + batch, n_nodes=fields, edge_prob=0.01, cap_lo=2, cap_hi=cap_hi, batch=batch, prefix_len=prefix, fixed_hi=2,
+                           hq=hq, hkv=hkv, head_dim=head_dim, dtype="bf16")
+    w.max_active, w.layers = w.n_nodes, 2
+    r = run_and_compare(w, check_steps={0, 1, 2, 11, 23, 38}, kernel=2, fused_append=fused)
+    assert r["checked"] > 0
+
+
+# fp32 with several layers a pass, whole schedules
+@pytest.mark.parametrize("head_dim,hq,hkv,fields,batch,prefix", [(64, 14, 2, 3, 2, 300), (128, 32, 8, 8, 2, 129), (128, 8, 2, 20, 1, 1000)])
+def test_fp32_cluster_kernel_whole_schedules(head_dim, hq, hkv, fields, batch, prefix):
+    w = wl.random_template(8300 + fields + batch, n_nodes=fields, edge_prob=0.1, cap_lo=2, cap_hi=30, batch=batch, prefix_len=prefix, fixed_hi=2,
+                           hq=hq, hkv=hkv, head_dim=head_dim, dtype="f32")
+    w.max_active, w.layers = w.n_nodes, 3
+    r = run_and_compare(w, check_steps={0, 1, 2, 11, 23, 38})
+    assert r["checked"] > 0

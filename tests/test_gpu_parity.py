@@ -491,3 +491,31 @@ def test_a_wait_of_a_whole_warp_gives_up_as_one():
     assert fdc.fdc_status(plan, clear=True) == fdc.FDC_DEV_TIMEOUT
     assert int(outcome.item()) == 64
     fdc.fdc_plan_destroy(plan)
+
+
+# The automatic choice between the bf16 kernels follows an estimate of their times; these run the cases above that it gives to
+# the cluster kernel on the tcgen05 kernel as well.
+@pytest.mark.parametrize("fused_append", [False, True], ids=["append_kernel", "append_inside_attention"])
+def test_more_pairs_than_thread_blocks_tcgen05(fused_append):
+    w = wl.cfg4_sweep(512, 4, 40)
+    r = run_and_compare(w, check_steps={0, 1, 2, 31, 62, 63}, kernel=3, fused_append=fused_append)
+    assert r["steps"] == 64 and r["checked"] > 0
+
+
+@pytest.mark.parametrize("which", ["cfg1", "ragged", "fixed_rows", "tail_phase"])
+def test_fused_append_in_the_tcgen05_kernel(which):
+    extra = 0
+    if which == "cfg1":
+        w, steps = wl.cfg1_7b(layers=2), set(range(0, 200, 7))
+    elif which == "ragged":
+        w, steps, extra = wl.random_template(3006, n_nodes=9, edge_prob=0.3, cap_lo=2, cap_hi=70, batch=3, prefix_len=200, fixed_hi=0,
+                                             hq=8, hkv=2, head_dim=128, dtype="bf16"), None, 30
+        w.max_active = w.n_nodes
+    elif which == "fixed_rows":
+        w, steps = wl.random_template(3000, n_nodes=5, edge_prob=0.3, cap_lo=2, cap_hi=70, batch=3, prefix_len=0, fixed_hi=3,
+                                      hq=8, hkv=2, head_dim=128, dtype="bf16"), None
+        w.max_active = w.n_nodes
+    else:
+        w, steps = _tail_template(), None
+    r = run_and_compare(w, check_steps=steps, extra_rows=extra, kernel=3, fused_append=True)
+    assert r["checked"] > 0

@@ -58,3 +58,15 @@ def test_row_form_split_of_long_prefixes(tiles_per_block, equal_shares):
     vis[torch.arange(fields), prefix + 64 * torch.arange(fields)] = True
     ref = oatt.attention(f32(q[s, :, 4 * h:4 * h + 4]), f32(k[s, 0, h:h + 1]), f32(v[s, 0, h:h + 1]), vis.numpy(), D ** -0.5)
     check_close(f32(out[s, :, 4 * h:4 * h + 4]), ref, "bf16")
+
+
+@pytest.mark.parametrize("hq,hkv,fields,batch,prefix", [(28, 4, 10, 3, 500), (32, 8, 20, 20, 129), (4, 2, 50, 1, 64)])
+def test_row_form_whole_schedules(hq, hkv, fields, batch, prefix):
+    """Several layers a pass (launches after the first read ahead of the dependency wait) with the append inside; the
+    cache is compared bit for bit at the end."""
+    w = wl.random_template(9400 + fields + batch, n_nodes=fields, edge_prob=0.02, cap_lo=2, cap_hi=30, batch=batch, prefix_len=prefix, fixed_hi=2,
+                           hq=hq, hkv=hkv, head_dim=128, dtype="bf16")
+    w.max_active, w.layers = w.n_nodes, 3
+    assert 64 < w.max_active * (hq // hkv) <= 128
+    r = run_and_compare(w, check_steps={0, 1, 2, 11, 23}, kernel=3, fused_append=True)
+    assert r["checked"] > 0
