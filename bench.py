@@ -3,7 +3,7 @@
 
 One "step" = one forward pass of the whole hot path for one batch of scenes:
 fdc_frontier -> fdc_build_masks -> for every layer: fdc_kv_append -> fdc_decode_attn
-(split-KV pass + combine pass).  The metric is achieved KV-cache bandwidth: the bytes the
+(the masked attention; with the append inside by default).  The metric is achieved KV-cache bandwidth: the bytes the
 method itself must move per step (every KV row visible to some branch read once for all
 branches and GQA heads, plus q, out, the appended rows and the bitmaps) divided by the
 step time.  Prints ONE JSON line on stdout (rank 0).
@@ -32,16 +32,18 @@ sys.path.insert(0, ROOT)
 # profiles/attn_tc_kernel_cfg2.md (dram__bytes_read.sum + dram__bytes_write.sum over the launch's
 # algorithmic bytes; traffic grows in proportion to the visited tiles, so it scales to a full-size
 # launch).  Only valid for the kernel source it was measured on: keyed by a hash of that source.
-NCU_TRAFFIC = {"kernel_sha256_16": "131986594b3087ed", "dram_bytes_per_algorithmic_byte": 1.096}
+NCU_TRAFFIC = {"kernel_sha256_16": "73b86e47dc05c024", "dram_bytes_per_algorithmic_byte": 1.094}
 
 
 def kernel_source_hash() -> str:
     import hashlib
-    path = os.path.join(ROOT, "paper_2602_02864_b200", "csrc", "fdc_attn_tc_kernel.cuh")
+    h = hashlib.sha256()
     try:
-        return hashlib.sha256(open(path, "rb").read()).hexdigest()[:16]
+        for name in ("fdc_attn_tc_kernel.cuh", "fdc_tc_common.cuh"):
+            h.update(open(os.path.join(ROOT, "paper_2602_02864_b200", "csrc", name), "rb").read())
     except OSError:
         return ""
+    return h.hexdigest()[:16]
 
 
 METRIC = "masked_decode_attn_kv_bandwidth"
@@ -64,6 +66,11 @@ def get_workload(name: str):
     f = {"cfg1": wl.cfg1_7b, "cfg2": wl.cfg2_batched, "cfg3": wl.cfg3_wide}[name]
     return f() if LAYERS_OVERRIDE is None else f(layers=LAYERS_OVERRIDE)
 
+
+# The attention kernel the library chooses for a workload's widest passes (the choice follows from the shapes).
+ATTENTION_KERNEL = {"cfg0": "attn_f32_kernel (fp32 FMAs, one cluster per scene and KV head)",
+                    "cfg1": "attn_cluster_kernel (mma.sync, clusters per scene and KV head)",
+                    "cfg2": "attn_tc_kernel (tcgen05, up to 32 query rows)", "cfg3": "attn_tc_kernel_g2 (tcgen05, 33 to 64 query rows)"}
 
 WORKLOAD_TEXT = {
     "cfg0": "configs[0] tiny fp32: 1 layer, 4q/2kv heads, D 64, batch 1, prefix 256, 6-field DAG, 16-token slots",
@@ -394,6 +401,7 @@ def run_fdc(args, rank: int, world: int):
 
     def measure(name: str, K: int, W: int, with_e2e: bool, sample_clocks: bool, reps: int, w=None):
         w = get_workload(name) if w is None else w
+        kernel_of = name if name in ATTENTION_KERNEL else "cfg2"          # (the variants are cfg2's shapes)
         n_sched = schedule_length(w)
         K = max(1, min(K, n_sched - W))
         total = W + K
@@ -460,7 +468,6 @@ def run_fdc(args, rank: int, world: int):
         prof = fdc.fdc_profile_read(sb.sess.plan)
         fdc.fdc_profile(sb.sess.plan, False)
         split_ms, split_n = prof["split_ms"], prof["split_launches"]
-        comb_ms = prof["combine_ms"]
         roof = None
         if split_n:
             iso_bytes = sum(step_bytes[W:W + n_iso]) / split_n
@@ -469,23 +476,18 @@ def run_fdc(args, rank: int, world: int):
             avg_bytes = timed_bytes / n_launch
             in_step_us = ms / n_launch * 1e3
             in_step_gbs = avg_bytes / (in_step_us * 1e-6) / 1e9
-            tc = w.dtype == "bf16" and w.head_dim == 128
             traffic = None
-            if tc and kernel_source_hash() == NCU_TRAFFIC["kernel_sha256_16"]:
+            if ATTENTION_KERNEL[kernel_of].startswith("attn_tc_kernel ") and kernel_source_hash() == NCU_TRAFFIC["kernel_sha256_16"]:
                 traffic = int(avg_bytes * NCU_TRAFFIC["dram_bytes_per_algorithmic_byte"])
-            kname = ("attn_tc_kernel (tcgen05 split-KV pass; appends the pass's rows and merges its partials itself)" if tc
-                     else "attn_ref_kernel (CUDA-core split-KV pass)")
-            roof = {"kernel": kname, "bound": "hbm", "achieved": round(in_step_gbs, 1), "peak": peak, "unit": "GB/s",
+            roof = {"kernel": ATTENTION_KERNEL[kernel_of], "bound": "hbm", "achieved": round(in_step_gbs, 1), "peak": peak, "unit": "GB/s",
                     "frac": round(in_step_gbs / peak, 4), "peak_source": peak_src,
-                    "frac_is": "frac_in_step: timed region / attention launches; frontier + build_masks (2 small kernels per "
-                               "step, < 1 %) are inside the region",
+                    "frac_is": "frac_in_step",               # timed region / attention launches; frontier + build_masks (< 1 %) are inside
                     "traffic": traffic, "launches": n_launch, "avg_launch_us": round(in_step_us, 2),
                     "algorithmic_bytes_per_launch": int(avg_bytes),
                     "frac_in_step": round(in_step_gbs / peak, 4),
                     "frac_isolated_launch": round(iso_gbs / peak, 4),
                     "isolated": {"achieved": round(iso_gbs, 1), "avg_launch_us": round(split_ms / split_n * 1e3, 2),
                                  "launches": split_n, "how": "CUDA events around every launch (no overlap with its neighbours)"},
-                    "combine_avg_launch_us": None if tc else round(comb_ms / split_n * 1e3, 2),
                     "frac_of_nominal_8TBs": round(in_step_gbs / NOMINAL_HBM_GBS, 4)}
 
         # host side: how long the calling thread needs to issue one pass (stream launches, no graph)
@@ -625,6 +627,20 @@ def run_fdc(args, rank: int, world: int):
         cpu = cpu_baseline(args.workload, budget_s=12.0)
 
     if rank == 0:
+        # the whole of it goes to stderr; the line holds what fits a short line
+        log("also", json.dumps(also))
+        log("phases", json.dumps(main["phases"]))
+        brief = {}
+        for k, v in also.items():
+            if k == "cfg4_sweep":
+                brief[k] = {"columns": ["prefix", "fields", "scenes", "layer_step_us", "speedup_over_chain"],
+                            "points": [[r["prefix"], r["branches"], r["scenes"], r["parallel"]["layer_step_us"], r["speedup_over_chain"]]
+                                       for r in v["points"]]}
+            elif k == "device_loop":
+                brief[k] = {"host_graphs_ms": v["host_replays_one_graph_per_pass"]["whole_schedule_ms"],
+                            "device_loop_ms": v["device_loop_one_graph_launch"]["whole_schedule_ms"], "passes": v["passes_counted_on_device"]}
+            else:
+                brief[k] = {x: v[x] for x in ("value", "layer_step_us", "pct_of_measured_copy")}
         line = {
             "metric": METRIC, "value": round(main["value"], 1), "unit": UNIT, "n_gpus": world, "steps": main["K"],
             "warmup": main["W"], "ms_per_step": round(main["ms_per_step"], 4), "higher_is_better": True,
@@ -642,13 +658,12 @@ def run_fdc(args, rank: int, world: int):
                                "frontier + build_masks + layers x (kv_append + decode_attn[split-KV pass with the combine fused in])"},
             "step_us": main["step_us"], "layer_step_us": main["layer_step_us"],
             "layer_step_us_separate_append": main["layer_step_us_separate_append"],
-            "region_ms": main["region_ms"], "phases": main["phases"],
+            "region_ms": main["region_ms"],
             "host_issue_us_per_step": main["host_issue_us_per_step"],
             "bytes_per_step": main["bytes_per_step"], "avg_active_branches_per_scene": round(main["avg_active_per_scene"], 2),
             "pct_of_8TBs": main["pct_of_8TBs"], "pct_of_measured_copy": main["pct_of_measured_copy"],
             "roofline": main["roofline"], "cpu_baseline": cpu, "e2e": main["e2e"], "clocks": main["clocks"],
-            "gpu_launches": int(main["launches"]), "device_status": main["status"], "also": also,
-            "paper_context": "paper reports 3.1-4.1x CoT speedup end to end on 1x A100 80GB (bf16); no kernel-level number",
+            "gpu_launches": int(main["launches"]), "device_status": main["status"], "also": brief,
         }
         print(json.dumps(line), flush=True)
 
