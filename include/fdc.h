@@ -204,14 +204,16 @@ int fdc_attn_workspace_bytes(const fdc_plan* plan, const fdc_kv_desc* kv, size_t
  * (prefix rows and the rows set in d_mask[s][b]).  q and out: DEVICE [batch][max_active][hq]
  * [head_dim] in the cache dtype; rows of unused branch slots are not touched.  Scores,
  * softmax and accumulation are fp32; bf16 output is rounded to nearest even.  Each visited
- * KV tile is read once for all branches and all heads of its KV group; invisible K/V rows
- * may hold anything (NaN included).  d_tiles must be what fdc_build_masks wrote: ascending,
+ * KV tile is read once for all branches and all heads of its KV group; K/V rows that no branch of
+ * the scene sees may hold anything (NaN included).  Infinities and NaN in a row that some branches see
+ * stay with these branches in fp32; the bf16 kernels multiply such a row by a weight of 0 for
+ * the scene's other branches, whose outputs then turn NaN too.  d_tiles must be what fdc_build_masks wrote: ascending,
  * the whole tiles of the prefix first (entry j = tile j); the kernel decides by list position
  * which tiles can hold rows that nobody may see (FDC_DEV_TILE_LIST if the list disagrees).
  * d_workspace: DEVICE, 256-byte aligned,
  * >= fdc_attn_workspace_bytes; its contents are undefined afterwards.
- * The tcgen05 kernel merges its split partials itself and keeps per-(scene, KV head) arrival
- * counters in the plan.  Its work split depends only on d_n_active / d_ntiles, so it is computed once
+ * All kernels but the CUDA-core one merge their split partials themselves; the tcgen05 kernels keep
+ * per-(scene, KV head) arrival counters for that in the plan.  Their work split depends only on d_n_active / d_ntiles, so it is computed once
  * per pass (by a small launch ahead of the pass's first attention call) and kept in the plan, checked
  * against the counts before every use: calls that use the same plan must be ordered on the GPU (one
  * stream, or events); use one plan per concurrently decoding batch.
@@ -270,11 +272,13 @@ int fdc_decode_attn_static(fdc_plan* plan, const fdc_kv_desc* kv, int32_t layer,
  * synchronising `stream`.  *host_bits receives the FDC_DEV_* bits; returns FDC_ERR_DEVICE if non-zero. */
 int fdc_status(fdc_plan* plan, int32_t* host_bits, int32_t clear, void* stream);
 
-/* Selects the split-pass kernel: 0 = automatic (fp32: 1; bf16: 3, or 2 for head_dim 64 and where
- * the shapes say that 2 is faster: few scenes, short prefixes), 1 = CUDA-core kernel (any dtype), 2 = TMA +
+/* Selects the attention kernel: 0 = automatic (fp32: TMA + packed fp32 FMAs, one thread-block cluster per
+ * (scene, KV head) or share of its query rows, a kernel that no other number selects; bf16: 3, or 2 for head_dim 64
+ * and where the shapes say that 2 is faster: few scenes, short prefixes), 1 = CUDA-core kernel (any dtype), 2 = TMA +
  * mma.sync kernel, one thread-block cluster per (scene, KV head) or per share of its query rows
  * (bf16), 3 = TMA + tcgen05/TMEM kernel (bf16, head_dim 128; head_dim 64 takes 2).  Unsupported
- * combinations use 1. */
+ * combinations use 1: fp32 with 2 or 3, and a cache that no tensor map describes (a stride of 0 over several
+ * scenes or KV heads). */
 int fdc_set_attn_kernel(fdc_plan* plan, int32_t which);
 const char* fdc_kernel_name(int32_t which);
 

@@ -252,7 +252,7 @@ namespace fdc {
 // fp32 only.  Clusters per pair: as many as 32 query rows each need, all of the same width; up to 8 and up to 16 query
 // rows are one group (QL 2, 4), up to 24 and 32 two (QL 3, 4): one group reads a stage once.  Blocks per cluster:
 // what keeps all clusters on the chip at once (one block per SM; clusters of 2, 4, 8 that fit a B200 at once: 74,
-// 33, 15), and no more than give every block at least four stages.
+// 33, 15), and no more than give every block at least two tiles (eight stages).
 int launch_attn_f32(const AttnParams& p, int head_dim, cudaStream_t st)
 {
     ClusterShape h{1, (p.mmax + 31) / 32, 1};
@@ -261,7 +261,7 @@ int launch_attn_f32(const AttnParams& p, int head_dim, cudaStream_t st)
     const long long clusters = (long long)p.batch * p.hkv * h.qsplit;
     static const int sizes[] = {2, 3, 4, 6, 8}, holds[] = {74, 45, 33, 22, 15};
     for (int i = 0; i < 5; ++i)
-        if (clusters <= (long long)holds[i] * p.n_cta / 148 && 2 * p.ntile_max >= 4 * sizes[i]) h.nblk = sizes[i];
+        if (clusters <= (long long)holds[i] * p.n_cta / 148 && p.ntile_max >= 2 * sizes[i]) h.nblk = sizes[i];
     return head_dim == 64 ? launch_d<64>(p, h, ql, st) : launch_d<128>(p, h, ql, st);
 }
 

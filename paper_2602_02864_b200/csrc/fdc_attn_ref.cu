@@ -1,7 +1,7 @@
 // Reference split-KV kernel on CUDA cores (any dtype, exact fp32 arithmetic) and the combine
 // pass.  Sec. 3.3: every visited KV tile of a (scene, KV head) pair is read once and serves
 // all branches and all GQA heads of that pair; the per-branch bitmap selects what each query
-// row may see.  Used for the fp32 configuration and as the fallback for every other one.
+// row may see.  The fallback: caches that no tensor map describes, and what asks for it by number.
 #include <cuda_bf16.h>
 
 #include "fdc_attn_common.cuh"

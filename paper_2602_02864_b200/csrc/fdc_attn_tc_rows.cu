@@ -13,7 +13,7 @@
 // In steady state a tile takes about 1150 cycles, which is what its 32 KB take at an SM's share of the memory (the
 // softmax warps need 1130 for every other tile); the first build of this form, with Q in shared memory, rounds of 128
 // rows and one thread at a time issuing behind "lane 0", took 2400.
-// One persistent CTA per SM, 12 warps (168 registers a thread):
+// One persistent CTA per SM, 12 warps (168 registers a thread, 112 bytes of spill stores and 68 of loads):
 //   warps 0-7    softmax, two groups on alternate tiles, each with an accumulator and (m, l) of its own (softmax_loop)
 //   warp 8       TMA producer of both rings (K and V stages of 16 KB, six each)
 //   warp 9       issues S = Q K^T; allocates / frees TMEM
@@ -55,7 +55,7 @@ __device__ __forceinline__ void umma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32
         ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// Barrier of the softmax warps (a named barrier).  Every call site is reached by all sixteen warps
+// Barrier of the softmax warps (a named barrier).  Every call site is reached by all eight warps
 // the same number of times whatever happens: a warp whose bounded wait ran out goes on without
 // waiting but still takes every one of these.
 __device__ __forceinline__ void soft_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NSOFT * 32) : "memory"); }
@@ -350,7 +350,8 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
 
 // One tile (64 KV rows) of one query row: the scores leave TMEM, the weights take their place (bf16 pairs in the first
 // 32 columns of the buffer).  The weights are made with the row's present reference while the maximum is taken;
-// where it turns out too low the reference is raised and the weights are made once more.  o_addr: the row's accumulator; settled() returns when no multiplication is in flight on it.
+// where it turns out too low the reference is raised and the weights are made once more.  o_addr: the row's accumulator;
+// settled() returns when no multiplication is in flight on it.
 template <bool MASKED, class F>
 __device__ __forceinline__ void softmax_tile(const uint32_t s_addr, const uint32_t o_addr, const uint64_t w, const float c, float& m, float& l,
                                              const bool begun, F&& settled)
@@ -447,7 +448,7 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, const Ctx& cx,
 {
     const int tid = threadIdx.x;                   // 0 .. NSOFT * 32 - 1
     const int grp = warp >> 2, q4 = warp & 3, gtid = tid & 127;
-    const int row = q4 * 32 + lane;                // query row; also the KV row of the round this thread clears in V
+    const int row = q4 * 32 + lane;                // query row
     const uint32_t lane_base = (uint32_t)(q4 * 32) << 16;
     const uint32_t o_addr = cx.tmem + lane_base + TM_O + grp * 128;
     const float c = p.scale_log2;

@@ -171,7 +171,8 @@ __device__ __forceinline__ float4 ld_cluster4(uint32_t addr)
     return v;
 }
 // Merge over the lanes of a block, for every (query row, 4 columns): `rows` = query rows of a lane's partial;
-// `done(row, column, m, l, sum)` takes the result.
+// `done(row, column, m, l, sum)` takes the result.  (The weights of the merges, fp32's too, are ex2.approx.ftz: two
+// units in the last place like exp2f, but a part whose maximum lies more than 2^126 below the highest counts 0.)
 template <class Math, int L, class F>
 __device__ __forceinline__ void merge_lanes_n(int tid, int M, int rows, const float2* ml, const float* part, F&& done)
 {

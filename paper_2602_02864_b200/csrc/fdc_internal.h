@@ -102,7 +102,7 @@ struct fdc_plan {
     uint32_t      tables_gen;        // bumped by every call that rewrites the pass tables (state_init, frontier, build_masks)
     uint32_t      split_gen;         // number of the last split launch (stored in the memo's header)
     fdc_split_key split_key;         // what the memo was computed for
-    uint32_t      attn_gen;          // tables_gen at the last attention launch of the tcgen05 kernel
+    uint32_t      attn_gen;          // tables_gen at the last attention launch of a kernel that reads ahead
     void*         attn_stream;       // and its stream
     int           attn_gen_valid;
     int           fuse_append;       // fdc_set_fused_append

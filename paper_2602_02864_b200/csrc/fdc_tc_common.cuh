@@ -284,11 +284,7 @@ struct SplitFinder {
                 }
             }
             __syncthreads();
-#ifdef FDC_EQUAL_SHARES
-            const bool one_part = false;                   // (development builds: always equal shares of the weighted length)
-#else
             const bool one_part = (long long)split_pairs * p.hkv <= p.n_cta;
-#endif
             if (one_part) {
                 // every thread tries sizes of its own; the smallest that fits wins
                 const uint32_t vmax = (uint32_t)vt_of(cx, split_max, split_max);

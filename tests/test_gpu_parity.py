@@ -73,8 +73,8 @@ def test_random_templates_with_fixed_tokens_and_ragged_prefix(seed):
                            prefix_len=[0, 1, 63, 64, 65, 130, 200, 7, 128, 31, 96, 5][seed], fixed_hi=seed % 4,
                            hq=8, hkv=2, head_dim=64 if seed % 2 else 128, dtype="f32" if seed % 3 else "bf16")
     w.max_active = w.n_nodes
-    # the fused-append option is on for half of them: only bf16 / head_dim 128 caches take it up, the
-    # others must go on appending with the kernel of its own
+    # the fused-append option is on for half of them: only bf16 caches take it up, the others must go on
+    # appending with the kernel of its own
     run_and_compare(w, extra_rows=seed * 5, fused_append=seed % 2 == 1 or seed == 6)
 
 
