@@ -178,7 +178,7 @@ struct MathBf16 {
     const int lane;
     const uint32_t qpanel, q_lane, k_lane, v_lane;         // lane addresses of the operands' fragments
 
-    static size_t q_bytes(int qrows) { return (size_t)qrows * D * 2; }
+    static __host__ __device__ __forceinline__ size_t q_bytes(int qrows) { return (size_t)qrows * D * 2; }
     static __device__ __forceinline__ uint32_t q_off(int qrows, int m, int dc) { return swz((uint32_t)qrows * 128, m, dc); }
     // Float offset of (row, column) of a partial [rows][D]: the columns' groups of 8 are permuted by the row
     // so that the accumulator fragments' stores spread over the banks.

@@ -35,7 +35,7 @@ struct MathF32 {
     const int qg, rg;
     const uint32_t q_lane, p_off;                          // p_off: place of the group's weights in the stage
 
-    static size_t q_bytes(int qrows) { return (size_t)qrows * QROW; }
+    static __host__ __device__ __forceinline__ size_t q_bytes(int qrows) { return (size_t)qrows * QROW; }
     static __device__ __forceinline__ uint32_t q_off(int, int m, int dc) { return (uint32_t)(m * QROW + dc * 16); }
     static __device__ __forceinline__ int part_off(int row, int col) { return row * D + col; }
     static __device__ __forceinline__ void store(float* out, const float4& x) { *reinterpret_cast<float4*>(out) = x; }

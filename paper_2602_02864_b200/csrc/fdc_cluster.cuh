@@ -15,6 +15,15 @@
 //                           it has read the stage's K rows for the last time and returns when all groups have); the warp's
 //                           accumulators and (m, l) to shared memory
 //   part_off, store         float offset of (row, column) of a partial; four results to the output
+//
+// How the blocks of a cluster merge.  Every block sends its (m, l, O), merged over its warps, straight into the shared
+// memory of the blocks that finish the rows: the result's chunks of 16 columns are dealt out over the blocks, and a
+// chunk's values travel as asynchronous stores (st.async) that count towards a barrier of the block that owns it.  That
+// is one one-way trip: no barrier of the cluster after the partials are written, no reads of other blocks' memory, none
+// at the end (a block's memory is written by those only whose bytes it waits for, and it reads its own alone).
+// Measured (us a layer, partials read from the other blocks between two barriers of the cluster / sent): one scene, 28/4
+// heads x 128, prefix 2048, six fields 11.9 / 10.1 (with the queries' lines asked into L2 ahead of the dependency wait);
+// one field, prefix 1024: 8.0 / 7.6; 16 scenes, 14/2 x 64, prefix 4096: 19.5 / 18.5; fp32, 8 scenes, prefix 2048: 87.2 / 84.8.
 #pragma once
 
 #include <cuda.h>
@@ -30,6 +39,7 @@ namespace fdc {
 constexpr int MAX_STAGES = 16;
 constexpr int MASK_WORDS = 1024;              // (tile part, field) visibility words kept in shared memory
 constexpr int MASK_HALVES = 64;               // tile parts among them at most
+constexpr int MAX_QROWS = 192;                // query rows of a cluster, whole groups
 constexpr int ROW0S = 256;                    // tile parts of the run whose first row is kept in shared memory
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
@@ -99,7 +109,9 @@ struct __align__(16) BlockState {
     int n_kept;                               // entries of kept[]
     int pad;
     float2 wml[NW * GROWS];                   // (m, l) per warp and row of its group ([lane][query row])
-    float2 cml[128];                          // (m, l) of the block per query row
+    uint64_t pushed;                          // the cluster's partials of this block's chunks have arrived
+    uint64_t pad2;
+    uint8_t fld[MAX_QROWS];                   // field of every query row of the cluster (0xff: a row past the last)
     int app_row[FDC_MAX_NODES];               // fused append: cache row of every field's new K/V vector, -1: not written
     uint32_t newbits[2 * FDC_MAX_NODES];      // [new rows 0-31, 32-63][field] the new rows that the field sees
     uint32_t seen[MASK_HALVES];               // rows of a tile part that some field sees
@@ -158,17 +170,28 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ float2 ld_cluster2(uint32_t addr)
+// Asynchronous stores into a block of the cluster; the bytes count towards `bar`, a barrier of the same block.
+__device__ __forceinline__ void st_async4(uint32_t addr, uint32_t bar, const float4& v)
 {
-    float2 v;
-    asm volatile("ld.shared::cluster.v2.f32 {%0,%1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
-    return v;
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
 }
-__device__ __forceinline__ float4 ld_cluster4(uint32_t addr)
+__device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, const float2& v)
 {
-    float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
-    return v;
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
+}
+// Where the partials of a block's chunks arrive: [block of the cluster][chunk][16 columns], then [block][chunk] (m, l).
+// Chunk k (query row k / (D / 16), columns 16 (k mod D / 16) ..) belongs to block k mod nblk and is its (k / nblk)-th.
+constexpr int CHUNK_BYTES = 16 * 4 + 8;
+__host__ __device__ __forceinline__ int chunks_of_block(int chunks, int nblk) { return (chunks + nblk - 1) / nblk; }
+// The wait for them.  A block that gives up elsewhere still sends what it has, after a second or so; the limit here is
+// several times that, so that nobody leaves while bytes for it are under way.
+static __device__ __noinline__ bool wait_pushed_slow(uint32_t bar, volatile int* abort_flag, int32_t* status)
+{
+    for (uint32_t i = 0; i < SPIN_LIMIT * 8; ++i)
+        if (mbar_try(bar, 0)) return true;
+    *abort_flag = 1;
+    atomicOr(status, FDC_DEV_TIMEOUT);
+    return false;
 }
 // Merge over the lanes of a block, for every (query row, 4 columns): `rows` = query rows of a lane's partial;
 // `done(row, column, m, l, sum)` takes the result.  (The weights of the merges, fp32's too, are ex2.approx.ftz: two
@@ -233,6 +256,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     extern __shared__ unsigned char smem_dyn[];
     unsigned char* ring = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     unsigned char* qs = ring + (size_t)nstage * STAGE_BYTES;
+    unsigned char* recv = qs + Math::q_bytes(qrows);       // partials of this block's chunks, from all blocks of the cluster
     float* part = reinterpret_cast<float*>(ring);          // after the last stage: [warp][GROWS][D] partials
     __shared__ BlockState<NW, GROWS> bs;
 
@@ -263,6 +287,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     r.np = r.h1 - r.p0;
     if (r.np > MASK_WORDS / A) r.np = MASK_WORDS / A;
     if (r.np > MASK_HALVES) r.np = MASK_HALVES;
+    const int chunks = M * (D / 16), slots = chunks_of_block(chunks, nblk);     // chunks of the result, of one block at most
     // ---- set-up: barriers, the run's rows, the fields' visibility beyond the prefix
     r.nx = p.app_row && rank == 0 ? (A + SROWS - 1) / SROWS : 0;
     if (tid == 0) {
@@ -274,11 +299,14 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             mbar_init(smem_u32(&bs.full[i]), 1);
             if (Math::K_REUSED) mbar_init(smem_u32(&bs.k_read[i]), groups);
         }
+        mbar_init(smem_u32(&bs.pushed), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
+        if (nblk > 1) mbar_expect_tx(smem_u32(&bs.pushed), nblk * ((chunks - rank + nblk - 1) / nblk) * CHUNK_BYTES);
         for (int i = 0; i < r.nx; ++i) mbar_arrive(smem_u32(&bs.full[i]));      // filled by this block itself, ahead of the main loop
     }
     if (tid < MASK_HALVES) bs.seen[tid] = 0u;
+    if (tid < MAX_QROWS) bs.fld[tid] = tid < M ? (uint8_t)((m0 + tid) / p.group) : (uint8_t)0xff;
     bool off_list = false;
     int beyond = 0x7fffffff;                               // first part of this thread's that reaches beyond the prefix
     for (int i = tid; i < r.h1 - r.h0; i += THREADS) {
@@ -288,6 +316,8 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
         off_list |= pos < PARTS * (p.P / FDC_TILE_ROWS) && row0 != pos * SROWS;
     }
     __syncthreads();
+    // (the barrier of the partials is there: the other blocks may send once they have seen this)
+    if (nblk > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     if (beyond != 0x7fffffff) atomicMin(&bs.first_beyond, beyond);
     auto cache_bits = [&]() {
         for (int i = tid; i < r.np * A; i += THREADS) {
@@ -356,7 +386,21 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             if (it >= r.nx) request(it, it, 1);
     }
     __syncwarp();
-    if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.early) {
+        // The queries and the new rows may still be written by the kernel ahead: their lines are only requested into L2
+        // (which stays coherent), so that the reads after the wait find them there.
+        constexpr int LINES = D * sizeof(typename Math::Elem) / 128;
+        for (int i = tid; i < M * LINES; i += THREADS) {
+            const int m = i / LINES, b = bs.fld[m], hg = m0 + m - b * p.group;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(p.q) + ((((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * LINES + (i - m * LINES)) * 128));
+        }
+        if (r.nx)
+            for (int i = tid; i < 2 * A * LINES; i += THREADS) {
+                const int x = i >= A * LINES, b = (i - x * A * LINES) / LINES;
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(x ? p.app_v : p.app_k) + ((((size_t)s * p.max_active + b) * p.hkv + g) * LINES + i % LINES) * 128));
+            }
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+    }
     if (lane == 0) {
         for (int it = warp; it < nstage && it < r.total; it += NW)
             if (it >= fb) request(it, it, 1);
@@ -401,9 +445,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     const int mg = warp % groups, kl = warp / groups;
     const int left = M - mg * GROWS;                       // rows of this warp's group that exist (<= 0: none)
     Math math(p, qs, qrows, left > 0 ? mg * GROWS : 0, lane);
-    int fld[Math::ROWS];                                   // fields of the thread's query rows
-#pragma unroll
-    for (int i = 0; i < Math::ROWS; ++i) fld[i] = math.row(i) < left ? (m0 + mg * GROWS + math.row(i)) / p.group : -1;
+    const uint8_t* fld = bs.fld + mg * GROWS;              // fields of the group's query rows
     bool alive = true;
     int st = kl, use = 1;                                  // slot of stage `it`, and how many stages (this one included) have used it
     while (st >= nstage) {
@@ -421,7 +463,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             if (it < r.nx) {
                 masked = true;
 #pragma unroll
-                for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[i] < 0 ? 0u : bs.newbits[it * FDC_MAX_NODES + fld[i]];
+                for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[math.row(i)] == 0xff ? 0u : bs.newbits[it * FDC_MAX_NODES + fld[math.row(i)]];
                 for (int b = 0; b < SROWS && it * SROWS + b < A; ++b)     // (values of rows that are not written do not count either)
                     if (bs.app_row[it * SROWS + b] < 0) seen &= ~(1u << b);
             } else if (it >= fb) {
@@ -430,12 +472,12 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
                     masked = true;
                     if (h >= 0 && h < r.np) {
 #pragma unroll
-                        for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[i] < 0 ? 0u : bs.bits[h * A + fld[i]];
+                        for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[math.row(i)] == 0xff ? 0u : bs.bits[h * A + fld[math.row(i)]];
                         seen = bs.seen[h];
                     } else {
                         const uint32_t fresh = p.app_row ? new_rows_of<SROWS>(bs.app_row, A, row0) : 0u;
 #pragma unroll
-                        for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[i] < 0 ? 0u : part_bits<SROWS>(r.mask + (size_t)fld[i] * p.W, p.W, p.P, row0) & ~fresh;
+                        for (int i = 0; i < Math::ROWS; ++i) mk[i] = fld[math.row(i)] == 0xff ? 0u : part_bits<SROWS>(r.mask + (size_t)fld[math.row(i)] * p.W, p.W, p.P, row0) & ~fresh;
                         seen = part_seen_slow<SROWS>(r.mask, p.W, p.P, A, row0) & ~fresh;
                     }
                 }
@@ -491,19 +533,20 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
         Math::store(reinterpret_cast<typename Math::Elem*>(p.out) + (((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * D + c4,
                     make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
     };
-    // block: merge over the warps of a group; with one block per pair that is the result
+    // block: merge over the warps of a group; with one block per pair that is the result, else it is sent to the chunk's block
+    if (nblk > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");       // (long complete: all blocks have set up their barriers)
+    const uint32_t recv0 = smem_u32(recv), recv_ml0 = recv0 + (uint32_t)(nblk * slots * 64), pushed = smem_u32(&bs.pushed);
+    const uint32_t by_nblk = 65536u / (uint32_t)nblk + 1u;                                  // k / nblk for k < 4096 by a multiplication
     merge_lanes<Math>(lanes, tid, M, groups * GROWS, bs.wml, part, [&](int mm, int c4, float mx, float lt, const float4& acc) {
         if (nblk == 1) {
             store_out(mm, c4, acc, lt);
         } else {
-            *reinterpret_cast<float4*>(part + Math::part_off(mm, c4)) = acc;          // in place of the first lane's partial (one thread reads and writes it)
-            if (c4 == 0) bs.cml[mm] = make_float2(mx, lt);
+            const uint32_t k = (uint32_t)(mm * (D / 16) + (c4 >> 4)), slot = (k * by_nblk) >> 16, owner = k - slot * (uint32_t)nblk;
+            const uint32_t at = (uint32_t)(rank * slots) + slot, bar = map_rank(pushed, owner);
+            st_async4(map_rank(recv0 + at * 64 + (uint32_t)(c4 & 15) * 4, owner), bar, acc);
+            if ((c4 & 15) == 0) st_async2(map_rank(recv_ml0 + at * 8, owner), bar, make_float2(mx, lt));
         }
     });
-    if (nblk > 1) {
-        __syncwarp();
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    }
     // fused append: the new rows whose tile parts are in this block's run go to the cache (this block's copies
     // from there have landed; clusters with the pair's other query rows may still be reading the
     // part, but to them, too, the row counts as unseen: its bytes there do not matter)
@@ -525,17 +568,17 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             }
         }
     if (nblk == 1) return;
-    // ---- cluster: every block merges its share of the (query row, 4 columns) items over all blocks
+    // ---- cluster: every block finishes its chunks once all blocks' partials of them are there
+    if (!mbar_try(pushed, 0)) wait_pushed_slow(pushed, abortp, p.status);
     __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     {
-        // Four threads per item, each with every fourth block (at most four: one trip), summed by shuffles.
-        const uint32_t ml0 = smem_u32(bs.cml), part0 = smem_u32(part);
-        const int q = tid & 3, items = M * (D / 4);
-        for (int i0 = (tid >> 2) * nblk + rank; __any_sync(0xffffffffu, i0 < items); i0 += (THREADS / 4) * nblk) {
-            const bool on = i0 < items;
-            const int mm = on ? i0 / (D / 4) : 0, c4 = on ? (i0 - mm * (D / 4)) * 4 : 0;
-            const uint32_t a_ml = ml0 + mm * 8, a_o = part0 + 4 * Math::part_off(mm, c4);
+        // Four threads per item (4 columns), each with every fourth block (at most four), summed by shuffles.
+        const float4* ro = reinterpret_cast<const float4*>(recv);
+        const float2* rml = reinterpret_cast<const float2*>(recv + (size_t)nblk * slots * 64);
+        const int q = tid & 3, items = (chunks - rank + nblk - 1) / nblk * 4;
+        for (int i = tid >> 2; __any_sync(0xffffffffu, i < items); i += THREADS / 4) {
+            const bool on = i < items;
+            const int slot = on ? i >> 2 : 0, k = slot * nblk + rank, mm = k / (D / 16), c4 = (k - mm * (D / 16)) * 16 + (i & 3) * 4;
             float2 v[4];
             float4 x[4];
 #pragma unroll
@@ -543,8 +586,9 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
                 v[j] = make_float2(-INFINITY, 0.f);
                 x[j] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (on && q + 4 * j < nblk) {
-                    v[j] = ld_cluster2(map_rank(a_ml, q + 4 * j));
-                    x[j] = ld_cluster4(map_rank(a_o, q + 4 * j));
+                    const int at = (q + 4 * j) * slots + slot;
+                    v[j] = rml[at];
+                    x[j] = ro[at * 4 + (i & 3)];
                 }
             }
             float mx = fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x));
@@ -573,9 +617,6 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             if (on && q == 0) store_out(mm, c4, acc, lt);
         }
     }
-    __syncwarp();
-    // nobody leaves while its shared memory is still being read
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // Host: which cluster sizes of one kernel the devices have been asked about and can place: bit n of a device's word for
@@ -607,7 +648,8 @@ template <class Math, class Kernel>
 int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const ClusterShape& h, cudaStream_t st)
 {
     const int qrows = ((p.mmax + Math::GROWS - 1) / Math::GROWS + h.qsplit - 1) / h.qsplit * Math::GROWS;
-    const size_t fixed = 1024 + Math::q_bytes(qrows);
+    const size_t recv = h.nblk > 1 ? (size_t)(qrows * (Math::D / 16) + h.nblk) * CHUNK_BYTES : 0;      // (for any number of blocks up to this one)
+    const size_t fixed = 1024 + Math::q_bytes(qrows) + recv;
     int nstage = (int)((room - sizeof(BlockState<Math::NW, Math::GROWS>) - 256 - fixed) / Math::STAGE_BYTES);
     if (nstage > MAX_STAGES) nstage = MAX_STAGES;
     if ((size_t)nstage * Math::STAGE_BYTES < (size_t)Math::NW * Math::GROWS * Math::D * 4) return FDC_ERR_SHAPE;      // the partials take the ring's place
