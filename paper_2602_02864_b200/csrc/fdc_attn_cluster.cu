@@ -297,6 +297,12 @@ int get_kv_tensor_map(const void* base, const AttnParams& p, int dtype, int head
     return get_map(base, p, dtype, head_dim, box_rows, reinterpret_cast<CUtensorMap*>(out_map));
 }
 
+static size_t block_room(int per_sm) { return per_sm > 1 ? 113 * 1024 : 227 * 1024; }       // two blocks per SM: 228 KB, less 1 KB each for the system
+// Whether a block of a cluster of n with `rows` query rows finds room for what the other blocks send it, beside a ring that its
+// own partials fit.  (With two blocks per SM and head_dim 128: up to 48 rows in clusters of more than one block.)
+template <int D>
+static bool fits(int rows, int n, int two) { return cluster_ring_stages<MathBf16<D>>(block_room(two + 1), rows, n) > 0; }
+
 // How a launch is cut: blocks per cluster (shares of a pair's rows), clusters per pair (shares of its query
 // rows; each reads all the pair's K/V, the later ones from L2) and blocks per SM, by the lowest estimate of
 //     fixed + waves x (one block's time)
@@ -328,6 +334,7 @@ ClusterShape pick_cluster(const ClusterProblem& c, float* us)
             for (int two = 0; two < 2; ++two) {
                 const float n = (float)sizes[i], clusters = pairs * (float)q, hold = (float)holds[two][i] * (float)c.sm_count / 148.f;
                 if (sizes[i] > 1 && stages < 2.f * n) continue;
+                if (!(d64 ? fits<64>(gl * 16, sizes[i], two) : fits<128>(gl * 16, sizes[i], two))) continue;
                 const float waves = clusters > hold ? clusters / hold + 0.4f : 1.f;
                 const float share = two ? fminf(2.f, fmaxf(1.f, clusters * n / (float)c.sm_count)) : 1.f;
                 const float sb = ceilf(stages / n);
@@ -347,7 +354,7 @@ ClusterShape pick_cluster(const ClusterProblem& c, float* us)
 // then uses the CUDA-core kernel).
 int launch_attn_cluster(const AttnParams& p, int head_dim, cudaStream_t st)
 {
-    const size_t room = p.cluster.per_sm > 1 ? 113 * 1024 : 227 * 1024;     // two blocks per SM: 228 KB, less 1 KB each for the system
+    const size_t room = block_room(p.cluster.per_sm);
     return head_dim == 64 ? launch_cluster<MathBf16<64>>(attn_cluster_kernel<64>, p, room, p.cluster, st)
                           : launch_cluster<MathBf16<128>>(attn_cluster_kernel<128>, p, room, p.cluster, st);
 }

@@ -643,17 +643,31 @@ inline bool cluster_placeable(const void* kernel, const cudaLaunchConfig_t& cfg,
     return clusters > 0;
 }
 
+// Host: shared memory of a block besides its ring, and the ring's stages in `room` bytes (0: the partials, which take the
+// ring's place after the last stage, would not fit it).
+template <class Math>
+size_t cluster_smem_fixed(int qrows, int nblk)
+{
+    const size_t recv = nblk > 1 ? (size_t)(qrows * (Math::D / 16) + nblk) * CHUNK_BYTES : 0;      // (for any number of blocks up to this one)
+    return 1024 + Math::q_bytes(qrows) + recv;
+}
+template <class Math>
+int cluster_ring_stages(size_t room, int qrows, int nblk)
+{
+    const long long left = (long long)room - (long long)(sizeof(BlockState<Math::NW, Math::GROWS>) + 256 + cluster_smem_fixed<Math>(qrows, nblk));
+    const int n = left > 0 ? (int)(left / Math::STAGE_BYTES) : 0;
+    if (n * Math::STAGE_BYTES < Math::NW * Math::GROWS * Math::D * 4) return 0;
+    return n > MAX_STAGES ? MAX_STAGES : n;
+}
+
 // Host: shared memory of a launch, tensor maps, launch attributes.  `room`: bytes a block may use.
 template <class Math, class Kernel>
 int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const ClusterShape& h, cudaStream_t st)
 {
     const int qrows = ((p.mmax + Math::GROWS - 1) / Math::GROWS + h.qsplit - 1) / h.qsplit * Math::GROWS;
-    const size_t recv = h.nblk > 1 ? (size_t)(qrows * (Math::D / 16) + h.nblk) * CHUNK_BYTES : 0;      // (for any number of blocks up to this one)
-    const size_t fixed = 1024 + Math::q_bytes(qrows) + recv;
-    int nstage = (int)((room - sizeof(BlockState<Math::NW, Math::GROWS>) - 256 - fixed) / Math::STAGE_BYTES);
-    if (nstage > MAX_STAGES) nstage = MAX_STAGES;
-    if ((size_t)nstage * Math::STAGE_BYTES < (size_t)Math::NW * Math::GROWS * Math::D * 4) return FDC_ERR_SHAPE;      // the partials take the ring's place
-    size_t smem = fixed + (size_t)nstage * Math::STAGE_BYTES;
+    const int nstage = cluster_ring_stages<Math>(room, qrows, h.nblk);
+    if (nstage == 0) return FDC_ERR_SHAPE;
+    size_t smem = cluster_smem_fixed<Math>(qrows, h.nblk) + (size_t)nstage * Math::STAGE_BYTES;
     if (h.per_sm <= 1 && smem < 120 * 1024) smem = 120 * 1024;        // (more than half of an SM's: no second block beside this one)
     static size_t attr_smem[kMaxDevices] = {};
     int rc = raise_dynamic_smem(reinterpret_cast<const void*>(kernel), smem, attr_smem);

@@ -101,3 +101,22 @@ def test_fp32_cluster_kernel_whole_schedules(head_dim, hq, hkv, fields, batch, p
     w.max_active, w.layers = w.n_nodes, 3
     r = run_and_compare(w, check_steps={0, 1, 2, 11, 23, 38})
     assert r["checked"] > 0
+
+
+# Every cut that the library takes can be launched: one kernel a call (a call that fell back would launch two).  The shapes' best cut by the
+# estimate alone, clusters of two blocks with 80 and 112 query rows and two blocks per SM, finds no room for the partials.
+@pytest.mark.parametrize("hq,hkv,fields,batch,prefix", [(20, 4, 16, 32, 1024), (28, 4, 16, 24, 2048), (128, 8, 8, 3, 512)])
+def test_the_cut_leaves_room_for_the_partials(hq, hkv, fields, batch, prefix):
+    from paper_2602_02864_b200 import fdc
+    sess = fdc.DecodeSession(fields, [], [16] * fields, None, prefix, fields, batch)
+    k, v = (torch.randn(batch, 1, hkv, prefix + 16 * fields, 128, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    q = torch.randn(batch, fields, hq, 128, device="cuda", dtype=torch.bfloat16)
+    sess.bind_cache(k, v, hq)
+    fdc.fdc_set_attn_kernel(sess.plan, 2)
+    sess.init(None)
+    sess.frontier()
+    sess.build_masks()
+    before = fdc.fdc_launch_count()
+    sess.decode_attn(0, q, torch.empty_like(q), 128 ** -0.5)
+    assert fdc.fdc_launch_count() == before + 1 and sess.status() == 0
+    sess.close()
