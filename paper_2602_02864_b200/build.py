@@ -1,15 +1,18 @@
-"""Builds libfdc.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libfdc.so (the C-ABI CUDA library) with nvcc for sm_100a and the binding's extension module, in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libfdc.so")
+BIND_SRC = os.path.join(CSRC, "fdc_bind.c")
+BIND = os.path.join(HERE, "_fdc_bind" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC,-Wall,-Wno-unused-function", "--expt-relaxed-constexpr"]
@@ -19,15 +22,25 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def _stale(out, deps) -> bool:
+    return not os.path.exists(out) or any(os.path.getmtime(d) > os.path.getmtime(out) for d in deps)
+
+
 def needs_build() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    return _stale(LIB, sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(ROOT, "include", "*.h")))
+
+
+def build_bind(force: bool = False) -> str:
+    if force or _stale(BIND, [BIND_SRC] + glob.glob(os.path.join(ROOT, "include", "*.h"))):
+        tmp = BIND + f".{os.getpid()}.tmp"
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                               "-I", os.path.join(ROOT, "include"), BIND_SRC, "-o", tmp])
+        os.replace(tmp, BIND)
+    return BIND
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_bind(force)
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libfdc.so: same names as the C ABI, argument marshalling only.
+"""Thin binding of libfdc.so: same names as the C ABI, argument marshalling only (ctypes; the calls of a pass go
+through the extension module _fdc_bind, which converts the usual arguments in a tenth of the time).
 
 Every step of the path (scheduling, bitmaps, KV append, attention) runs in the library's
 CUDA kernels; PyTorch is used here for device memory and streams.  Importing this module
@@ -19,6 +20,7 @@ if not os.path.exists(LIB_PATH):
     raise ImportError(f"{LIB_PATH} is missing: build it with `python -m paper_2602_02864_b200.build` "
                       "(there is no fallback path)")
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _fdc_bind  # noqa: E402  (built beside the library)
 
 FDC_MAX_NODES, FDC_TILE_ROWS, FDC_MAX_QROWS, FDC_MAX_BATCH = 64, 64, 128, 4096
 FDC_OK = 0
@@ -86,6 +88,10 @@ _profile_read = _sig("fdc_profile_read", c_i32, c_vp, ctypes.POINTER(ctypes.c_fl
 _launch_count = _sig("fdc_launch_count", c_i64)
 _strerror = _sig("fdc_strerror", ctypes.c_char_p, c_i32)
 _last_cuda_error = _sig("fdc_last_cuda_error", ctypes.c_char_p)
+
+
+# A call of these returns None when an argument is not of the usual kind: the same call is then made through ctypes.
+_fdc_bind.setup(torch.Tensor, fdc_kv_desc, *(ctypes.cast(f, c_vp).value for f in (_frontier, _build_masks, _kv_append, _decode_attn)))
 
 
 class FdcError(RuntimeError):
@@ -172,18 +178,28 @@ def fdc_state_init(plan, batch, d_len, d_state, stream=None) -> None:
 
 def fdc_frontier(plan, batch, d_state, d_finish, d_n_active, d_node, d_tok_idx, d_kv_row, d_pos_id, d_all_done,
                  stream=None) -> None:
-    _check(_frontier(plan, batch, _ptr(d_state), _ptr(d_finish), _ptr(d_n_active), _ptr(d_node), _ptr(d_tok_idx),
-                     _ptr(d_kv_row), _ptr(d_pos_id), _ptr(d_all_done), _stream(stream)), "fdc_frontier")
+    st = _stream(stream)
+    rc = _fdc_bind.frontier(plan, batch, d_state, d_finish, d_n_active, d_node, d_tok_idx, d_kv_row, d_pos_id, d_all_done, st)
+    if rc is None:
+        rc = _frontier(plan, batch, _ptr(d_state), _ptr(d_finish), _ptr(d_n_active), _ptr(d_node), _ptr(d_tok_idx), _ptr(d_kv_row),
+                       _ptr(d_pos_id), _ptr(d_all_done), st)
+    _check(rc, "fdc_frontier")
 
 
 def fdc_build_masks(plan, batch, d_state, d_mask, d_umask, d_tiles, d_ntiles, stream=None) -> None:
-    _check(_build_masks(plan, batch, _ptr(d_state), _ptr(d_mask), _ptr(d_umask), _ptr(d_tiles), _ptr(d_ntiles),
-                        _stream(stream)), "fdc_build_masks")
+    st = _stream(stream)
+    rc = _fdc_bind.build_masks(plan, batch, d_state, d_mask, d_umask, d_tiles, d_ntiles, st)
+    if rc is None:
+        rc = _build_masks(plan, batch, _ptr(d_state), _ptr(d_mask), _ptr(d_umask), _ptr(d_tiles), _ptr(d_ntiles), st)
+    _check(rc, "fdc_build_masks")
 
 
 def fdc_kv_append(plan, kv: fdc_kv_desc, layer, d_n_active, d_kv_row, d_k_new, d_v_new, stream=None) -> None:
-    _check(_kv_append(plan, ctypes.byref(kv), layer, _ptr(d_n_active), _ptr(d_kv_row), _ptr(d_k_new), _ptr(d_v_new),
-                      _stream(stream)), "fdc_kv_append")
+    st = _stream(stream)
+    rc = _fdc_bind.kv_append(plan, kv, layer, d_n_active, d_kv_row, d_k_new, d_v_new, st)
+    if rc is None:
+        rc = _kv_append(plan, ctypes.byref(kv), layer, _ptr(d_n_active), _ptr(d_kv_row), _ptr(d_k_new), _ptr(d_v_new), st)
+    _check(rc, "fdc_kv_append")
 
 
 def fdc_kv_write_fixed(plan, kv: fdc_kv_desc, layer, d_k_fixed, d_v_fixed, stream=None) -> None:
@@ -199,9 +215,12 @@ def fdc_attn_workspace_bytes(plan, kv: fdc_kv_desc) -> int:
 
 def fdc_decode_attn(plan, kv: fdc_kv_desc, layer, d_n_active, d_mask, d_tiles, d_ntiles, d_q, d_out, scale,
                     d_workspace, ws_bytes, stream=None) -> None:
-    _check(_decode_attn(plan, ctypes.byref(kv), layer, _ptr(d_n_active), _ptr(d_mask), _ptr(d_tiles), _ptr(d_ntiles),
-                        _ptr(d_q), _ptr(d_out), float(scale), _ptr(d_workspace), int(ws_bytes), _stream(stream)),
-           "fdc_decode_attn")
+    st = _stream(stream)
+    rc = _fdc_bind.decode_attn(plan, kv, layer, d_n_active, d_mask, d_tiles, d_ntiles, d_q, d_out, scale, d_workspace, ws_bytes, st)
+    if rc is None:
+        rc = _decode_attn(plan, ctypes.byref(kv), layer, _ptr(d_n_active), _ptr(d_mask), _ptr(d_tiles), _ptr(d_ntiles), _ptr(d_q), _ptr(d_out),
+                          float(scale), _ptr(d_workspace), int(ws_bytes), st)
+    _check(rc, "fdc_decode_attn")
 
 
 def fdc_decode_attn_static(plan, kv: fdc_kv_desc, layer, d_n_active, d_mask, d_tiles, d_ntiles, d_q, d_out, scale,
