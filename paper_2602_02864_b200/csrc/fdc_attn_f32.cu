@@ -19,10 +19,10 @@ using namespace fdc;
 
 namespace {
 
-template <int HEAD_DIM, int QLANE>
+template <int HEAD_DIM, int QLANE, int NWARPS, int NGROUPS>
 struct MathF32 {
     using Elem = float;
-    static constexpr int D = HEAD_DIM, NW = 12, SROWS = 16, JR = SROWS / 8, QL = QLANE, GROWS = 4 * QL, GROUPS = 2, ROWS = QL, STAGE_BYTES = 2 * SROWS * D * 4;
+    static constexpr int D = HEAD_DIM, NW = NWARPS, SROWS = 16, JR = SROWS / 8, QL = QLANE, GROWS = 4 * QL, GROUPS = NGROUPS, ROWS = QL, STAGE_BYTES = 2 * SROWS * D * 4;
     static constexpr bool PREFIX_FIRST = false, FUSES = false, K_REUSED = true;
     static constexpr int QP = (QL + 1) / 2 * 2;            // weights per lane and KV row in shared memory (pairs)
     static constexpr int QROW = (D + 4) * 4;               // bytes of a query row in shared memory (16 more: neighbouring rows on other banks)
@@ -226,12 +226,12 @@ struct MathF32 {
     }
 };
 
-template <int D, int QL>
-__global__ void __launch_bounds__(MathF32<D, QL>::NW * 32, 1)
+template <int D, int QL, int NW, int GROUPS>
+__global__ void __launch_bounds__(NW * 32, 1)
 attn_f32_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const int nstage,
                 const int nblk, const int qsplit, const int qrows)
 {
-    attn_cluster_body<MathF32<D, QL>>(p, tm_k, tm_v, nstage, nblk, qsplit, qrows);
+    attn_cluster_body<MathF32<D, QL, NW, GROUPS>>(p, tm_k, tm_v, nstage, nblk, qsplit, qrows);
 }
 
 template <int D>
@@ -239,9 +239,10 @@ int launch_d(const AttnParams& p, const ClusterShape& h, int ql, cudaStream_t st
 {
     const size_t room = 227 * 1024;
     switch (ql) {
-        case 2: return launch_cluster<MathF32<D, 2>>(attn_f32_kernel<D, 2>, p, room, h, st);
-        case 3: return launch_cluster<MathF32<D, 3>>(attn_f32_kernel<D, 3>, p, room, h, st);
-        default: return launch_cluster<MathF32<D, 4>>(attn_f32_kernel<D, 4>, p, room, h, st);
+        case 2: return launch_cluster<MathF32<D, 2, 12, 2>>(attn_f32_kernel<D, 2, 12, 2>, p, room, h, st);
+        case 4: return launch_cluster<MathF32<D, 4, 12, 2>>(attn_f32_kernel<D, 4, 12, 2>, p, room, h, st);
+        case 6: return launch_cluster<MathF32<D, 6, 8, 1>>(attn_f32_kernel<D, 6, 8, 1>, p, room, h, st);
+        default: return launch_cluster<MathF32<D, 8, 8, 1>>(attn_f32_kernel<D, 8, 8, 1>, p, room, h, st);
     }
 }
 
@@ -256,8 +257,8 @@ namespace fdc {
 int launch_attn_f32(const AttnParams& p, int head_dim, cudaStream_t st)
 {
     ClusterShape h{1, (p.mmax + 31) / 32, 1};
-    const int per = (p.mmax + h.qsplit - 1) / h.qsplit, ql = per <= 8 ? 2 : (per > 16 && per <= 24 ? 3 : 4);
-    if (ql == 3) h.qsplit = (p.mmax + 23) / 24;
+    const int per = (p.mmax + h.qsplit - 1) / h.qsplit, ql = per <= 8 ? 2 : (per <= 16 ? 4 : (per <= 24 ? 6 : 8));
+    if (ql == 6) h.qsplit = (p.mmax + 23) / 24;
     const long long clusters = (long long)p.batch * p.hkv * h.qsplit;
     static const int sizes[] = {2, 3, 4, 6, 8}, holds[] = {74, 45, 33, 22, 15};
     for (int i = 0; i < 5; ++i)
