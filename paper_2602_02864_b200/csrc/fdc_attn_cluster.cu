@@ -202,13 +202,13 @@ struct MathBf16 {
     {
         process_stage<D>(kb + k_lane, kb + v_lane, q_lane, qpanel, o, l, m, masked, mk[0], mk[1], seen, c, lane);
     }
-    __device__ __forceinline__ void write(float* part, float2* ml) const
+    __device__ __forceinline__ void write(float* part, float2* ml, int rows) const      // (of the first `rows` query rows)
     {
         const int gq = lane >> 2, cq = lane & 3;
 #pragma unroll
         for (int n = 0; n < D / 8; ++n) {
-            *reinterpret_cast<float2*>(part + part_off(gq, n * 8 + 2 * cq)) = make_float2(o[n][0], o[n][1]);
-            *reinterpret_cast<float2*>(part + part_off(gq + 8, n * 8 + 2 * cq)) = make_float2(o[n][2], o[n][3]);
+            if (gq < rows) *reinterpret_cast<float2*>(part + part_off(gq, n * 8 + 2 * cq)) = make_float2(o[n][0], o[n][1]);
+            if (gq + 8 < rows) *reinterpret_cast<float2*>(part + part_off(gq + 8, n * 8 + 2 * cq)) = make_float2(o[n][2], o[n][3]);
         }
         if (cq == 0) {
             ml[gq] = make_float2(m[0] * c, l[0]);

@@ -118,27 +118,34 @@ struct MathF32 {
         for (int i = 0; i < QL; ++i)
 #pragma unroll
             for (int j = 0; j < JR; ++j) s2[i][j] = 0ull;
-        // S = Q K^T: columns 4 d4 .. + 3 sit in chunk d4 of their panel, XORed with the row.  (Reading a step's operands
-        // ahead of the step before costs registers and gains nothing here, unlike below.)
+        // S = Q K^T: columns 4 d4 .. + 3 sit in chunk d4 of their panel, XORed with the row.  With two warps per scheduler (one
+        // group) a step's operands are read a step ahead; with three that costs registers and gains nothing.
+        constexpr int AHEAD = GROUPS == 1 && QL <= 6 ? 1 : 0;
+        uint64_t k[AHEAD + 1][JR][2], q[AHEAD + 1][QL][2];
+        auto load = [&](auto B, uint32_t kc, uint32_t qc) {
+#pragma unroll
+            for (int j = 0; j < JR; ++j) lds4(kc + j * 1024, k[B][j][0], k[B][j][1]);
+#pragma unroll
+            for (int i = 0; i < QL; ++i) lds4(qc + i * 4 * QROW, q[B][i][0], q[B][i][1]);
+        };
+        uint32_t ka = kb + (uint32_t)rg * 128, qa = q_lane;
+        if (AHEAD) load(std::integral_constant<int, 0>{}, ka + (uint32_t)(rg << 4), qa);
 #pragma unroll 1
         for (int h = 0; h < D / 32; ++h) {
-            const uint32_t ka = kb + (uint32_t)h * (SROWS * 128) + (uint32_t)rg * 128, qa = q_lane + (uint32_t)h * 128;
-#pragma unroll
-            for (int d4 = 0; d4 < 8; ++d4) {
-                uint64_t k[JR][2];
-                const uint32_t kc = ka + (uint32_t)((d4 ^ rg) << 4);
-#pragma unroll
-                for (int j = 0; j < JR; ++j) lds4(kc + j * 1024, k[j][0], k[j][1]);
+            static_for<8>([&](auto D4) {
+                constexpr int d4 = D4, at = (d4 + AHEAD) & 7, step = (d4 + AHEAD) >> 3;     // (past the last panel: what lies there is not used)
+                load(std::integral_constant<int, AHEAD ? (d4 + 1) & 1 : 0>{}, ka + step * (SROWS * 128) + (uint32_t)((at ^ rg) << 4), qa + step * 128 + at * 16);
+                constexpr int use = AHEAD ? d4 & 1 : 0;
 #pragma unroll
                 for (int i = 0; i < QL; ++i) {
-                    uint64_t q0, q1;
-                    lds4(qa + i * 4 * QROW + d4 * 16, q0, q1);
 #pragma unroll
-                    for (int j = 0; j < JR; ++j) s2[i][j] = fma2(q0, k[j][0], s2[i][j]);
+                    for (int j = 0; j < JR; ++j) s2[i][j] = fma2(q[use][i][0], k[use][j][0], s2[i][j]);
 #pragma unroll
-                    for (int j = 0; j < JR; ++j) s2[i][j] = fma2(q1, k[j][1], s2[i][j]);
+                    for (int j = 0; j < JR; ++j) s2[i][j] = fma2(q[use][i][1], k[use][j][1], s2[i][j]);
                 }
-            }
+            });
+            ka += SROWS * 128;
+            qa += 128;
         }
         float s[QL][JR];
 #pragma unroll
@@ -212,7 +219,7 @@ struct MathF32 {
         __syncwarp();
         fence_async_smem();                                // the stage's next copy goes through the asynchronous proxy
     }
-    __device__ __forceinline__ void write(float* part, float2* ml)
+    __device__ __forceinline__ void write(float* part, float2* ml, int)
     {
 #pragma unroll
         for (int i = 0; i < QL; ++i) {

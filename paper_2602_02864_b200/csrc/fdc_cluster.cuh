@@ -130,11 +130,24 @@ struct Run {
     int nx;                                   // stages of new rows, ahead of the tile parts
     int total;                                // stages
 };
+// First position of block `rank`'s run among `parts` tile parts, the first `pre` of them whole prefix.  A part beyond the
+// prefix counts half: while fields are being decoded, about half of their slots' parts hold no row yet and are left out.
+__device__ __forceinline__ int run_begin(int rank, int nblk, int parts, int pre)
+{
+    if (pre > parts) pre = parts;
+    const int x = (int)((long long)rank * (parts + pre) / nblk);
+    return x <= 2 * pre ? (x + 1) >> 1 : x - pre;
+}
+template <int SROWS>
+__device__ __forceinline__ int list_row0(const Run& r, int pos)
+{
+    return r.tiles[pos / (FDC_TILE_ROWS / SROWS)] * FDC_TILE_ROWS + pos % (FDC_TILE_ROWS / SROWS) * SROWS;
+}
 template <int SROWS, class Block>
 __device__ __forceinline__ int part_row0(const Run& r, const Block& bs, int pos)
 {
     const int i = pos - r.h0;
-    return i < ROW0S ? bs.row0[i] : r.tiles[pos / (FDC_TILE_ROWS / SROWS)] * FDC_TILE_ROWS + pos % (FDC_TILE_ROWS / SROWS) * SROWS;
+    return i < ROW0S ? bs.row0[i] : list_row0<SROWS>(r, pos);
 }
 template <class Block>
 __device__ __forceinline__ int stage_pos(const Run& r, const Block& bs, int it)
@@ -269,6 +282,8 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     // tables and the prefix rows may be read ahead of the wait; every thread passes the wait.
     if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // (the launch may be ahead of whatever writes the new rows' numbers: what is read here is checked after the wait)
+    int ar0 = p.app_row && tid < p.max_active ? p.app_row[(size_t)s * p.max_active + tid] : -1;
     const int A = p.n_active[s], nt = p.ntiles[s];
     if (A * p.group <= m0 || nt <= 0) {                    // nothing to do (all blocks of the cluster agree)
         if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -279,8 +294,8 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     Run r;
     r.tiles = p.tiles + (size_t)s * p.ntile_max;
     r.mask = p.mask + (size_t)s * p.max_active * p.W;
-    r.h0 = (int)((long long)rank * PARTS * nt / nblk);
-    r.h1 = (int)((long long)(rank + 1) * PARTS * nt / nblk);
+    r.h0 = run_begin(rank, nblk, PARTS * nt, PARTS * (p.P / FDC_TILE_ROWS));
+    r.h1 = run_begin(rank + 1, nblk, PARTS * nt, PARTS * (p.P / FDC_TILE_ROWS));
     r.p0 = PARTS * (p.P / FDC_TILE_ROWS);                      // the whole tiles of the prefix come first in a list
     if (r.p0 < r.h0) r.p0 = r.h0;
     if (r.p0 > r.h1) r.p0 = r.h1;
@@ -288,41 +303,69 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     if (r.np > MASK_WORDS / A) r.np = MASK_WORDS / A;
     if (r.np > MASK_HALVES) r.np = MASK_HALVES;
     const int chunks = M * (D / 16), slots = chunks_of_block(chunks, nblk);     // chunks of the result, of one block at most
-    // ---- set-up: barriers, the run's rows, the fields' visibility beyond the prefix
+    // ---- set-up: barriers, the prefix's first stages, the run's rows, the fields' visibility beyond the prefix
     r.nx = p.app_row && rank == 0 ? (A + SROWS - 1) / SROWS : 0;
-    if (tid == 0) {
-        bs.abort_flag = 0;
-        bs.first_beyond = r.h1 - r.h0;
-        for (int i = 0; i < nstage; ++i) {
-            bs.used[i] = 0;
-            bs.asked[i] = i < r.nx ? 1 : 0;
-            mbar_init(smem_u32(&bs.full[i]), 1);
-            if (Math::K_REUSED) mbar_init(smem_u32(&bs.k_read[i]), groups);
+    if (tid < nstage) {
+        bs.used[tid] = 0;
+        bs.asked[tid] = tid < r.nx ? 1 : 0;
+        mbar_init(smem_u32(&bs.full[tid]), 1);
+        if (Math::K_REUSED) mbar_init(smem_u32(&bs.k_read[tid]), groups);
+        if (tid == 0) {
+            bs.abort_flag = 0;
+            bs.first_beyond = r.h1 - r.h0;
+            mbar_init(smem_u32(&bs.pushed), 1);
         }
-        mbar_init(smem_u32(&bs.pushed), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
-        if (nblk > 1) mbar_expect_tx(smem_u32(&bs.pushed), nblk * ((chunks - rank + nblk - 1) / nblk) * CHUNK_BYTES);
-        for (int i = 0; i < r.nx; ++i) mbar_arrive(smem_u32(&bs.full[i]));      // filled by this block itself, ahead of the main loop
+        if (tid == 0 && nblk > 1) mbar_expect_tx(smem_u32(&bs.pushed), nblk * ((chunks - rank + nblk - 1) / nblk) * CHUNK_BYTES);
+        if (tid < r.nx) mbar_arrive(smem_u32(&bs.full[tid]));         // filled by this block itself, ahead of the main loop
     }
     if (tid < MASK_HALVES) bs.seen[tid] = 0u;
     if (tid < MAX_QROWS) bs.fld[tid] = tid < M ? (uint8_t)((m0 + tid) / p.group) : (uint8_t)0xff;
+    __syncthreads();
+    // (the barrier of the partials is there: the other blocks may send once they have seen this)
+    if (nblk > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    volatile int* abortp = &bs.abort_flag;
+    const uint32_t full0 = smem_u32(bs.full), ring0 = smem_u32(ring);
+    auto request_rows = [&](int row0, int st, int n) {     // one thread: the copies of a stage, the n-th to use slot st
+        const uint32_t bar = full0 + 8 * st, dst = ring0 + (uint32_t)st * STAGE_BYTES;
+        mbar_expect_tx(bar, STAGE_BYTES);
+#pragma unroll
+        for (int h = 0; h < STAGE_BYTES / (2 * SROWS * 128); ++h) {
+            tma_load_4d(dst + h * (SROWS * 128), &tm_k, bar, h * 8 * CHUNK, row0, g, s);
+            tma_load_4d(dst + STAGE_BYTES / 2 + h * (SROWS * 128), &tm_v, bar, h * 8 * CHUNK, row0, g, s);
+        }
+        __threadfence_block();
+        *(volatile int*)&bs.asked[st] = n;
+    };
+    // The first stages (warp w requests w, w + NW, ..): those of the prefix right away, so that they are on their way while
+    // the rest is set up; stages fb1.. may hold rows beyond the prefix and wait for the kernel ahead.
+    int fb1 = r.nx + r.p0 - r.h0;
+    if (!Math::PREFIX_FIRST) {                             // (any order of the list is served)
+        const int pos = r.h0 + lane;
+        const unsigned beyond = __ballot_sync(0xffffffffu, pos < r.p0 && r.tiles[pos / PARTS] * FDC_TILE_ROWS + pos % PARTS * SROWS + SROWS > p.P);
+        if (beyond) fb1 = r.nx + __ffs(beyond) - 1;
+    }
+    if (lane == 0)
+        for (int it = warp; it < nstage && it < fb1; it += NW)
+            if (it >= r.nx) {
+                const int pos = r.h0 + it - r.nx;
+                request_rows((Math::PREFIX_FIRST ? pos / PARTS : r.tiles[pos / PARTS]) * FDC_TILE_ROWS + pos % PARTS * SROWS, it, 1);
+            }
+    __syncwarp();
     bool off_list = false;
     int beyond = 0x7fffffff;                               // first part of this thread's that reaches beyond the prefix
     for (int i = tid; i < r.h1 - r.h0; i += THREADS) {
-        const int pos = r.h0 + i, row0 = r.tiles[pos / (FDC_TILE_ROWS / SROWS)] * FDC_TILE_ROWS + pos % (FDC_TILE_ROWS / SROWS) * SROWS;
+        const int pos = r.h0 + i, row0 = list_row0<SROWS>(r, pos);
         if (i < ROW0S) bs.row0[i] = row0;
         if (row0 + SROWS > p.P && beyond == 0x7fffffff) beyond = i;
         off_list |= pos < PARTS * (p.P / FDC_TILE_ROWS) && row0 != pos * SROWS;
     }
-    __syncthreads();
-    // (the barrier of the partials is there: the other blocks may send once they have seen this)
-    if (nblk > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     if (beyond != 0x7fffffff) atomicMin(&bs.first_beyond, beyond);
     auto cache_bits = [&]() {
         for (int i = tid; i < r.np * A; i += THREADS) {
             const int h = i / A, b = i - h * A;
-            const uint32_t x = part_bits<SROWS>(r.mask + (size_t)b * p.W, p.W, p.P, part_row0<SROWS>(r, bs, r.p0 + h));
+            const uint32_t x = part_bits<SROWS>(r.mask + (size_t)b * p.W, p.W, p.P, list_row0<SROWS>(r, r.p0 + h));
             bs.bits[i] = x;
             if (x) atomicOr(&bs.seen[h], x);
         }
@@ -345,8 +388,6 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             if (lane == 0) bs.newbits[x * FDC_MAX_NODES + b] = bits;
         }
     };
-    // (the launch may be ahead of whatever writes the row numbers: what is read here is checked after the wait)
-    int ar0 = p.app_row && tid < A ? p.app_row[(size_t)s * p.max_active + tid] : -1;
     if (tid < A) bs.app_row[tid] = ar0 >= p.P && ar0 < p.rows ? ar0 : -1;
     cache_bits();
     __syncthreads();
@@ -366,26 +407,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     r.total = r.nx + (r.h1 - r.h0) - (r.np - bs.n_kept);
     // stages fb.. may hold rows beyond the prefix (parts ahead of p0 are never left out)
     const int fb = r.nx + (bs.first_beyond < r.p0 - r.h0 ? bs.first_beyond : r.p0 - r.h0);
-    volatile int* abortp = &bs.abort_flag;
-    const uint32_t full0 = smem_u32(bs.full), ring0 = smem_u32(ring);
-    auto request = [&](int it, int st, int n) {            // one thread: the copies of stage `it`, the n-th to use slot st
-        const uint32_t bar = full0 + 8 * st, dst = ring0 + (uint32_t)st * STAGE_BYTES;
-        const int row0 = part_row0<SROWS>(r, bs, stage_pos(r, bs, it));
-        mbar_expect_tx(bar, STAGE_BYTES);
-#pragma unroll
-        for (int h = 0; h < STAGE_BYTES / (2 * SROWS * 128); ++h) {
-            tma_load_4d(dst + h * (SROWS * 128), &tm_k, bar, h * 8 * CHUNK, row0, g, s);
-            tma_load_4d(dst + STAGE_BYTES / 2 + h * (SROWS * 128), &tm_v, bar, h * 8 * CHUNK, row0, g, s);
-        }
-        __threadfence_block();
-        *(volatile int*)&bs.asked[st] = n;
-    };
-    // the first stages: warp w requests w and w + 8; those of the prefix ahead of the dependency wait
-    if (lane == 0) {
-        for (int it = warp; it < nstage && it < fb; it += NW)
-            if (it >= r.nx) request(it, it, 1);
-    }
-    __syncwarp();
+    auto request = [&](int it, int st, int n) { request_rows(part_row0<SROWS>(r, bs, stage_pos(r, bs, it)), st, n); };
     if (p.early) {
         // The queries and the new rows may still be written by the kernel ahead: their lines are only requested into L2
         // (which stays coherent), so that the reads after the wait find them there.
@@ -403,7 +425,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     }
     if (lane == 0) {
         for (int it = warp; it < nstage && it < r.total; it += NW)
-            if (it >= fb) request(it, it, 1);
+            if (it >= fb1) request(it, it, 1);
     }
     __syncwarp();
     // queries of the pair: row m = field * group + head-in-group; rows M.. up to a whole group are zero
@@ -525,7 +547,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     }
     // ---- the warps' results meet in shared memory (the ring is free: every stage has been consumed)
     __syncthreads();
-    if (left > 0) math.write(part + warp * (GROWS * D), bs.wml + warp * GROWS);
+    if (left > 0) math.write(part + warp * (GROWS * D), bs.wml + warp * GROWS, left);
     __syncthreads();
     auto store_out = [&](int mm, int c4, const float4& acc, float lt) {
         const float inv = 1.f / lt;
