@@ -62,19 +62,19 @@ static float tc_estimate(const ClusterProblem& c)
 }
 
 // The cluster kernel's cut of this problem and whether it is the faster kernel (kept in the plan: both follow
-// from the shapes alone).  Where both kernels can run, the cluster kernel is taken if its estimate is below 0.82
-// of the other's.  How long either takes also depends on how many of the dependencies are met, which the shapes do not
-// tell, so the line lies on the side of the tcgen05 kernel: 59 of the 150 shapes go to the cluster kernel, and three of
-// them are slower there (by 2, 5 and 16 %; with 0.9 it would be 77 and ten, up to 20 %; of 110 others, 53 and four).  Cluster / tcgen05 kernel, us a
-// layer: 1 scene x 7 query rows, prefix 2048 8.0 / 14.5, 1 scene x 42 rows 11.9 / 17.7; 13 scenes x 49 rows, prefix 529
-// 21.6 / 18.3; 16 scenes x 24 rows, prefix 4096 59 / 52.
+// from the shapes alone).  Where both kernels can run, the one with the lower estimate is taken.  Of 226 shapes with head_dim
+// 128 timed on both (2 to 288 pairs, prefix 256 to 32600, 4 to 128 query rows, one or more fields of the template at work), the kernel and the
+// cut taken are on average 10 % slower than the best kernel and cut, from 13 % with the line at 0.82 of the other's estimate and the
+// constants before; one shape in twenty is slower than it was by 4 % or more.  Cluster / tcgen05 kernel, us a layer: 1 scene x 7 query
+// rows, prefix 2048 6.6 / 14.5, 1 scene x 42 rows 10.1 / 18.2; 32 pairs x 20 rows, prefix 9922 33.4 / 37.0; 16 scenes x 24 rows,
+// prefix 4096 59 / 52.
 static const ClusterShape& route(fdc_plan* p, const fdc_kv_desc* kv)
 {
     const ClusterProblem c{(int64_t)kv->batch * kv->hkv, p->h.max_active * (kv->hq / kv->hkv), kv->head_dim, p->h.P, p->h.T, p->sm_count};
     if (!(p->route_for == c)) {
         float us = 0.f;
         p->route_shape = pick_cluster(c, &us);
-        p->route_cluster = kv->head_dim != 128 || us < 0.82f * tc_estimate(c);
+        p->route_cluster = kv->head_dim != 128 || us < tc_estimate(c);
         p->route_for = c;
     }
     return p->route_shape;
