@@ -243,7 +243,6 @@ int fdc_decode_attn(fdc_plan* p, const fdc_kv_desc* kv, int32_t layer, const int
     a.pair_cnt = nullptr;
     a.split_memo = nullptr;
     a.seq = 0;
-    a.paired = 0;
     bool fused = false;                 // the kernel merged the partials itself
     // Reading ahead of the dependency wait: allowed from the second attention launch of a pass on
     // the same stream.  The first one waits for everything before it (the pass tables, the split)
@@ -259,11 +258,6 @@ int fdc_decode_attn(fdc_plan* p, const fdc_kv_desc* kv, int32_t layer, const int
         if (!takes_cluster_kernel(p, kv)) {
             if ((long long)kv->batch * kv->hkv <= FDC_PAIR_COUNTERS) a.pair_cnt = p->d_pair_cnt;
             a.split_memo = (a.pair_cnt && kv->batch <= FDC_MEMO_BATCH && a.n_cta <= FDC_MEMO_CTAS) ? p->d_split_memo : nullptr;
-            // Clusters of two where the split cuts every pair in two (there is a second CTA for each pair, but no third) and a CTA's run
-            // is at most 64 tiles: what the exchange saves is a few us of a launch, and from 100 (200) tiles the split may
-            // take equal shares, whose parts are not two to a cluster.
-            const long long pairs = (long long)kv->batch * kv->hkv;
-            a.paired = a.pair_cnt && 2 * pairs <= a.n_cta && 3 * pairs > a.n_cta && !(a.n_cta & 1) && pairs * a.ntile_max <= 64ll * a.n_cta;
             // The work split depends only on the pass tables, so it is computed once per pass, by a launch
             // of its own ahead of the pass's first attention launch (an ordinary launch: it begins after
             // everything before it in the stream has completed).

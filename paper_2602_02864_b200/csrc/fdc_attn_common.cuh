@@ -143,37 +143,4 @@ __device__ __forceinline__ Segment decode_segment(long long u, long long hi, con
 // boxes of 128 bytes x box_rows rows and 128-byte swizzle.  out_map points to a CUtensorMap.
 int get_kv_tensor_map(const void* base, const AttnParams& p, int dtype, int head_dim, int box_rows, void* out_map);
 
-// ---- between the blocks of a cluster
-__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank)
-{
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-// Asynchronous stores into a block of the cluster; the bytes count towards `bar`, a barrier of the same block.
-__device__ __forceinline__ void st_async4(uint32_t addr, uint32_t bar, const float4& v)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, const float2& v)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void st_async1(uint32_t addr, uint32_t bar, float v)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(addr), "f"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-// The wait for what the other blocks send.  A block that gives up elsewhere still sends what it has, after a second or so; the limit here is
-// several times that, so that nobody leaves while bytes for it are under way.
-static __device__ __noinline__ bool wait_pushed_slow(uint32_t bar, volatile int* abort_flag, int32_t* status)
-{
-    for (uint32_t i = 0; i < SPIN_LIMIT * 8; ++i)
-        if (mbar_try(bar, 0)) return true;
-    *abort_flag = 1;
-    atomicOr(status, FDC_DEV_TIMEOUT);
-    return false;
-}
-
 }  // namespace fdc

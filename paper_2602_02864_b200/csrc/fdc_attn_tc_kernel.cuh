@@ -124,7 +124,6 @@ struct __align__(8) CtaFlags {
     uint64_t raise_bar;              // mbarrier of the reference-raising path (raise_sync)
     int abort_flag;                  // a bounded wait ran out somewhere in the CTA
     int v_steps[4];
-    PeerArgs peer;
 };
 constexpr uint32_t RAISE_BAR_BEFORE_ABORT_FLAG = 8;
 static_assert(offsetof(CtaFlags, abort_flag) - offsetof(CtaFlags, raise_bar) == RAISE_BAR_BEFORE_ABORT_FLAG, "layout");
@@ -144,7 +143,6 @@ struct Ctx : Split {
     __device__ __forceinline__ uint32_t q_ready() const { return bar0 + 32 * MAXST + 96; }
     __device__ __forceinline__ uint32_t o_free() const { return bar0 + 32 * MAXST + 104; }
     __device__ __forceinline__ uint32_t app_done() const { return bar0 + 32 * MAXST + 112; }
-    __device__ __forceinline__ uint32_t peer_sent() const { return bar0 + 32 * MAXST + 120; }
     int ns, s_stride;                // S^T buffers in TMEM (4 of 64 columns) and their distance
     uint32_t tmem;
     unsigned char *kring, *vring, *qs, *ps, *ones;
@@ -156,7 +154,6 @@ struct Ctx : Split {
     uint64_t* sunion;                // [2][UW] their OR over the scene's active branches (when mstaged and W <= UW)
     int mstaged;
     volatile int* abortp;
-    PeerArgs* peer;
     volatile int* v_steps;           // [2][2] per P^T buffer and tile of the round: the 16-row steps to multiply (bit k: rows 16k..)
     int nk, nv, q_panel, p_buf, npb; // ring depths, bytes per 64-column panel of Q^T, bytes per P^T buffer, P^T buffers (2)
 };
@@ -599,81 +596,6 @@ __device__ __noinline__ int raise_references(const RaiseArgs a)
     return dead ? 1 : 0;
 }
 
-// A pair that is cut in two, its parts in the two CTAs of a cluster: each CTA finishes half of the (padded) query rows.  What
-// the other CTA finishes is sent into its K ring, whose stages have all been consumed, as asynchronous stores that it waits
-// for (all softmax threads; thread = head_dim index x the columns of its part).  It replaces the partial written to the workspace, a counter
-// in L2 and the merge by whoever comes second.  Measured, 8 scenes x 8 KV heads, 64 query rows, prefix 8192, us a layer: 59.0 / 56.5.
-constexpr int PEER_ML = (NP_MAX / 2) * D * 4;    // [query row][D] sums, then [query row] (reference, sum)
-static_assert(PEER_ML + NP_MAX * 4 <= 2 * STAGE, "room in the K ring");
-__device__ __noinline__ void merge_with_peer(const PeerArgs* pa, const float* mneg, float* alpha, float* lred, const bool dead)
-{
-    const PeerArgs a = *pa;
-    const int part = threadIdx.x >> 7, krow = threadIdx.x & 127;
-    const uint32_t peer = (blockIdx.x & 1u) ^ 1u;
-    const int tid = threadIdx.x, H = a.np / 2, own0 = peer ? 0 : H, peer0 = peer ? H : 0;
-    const int rows = a.M - own0 < 0 ? 0 : (a.M - own0 < H ? a.M - own0 : H);
-    if (tid == 0) mbar_expect_tx(a.sent, (uint32_t)rows * (D * 4 + 8));
-    cluster_arrive();                              // this CTA's ring is free, its barrier is set
-    cluster_wait();
-    __syncwarp();
-    float m = -INFINITY, lt = 0.f;
-    if (tid < a.M) {
-        lt = (lred[tid] + lred[128 + tid]) + (lred[256 + tid] + lred[384 + tid]);
-        if (mneg[tid] != UNSET) m = -mneg[tid];
-    }
-    const uint32_t to = map_rank(a.buf, peer), bar = map_rank(a.sent, peer);
-    if (tid < a.M && tid >= peer0 && tid < peer0 + H) st_async2(to + PEER_ML + (uint32_t)(tid - peer0) * 8, bar, make_float2(m, lt));
-    const bool own = (uint32_t)(part >> 1) != peer;          // the columns of parts 0, 1 are the first half
-    const int nch = a.np >> 5, col0 = part * (a.np >> 2);
-    const uint32_t o_addr = a.tmem + ((uint32_t)(krow & ~31) << 16) + TM_O + col0;
-    if (!own) {
-#pragma unroll 1
-        for (int ch = 0; ch < nch; ++ch) {
-            uint32_t ov[8];
-            tmem_ld<8>(o_addr + ch * 8, ov);
-            tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int n = col0 + ch * 8 + i;
-                if (n < a.M) st_async1(to + (uint32_t)((n - peer0) * D + krow) * 4, bar, dead ? 0.f : __uint_as_float(ov[i]));
-            }
-        }
-    }
-    if (!mbar_try(a.sent, 0)) wait_pushed_slow(a.sent, a.abortp, a.status);
-    __syncwarp();
-    if (tid < a.M && tid >= own0 && tid < own0 + H) {
-        float pm, pl;
-        asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(pm), "=f"(pl) : "r"(a.buf + PEER_ML + (uint32_t)(tid - own0) * 8) : "memory");
-        const float nm = fmaxf(m, pm), ms = nm == -INFINITY ? 0.f : nm;
-        const float w0 = fast_exp2(m - ms), w1 = fast_exp2(pm - ms), inv = 1.f / (lt * w0 + pl * w1);
-        alpha[tid] = w0 * inv;
-        lred[tid] = w1 * inv;                    // (read by this thread alone before)
-    }
-    soft_sync();
-    if (own && !dead) {
-#pragma unroll 1
-        for (int ch = 0; ch < nch; ++ch) {
-            uint32_t ov[8];
-            tmem_ld<8>(o_addr + ch * 8, ov);
-            tmem_wait_ld();
-            int b = (col0 + ch * 8) / a.G, hg = (col0 + ch * 8) - b * a.G;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int n = col0 + ch * 8 + i;
-                if (n < a.M) {
-                    float o;
-                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o) : "r"(a.buf + (uint32_t)((n - own0) * D + krow) * 4) : "memory");
-                    a.out[((size_t)b * a.hq + hg) * D + krow] = __float2bfloat16_rn(__uint_as_float(ov[i]) * alpha[n] + o * lred[n]);
-                }
-                if (++hg == a.G) {
-                    hg = 0;
-                    ++b;
-                }
-            }
-        }
-    }
-}
-
 // The softmax warps' work on one segment; nphj = a quarter of the pair's padded query columns NP (8,
 // 16 or 32).  Columns are handled eight at a time in real loops with the references read from
 // shared memory, so that the same small loop serves every width.
@@ -989,14 +911,10 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, const Ctx& 
     } else {
         cx.lred[part * 128 + krow] = 0.f;
     }
-    const bool whole = sg.j0 == 0 && sg.j1 == sg.nt;       // this CTA saw every tile of the pair
-    const bool both = !whole && parts_in_cluster(p, cx, sg.s, sg.g);         // the other part is in the cluster's other CTA
-    if (both && tid == 0)
-        *cx.peer = PeerArgs{cx.peer_sent(), smem_u32(cx.kring), cx.tmem, M, np, G, p.hq,
-                            reinterpret_cast<__nv_bfloat16*>(p.out) + ((size_t)sg.s * p.max_active * p.hq + (size_t)sg.g * G) * D, cx.abortp, p.status};
     soft_sync();
     const int pair = sg.s * p.hkv + sg.g;
     const int slot = blockIdx.x + pair;
+    const bool whole = sg.j0 == 0 && sg.j1 == sg.nt;       // this CTA saw every tile of the pair
     if (p.pair_cnt && whole) {
         // no other partial exists: normalise and write the output directly
         if (tid < np) cx.alpha[tid] = 1.f / ((cx.lred[tid] + cx.lred[128 + tid]) + (cx.lred[256 + tid] + cx.lred[384 + tid]));
@@ -1022,8 +940,6 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, const Ctx& 
                 }
             }
         }
-    } else if (both) {
-        merge_with_peer(cx.peer, cx.mneg, cx.alpha, cx.lred, dead);
     } else {
         if (!dead) {
             if (tid < M) {
@@ -1111,7 +1027,6 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
     __shared__ CtaFlags cta_flags;
     cx.abortp = &cta_flags.abort_flag;
     cx.v_steps = cta_flags.v_steps;
-    cx.peer = &cta_flags.peer;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -1143,7 +1058,6 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
         mbar_init(cx.q_ready(), NSOFT);
         mbar_init(cx.o_free(), NSOFT);
         mbar_init(cx.app_done(), 1);
-        mbar_init(cx.peer_sent(), 1);
         mbar_init(smem_u32(&cta_flags.raise_bar), NSOFT);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
@@ -1209,7 +1123,6 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
             u = sg.next_u;
         }
     }
-    if (p.paired && active && warp >= NSOFT) cluster_arrive();         // (the softmax warps of both CTAs meet there, see merge_with_peer)
     // ---- teardown: everybody is done with TMEM before it is freed
     tc_fence_before();
     __syncthreads();
@@ -1262,9 +1175,11 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
         cfg.blockDim = dim3(THREADS);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
-        cudaLaunchAttribute at[2];
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
-        cfg.numAttrs = tc_launch_attrs(at, p, split_only);
+        cfg.numAttrs = split_only ? 0 : 1;
         cudaError_t e = cudaLaunchKernelEx(&cfg, FDC_TC_KERNEL, p, tk, tv, nk, nv, split_only);
         if (e != cudaSuccess) return set_cuda_error(e);
     }

@@ -65,7 +65,6 @@ struct CtaFlags {
     int abort_flag;                  // a bounded wait ran out somewhere in the CTA
     int v_steps[NBAR];
     int merge[3];                    // last arriver of the pair, first and last CTA of the pair
-    PeerArgs peer;
 };
 
 // Everything a role needs to find its barriers and buffers.
@@ -82,12 +81,10 @@ struct Ctx : Split {
     __device__ __forceinline__ uint32_t q_ready() const { return bar0 + 32 * MAXST + 24 * NBAR; }
     __device__ __forceinline__ uint32_t o_free() const { return bar0 + 32 * MAXST + 24 * NBAR + 8; }
     __device__ __forceinline__ uint32_t app_done() const { return bar0 + 32 * MAXST + 24 * NBAR + 16; }
-    __device__ __forceinline__ uint32_t peer_sent() const { return bar0 + 32 * MAXST + 24 * NBAR + 24; }
     uint32_t tmem;
     unsigned char *kring, *vring;
     float2* ml;                      // [2][128] (reference, sum) of each group's rows at the end of a segment
     int* merge;
-    PeerArgs* peer;
     uint64_t* smask;                 // [2][mbuf] the current segment's scene bitmaps (when mstaged)
     int mbuf;                        // words per buffer
     uint64_t* sunion;                // [2][UW] their OR over the scene's active branches (when mstaged and W <= UW)
@@ -321,82 +318,6 @@ __device__ __noinline__ void merge_pair(const float* ws_ml, const float* ws_o, _
                     make_uint4(pack2(acc[i][0] * inv, acc[i][1] * inv), pack2(acc[i][2] * inv, acc[i][3] * inv), pack2(acc[i][4] * inv, acc[i][5] * inv),
                                pack2(acc[i][6] * inv, acc[i][7] * inv));
             }
-        }
-    }
-}
-
-// A pair that is cut in two, its parts in the two CTAs of a cluster: each CTA finishes half of the columns.  What the other
-// CTA finishes is sent into its K ring, whose stages have all been consumed, as asynchronous stores that it waits for
-// (all softmax threads; thread = query row x 32 columns of either half).
-// It replaces the partial written to the workspace, a counter in L2 and the merge by whoever comes second.  Measured, 8 scenes x 8 KV heads, 128 query
-// rows, prefix 1024, us a layer through the workspace / inside the cluster: 39.2 / 34.3.
-constexpr int PEER_ML = (D / 2) * MROWS * 4;       // [D / 8 chunks of 4 columns][row] sums, then [row] (reference, sum)
-static_assert(PEER_ML + MROWS * 8 <= 3 * STAGE, "room in the K ring");
-__device__ __noinline__ void merge_with_peer(const PeerArgs* pa, const float2* ml, const int* holds, const bool dead)
-{
-    const PeerArgs ar = *pa;
-    const int row = threadIdx.x & 127, grp = threadIdx.x >> 7, M = ar.M;
-    const uint32_t sent = ar.sent, buf = ar.buf, o_addr = ar.tmem + ((uint32_t)(row & ~31) << 16) + TM_O;
-    // the two groups' results of the row
-    const float2 a0 = ml[row], a1 = ml[MROWS + row];
-    const bool has0 = holds[0] != 0, has1 = holds[1] != 0;
-    const float mx = fmaxf(a0.x, a1.x), mf = mx == -INFINITY ? 0.f : mx;
-    const float f0 = fast_exp2(a0.x - mf), f1 = fast_exp2(a1.x - mf), lt = a0.y * f0 + a1.y * f1;
-    const uint32_t rank = blockIdx.x & 1u, peer = rank ^ 1u;
-    if (threadIdx.x == 0) mbar_expect_tx(sent, (uint32_t)M * (D / 2 * 4 + 8));
-    cluster_arrive();                              // this CTA's ring is free, its barrier is set
-    cluster_wait();
-    __syncwarp();
-    const bool here = (row & ~31) < M;             // (uniform over the warp)
-    auto half = [&](uint32_t side, int h, float (&v)[16]) {
-        const uint32_t c0 = side * (D / 2) + (uint32_t)(grp * 32 + h * 16);
-        uint32_t x[16], y[16];
-        const bool b0 = has0 && !dead, b1 = has1 && !dead;
-        tmem_ld<16>(o_addr + c0, x);
-        tmem_ld<16>(o_addr + 128 + c0, y);
-        tmem_wait_ld();
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = (b0 ? __uint_as_float(x[i]) * f0 : 0.f) + (b1 ? __uint_as_float(y[i]) * f1 : 0.f);
-    };
-    if (here) {
-        const uint32_t to = map_rank(buf, peer), bar = map_rank(sent, peer);
-        if (grp == 0 && row < M) st_async2(to + PEER_ML + row * 8, bar, make_float2(mx, lt));
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            float v[16];
-            half(peer, h, v);
-            if (row < M) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    st_async4(to + (uint32_t)(((grp * 8 + h * 4 + i) * MROWS + row) * 16), bar, make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]));
-            }
-        }
-    }
-    if (!mbar_try(sent, 0)) wait_pushed_slow(sent, ar.abortp, ar.status);
-    __syncwarp();
-    if (!here) return;
-    float pm, pl;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(pm), "=f"(pl) : "r"(buf + PEER_ML + (uint32_t)row * 8) : "memory");
-    const float nm = fmaxf(mx, pm), ms = nm == -INFINITY ? 0.f : nm;
-    const float w0 = fast_exp2(mx - ms), w1 = fast_exp2(pm - ms), inv = 1.f / (lt * w0 + pl * w1), a = w0 * inv, b = w1 * inv;
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        float v[16];
-        half(rank, h, v);
-        if (row < M) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                float4 o;
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.x), "=f"(o.y), "=f"(o.z), "=f"(o.w) : "r"(buf + (uint32_t)(((grp * 8 + h * 4 + i) * MROWS + row) * 16)) : "memory");
-                v[4 * i] = v[4 * i] * a + o.x * b;
-                v[4 * i + 1] = v[4 * i + 1] * a + o.y * b;
-                v[4 * i + 2] = v[4 * i + 2] * a + o.z * b;
-                v[4 * i + 3] = v[4 * i + 3] * a + o.w * b;
-            }
-            __nv_bfloat16* to = ar.out + ((size_t)(row / ar.G) * ar.hq + row % ar.G) * D + rank * (D / 2) + grp * 32 + h * 16;
-#pragma unroll
-            for (int i = 0; i < 16; i += 8)
-                *reinterpret_cast<uint4*>(to + i) = make_uint4(pack2(v[i], v[i + 1]), pack2(v[i + 2], v[i + 3]), pack2(v[i + 4], v[i + 5]), pack2(v[i + 6], v[i + 7]));
         }
     }
 }
@@ -743,11 +664,6 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, const Ctx& cx,
         // ---- end of segment: the two groups' results of a row are one row's result
         if (any_tile) wait_u(cx.pv_done() + 8 * (last % NBAR), (last / NBAR) & 1);
         tc_fence_after();
-        const bool whole = sg.j0 == 0 && sg.j1 == sg.nt;   // this CTA saw every tile of the pair
-        const bool both = !whole && parts_in_cluster(p, cx, sg.s, sg.g);       // the pair's other part is in the cluster's other CTA
-        if (both && tid == 0)
-            *cx.peer = PeerArgs{cx.peer_sent(), smem_u32(cx.kring), cx.tmem, M, MROWS, G, p.hq,
-                                reinterpret_cast<__nv_bfloat16*>(p.out) + ((size_t)sg.s * p.max_active * p.hq + (size_t)sg.g * G) * D, cx.abortp, p.status};
         cx.ml[grp * MROWS + row] = make_float2(begun ? m : -INFINITY, l);
         if (lane == 0 && q4 == 0) cx.merge[grp] = begun;
         soft_sync();
@@ -755,12 +671,12 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, const Ctx& cx,
         const bool has0 = cx.merge[0] != 0, has1 = cx.merge[1] != 0;
         const float mx = fmaxf(a0.x, a1.x), ms = mx == -INFINITY ? 0.f : mx;
         const float f0 = fast_exp2(a0.x - ms), f1 = fast_exp2(a1.x - ms), lt = a0.y * f0 + a1.y * f1;
+        soft_sync();                               // (merge[] is used again below)
         const int pair = sg.s * p.hkv + sg.g;
         const int slot = blockIdx.x + pair;
+        const bool whole = sg.j0 == 0 && sg.j1 == sg.nt;   // this CTA saw every tile of the pair
         const bool direct = p.pair_cnt && whole;           // no other partial exists: normalise and write the output
-        if (both) {
-            merge_with_peer(cx.peer, cx.ml, cx.merge, dead);
-        } else if (rows_here && !dead) {
+        if (rows_here && !dead) {
             const float inv = direct ? 1.f / lt : 1.f, g0 = f0 * inv, g1 = f1 * inv;
             const int b = row / G, hg = row - b * G;
             __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (((size_t)sg.s * p.max_active + b) * p.hq + (size_t)sg.g * G + hg) * D;
@@ -791,9 +707,9 @@ __device__ __forceinline__ void softmax_loop(const AttnParams& p, const Ctx& cx,
             }
             if (!direct && grp == 0 && row < M) *reinterpret_cast<float2*>(p.ws_ml + ((size_t)slot * p.mmax + row) * 2) = make_float2(mx, lt);
         }
-        if (p.pair_cnt && !whole && !both) {
+        if (p.pair_cnt && !whole) {
             // the CTA that delivers the last partial of a pair merges them all (no second kernel)
-            soft_sync();                           // (and merge[] is used again)
+            soft_sync();
             if (tid == 0) {
                 __threadfence();                   // (everybody's stores: they came before the barrier)
                 int c_first, c_last;
@@ -844,7 +760,6 @@ attn_tc_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k
     cx.abortp = &cta_flags.abort_flag;
     cx.v_steps = cta_flags.v_steps;
     cx.merge = cta_flags.merge;
-    cx.peer = &cta_flags.peer;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -868,7 +783,6 @@ attn_tc_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k
         mbar_init(cx.q_ready(), NSOFT / 2);
         mbar_init(cx.o_free(), NSOFT);
         mbar_init(cx.app_done(), 1);
-        mbar_init(cx.peer_sent(), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
@@ -917,7 +831,6 @@ attn_tc_rows_kernel(const AttnParams p, const __grid_constant__ CUtensorMap tm_k
     } else {
         softmax_loop(p, cx, lo, hi, warp, lane);
     }
-    if (p.paired && active && warp >= NSOFT) cluster_arrive();         // (the softmax warps of both CTAs meet there, see merge_with_peer)
     // ---- teardown: everybody is done with TMEM before it is freed
     tc_fence_before();
     __syncthreads();
@@ -964,9 +877,11 @@ int launch_tc_rows(const AttnParams& p, int head_dim, cudaStream_t st, int split
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[2];
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = tc_launch_attrs(at, p, split_only);
+    cfg.numAttrs = split_only ? 0 : 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, attn_tc_rows_kernel, p, tk, tv, nk, nv, split_only);
     if (e != cudaSuccess) return set_cuda_error(e);
     note_launch();

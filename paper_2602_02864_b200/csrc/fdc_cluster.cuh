@@ -177,10 +177,35 @@ __device__ __noinline__ uint32_t new_rows_of(const int* app_row, int A, int row0
     return __reduce_or_sync(0xffffffffu, x);
 }
 
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank)
+{
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Asynchronous stores into a block of the cluster; the bytes count towards `bar`, a barrier of the same block.
+__device__ __forceinline__ void st_async4(uint32_t addr, uint32_t bar, const float4& v)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, const float2& v)
+{
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
+}
 // Where the partials of a block's chunks arrive: [block of the cluster][chunk][16 columns], then [block][chunk] (m, l).
 // Chunk k (query row k / (D / 16), columns 16 (k mod D / 16) ..) belongs to block k mod nblk and is its (k / nblk)-th.
 constexpr int CHUNK_BYTES = 16 * 4 + 8;
 __host__ __device__ __forceinline__ int chunks_of_block(int chunks, int nblk) { return (chunks + nblk - 1) / nblk; }
+// The wait for them.  A block that gives up elsewhere still sends what it has, after a second or so; the limit here is
+// several times that, so that nobody leaves while bytes for it are under way.
+static __device__ __noinline__ bool wait_pushed_slow(uint32_t bar, volatile int* abort_flag, int32_t* status)
+{
+    for (uint32_t i = 0; i < SPIN_LIMIT * 8; ++i)
+        if (mbar_try(bar, 0)) return true;
+    *abort_flag = 1;
+    atomicOr(status, FDC_DEV_TIMEOUT);
+    return false;
+}
 // Merge over the lanes of a block, for every (query row, 4 columns): `rows` = query rows of a lane's partial;
 // `done(row, column, m, l, sum)` takes the result.  (The weights of the merges, fp32's too, are ex2.approx.ftz: two
 // units in the last place like exp2f, but a part whose maximum lies more than 2^126 below the highest counts 0.)

@@ -140,7 +140,6 @@ struct AttnParams {
     int32_t*        pair_cnt;        // per (scene, KV head) arrival counters: the split kernel also combines (nullptr: it does not)
     int32_t*        split_memo;      // [FDC_MEMO_INTS] (nullptr: the work split is always computed)
     uint32_t        seq;             // number of the split launch the memo must come from
-    int32_t         paired;          // launched as clusters of two CTAs: the two parts of a pair that is cut in two meet inside one (tcgen05 kernels)
     int32_t         early;           // the pass tables, the memo and the prefix rows were complete before the kernel
                                      // preceding this one in the stream began: they may be read ahead of the dependency wait
     ClusterShape    cluster;         // cut of the launch (cluster kernel)

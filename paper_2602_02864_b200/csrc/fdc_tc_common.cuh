@@ -109,14 +109,6 @@ __device__ __forceinline__ void cp_async_wait_all()
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
 }
 
-// What merge_with_peer needs of its CTA: in shared memory, so that the call costs the softmax loop no registers.
-struct PeerArgs {
-    uint32_t sent, buf, tmem;        // barrier of the bytes the other CTA sends, where they go (the K ring), TMEM base
-    int M, np, G, hq;                // the pair's query rows (np: padded)
-    __nv_bfloat16* out;              // its first query row
-    volatile int* abortp;
-    int32_t* status;
-};
 // A CTA's view of the pass and of the work split.
 struct Split {
     int *pre, *nact;                 // [batch + 1] tile prefix sums, [batch] active branches per scene
@@ -178,13 +170,6 @@ __device__ __forceinline__ void pair_ctas(const AttnParams& p, const Split& cx, 
         c_first = (int)((v0 * cx.n_cta) / cx.vtot);
         c_last = (int)(((v0 + vt_of(cx, nt, nt - 1)) * cx.n_cta) / cx.vtot);
     }
-}
-
-// Whether pair (s, g), cut in two, has its two parts in the two CTAs of one cluster.
-__device__ __forceinline__ bool parts_in_cluster(const AttnParams& p, const Split& cx, int s, int g)
-{
-    if (!p.paired || !cx.tpart || cx.prev[s + 1] - cx.prev[s] != 2) return false;
-    return ((cx.prev[s] * p.hkv) & 1) == 0;                // (its first part is CTA prev[s] hkv + 2 g)
 }
 
 // The CTA's run of units.
@@ -645,19 +630,6 @@ __device__ __noinline__ uint64_t tile_seen_rows(const uint64_t* un, const uint64
     const uint32_t ul = __reduce_or_sync(0xffffffffu, (uint32_t)um);
     const uint32_t uh = __reduce_or_sync(0xffffffffu, (uint32_t)(um >> 32));
     return ((uint64_t)uh << 32) | ul;
-}
-
-// Attributes of a launch: dependent on the kernel ahead, and clusters of two where pairs are cut in two.
-inline unsigned tc_launch_attrs(cudaLaunchAttribute (&at)[2], const AttnParams& p, int split_only)
-{
-    if (split_only) return 0;
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = 2;
-    at[1].val.clusterDim.y = 1;
-    at[1].val.clusterDim.z = 1;
-    return p.paired ? 2 : 1;
 }
 
 }  // namespace
