@@ -13,7 +13,7 @@
 // Measured (us a layer, 32/8 heads x 128, prefix 2000):  8 warps x 32-row stages x 24 query rows 94 at 8 scenes with
 // six fields, 12 warps in two groups on 32-row stages 83, on 16-row stages 86; eight fields at 4 scenes 100 / 70 / 66;
 // three fields at 8 scenes 66 / 85 / 63.  The kernel that ran before (one warp per query row) took 955 in the first.
-// That holds up to 16 query rows (two groups of warps share a stage only above 8).  With 17 to 32 the two groups read every K and V row twice,
+// Up to 16 query rows one group of 12 warps does (tiles of 2 and 4).  With 17 to 32, two groups would read every K and V row twice,
 // and the port (14 cycles for 6 of FMAs in the scores, 18 for 12 in the result) is what they wait for; one group of 8 warps with tiles of
 // 6 or 8 query rows a lane (20 for 12, 20 for 24) takes 75 instead of 85 us a layer at 8 scenes with six fields, and 71 with runs cut evenly and the scores'
 // operands read a step ahead.
