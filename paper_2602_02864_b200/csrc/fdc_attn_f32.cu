@@ -253,7 +253,9 @@ int launch_d(const AttnParams& p, const ClusterShape& h, int ql, cudaStream_t st
         case 2: return launch_cluster<MathF32<D, 2, 12, 2>>(attn_f32_kernel<D, 2, 12, 2>, p, room, h, st);
         case 4: return launch_cluster<MathF32<D, 4, 12, 2>>(attn_f32_kernel<D, 4, 12, 2>, p, room, h, st);
         case 6: return launch_cluster<MathF32<D, 6, 8, 1>>(attn_f32_kernel<D, 6, 8, 1>, p, room, h, st);
-        default: return launch_cluster<MathF32<D, 8, 8, 1>>(attn_f32_kernel<D, 8, 8, 1>, p, room, h, st);
+        default:
+            if constexpr (D == 64) return launch_cluster<MathF32<D, 8, 8, 1>>(attn_f32_kernel<D, 8, 8, 1>, p, room, h, st);
+            return FDC_ERR_SHAPE;
     }
 }
 
@@ -268,7 +270,8 @@ namespace fdc {
 int launch_attn_f32(const AttnParams& p, int head_dim, cudaStream_t st)
 {
     ClusterShape h{1, (p.mmax + 31) / 32, 1};
-    const int per = (p.mmax + h.qsplit - 1) / h.qsplit, ql = per <= 8 ? 2 : (per <= 16 ? 4 : (per <= 24 ? 6 : 8));
+    const int per = (p.mmax + h.qsplit - 1) / h.qsplit;
+    const int ql = per <= 8 ? 2 : (per <= 16 ? 4 : (per <= 24 ? 6 : (head_dim == 64 && h.qsplit > 1 ? 8 : 4)));
     if (ql == 6) h.qsplit = (p.mmax + 23) / 24;
     const long long clusters = (long long)p.batch * p.hkv * h.qsplit;
     static const int sizes[] = {2, 3, 4, 6, 8}, holds[] = {74, 45, 33, 22, 15};
