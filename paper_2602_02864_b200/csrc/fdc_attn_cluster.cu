@@ -187,7 +187,7 @@ struct MathBf16 {
     {
         *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
     }
-    __device__ __forceinline__ MathBf16(const AttnParams& p, const unsigned char* qs, int qrows, int q0, int ln)
+    __device__ __forceinline__ MathBf16(const AttnParams& p, const unsigned char* qs, int qrows, int q0, int ln, int)
         : c(p.scale_log2), lane(ln), qpanel((uint32_t)qrows * 128), q_lane(smem_u32(qs) + (uint32_t)q0 * 128 + swz((uint32_t)qrows * 128, ln & 15, ln >> 4)),
           k_lane(swz(SROWS * 128, ln & 7, ln >> 3)), v_lane(STAGE_BYTES / 2 + swz(SROWS * 128, (ln & 7) + ((ln >> 3) & 1) * 8, ln >> 4))
     {

@@ -38,13 +38,14 @@ struct MathF32 {
     const float scale;
     const int qg, rg;
     const uint32_t q_lane, p_off;                          // p_off: place of the group's weights in the stage
+    const bool few;                                        // at most half of the group's rows exist: half tiles serve them
 
     static __host__ __device__ __forceinline__ size_t q_bytes(int qrows) { return (size_t)qrows * QROW; }
     static __device__ __forceinline__ uint32_t q_off(int, int m, int dc) { return (uint32_t)(m * QROW + dc * 16); }
     static __device__ __forceinline__ int part_off(int row, int col) { return row * D + col; }
     static __device__ __forceinline__ void store(float* out, const float4& x) { *reinterpret_cast<float4*>(out) = x; }
-    __device__ __forceinline__ MathF32(const AttnParams& p, const unsigned char* qs, int, int q0, int lane)
-        : scale(p.scale_log2), qg(lane >> 3), rg(lane & 7), q_lane(smem_u32(qs) + (q0 + (lane >> 3)) * QROW), p_off(q0 ? SROWS * PROW : 0)
+    __device__ __forceinline__ MathF32(const AttnParams& p, const unsigned char* qs, int, int q0, int lane, int rows)
+        : scale(p.scale_log2), qg(lane >> 3), rg(lane & 7), q_lane(smem_u32(qs) + (q0 + (lane >> 3)) * QROW), p_off(q0 ? SROWS * PROW : 0), few(rows <= GROWS / 2)
     {
 #pragma unroll
         for (int i = 0; i < QL; ++i) {
@@ -89,21 +90,22 @@ struct MathF32 {
     struct Row {
         float w[QP];
         uint64_t v[D / 32][2];
+        template <int N>
         __device__ __forceinline__ void load(uint32_t pr, uint32_t vb, int rg, int r)
         {
 #pragma unroll
-            for (int i = 0; i < QP; i += 2)
+            for (int i = 0; i < (N + 1) / 2 * 2; i += 2)
                 asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(w[i]), "=f"(w[i + 1]) : "r"(pr + (uint32_t)(r * PROW + i * 4)) : "memory");
             const uint32_t a = vb + (uint32_t)(r * 128) + (uint32_t)((rg ^ (r & 7)) << 4);
 #pragma unroll
             for (int h = 0; h < D / 32; ++h) lds4(a + (uint32_t)(h * (SROWS * 128)), v[h][0], v[h][1]);
         }
         // SOME: only for the query rows that see the KV row, r (a weight of 0 is no help against an infinite or NaN value)
-        template <bool SOME>
+        template <int N, bool SOME>
         __device__ __forceinline__ void fma(uint64_t (&o)[QL][D / 32][2], const uint32_t (&mk)[ROWS], int r) const
         {
 #pragma unroll
-            for (int i = 0; i < QL; ++i) {
+            for (int i = 0; i < N; ++i) {
                 if (SOME && !((mk[i] >> r) & 1u)) continue;
                 const uint64_t w2 = pair(w[i], w[i]);
 #pragma unroll
@@ -117,20 +119,27 @@ struct MathF32 {
     template <class F>
     __device__ __forceinline__ void stage(uint32_t kb, bool masked, const uint32_t (&mk)[ROWS], uint32_t, F&& k_read)
     {
-        uint64_t s2[QL][JR];                               // (sum over even columns, sum over odd columns)
+        // (one group: its tile is made for the widest frontier, and a single field would pay for all of it)
+        if (GROUPS == 1 && few) stage_rows<QL / 2>(kb, masked, mk, k_read);
+        else stage_rows<QL>(kb, masked, mk, k_read);
+    }
+    template <int N, class F>
+    __device__ __forceinline__ void stage_rows(uint32_t kb, bool masked, const uint32_t (&mk)[ROWS], F&& k_read)
+    {
+        uint64_t s2[N][JR];                               // (sum over even columns, sum over odd columns)
 #pragma unroll
-        for (int i = 0; i < QL; ++i)
+        for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int j = 0; j < JR; ++j) s2[i][j] = 0ull;
         // S = Q K^T: columns 4 d4 .. + 3 sit in chunk d4 of their panel, XORed with the row.  With two warps per scheduler (one
         // group) a step's operands are read a step ahead; with three that costs registers and gains nothing.
         constexpr int AHEAD = GROUPS == 1 && QL <= 6 ? 1 : 0;
-        uint64_t k[AHEAD + 1][JR][2], q[AHEAD + 1][QL][2];
+        uint64_t k[AHEAD + 1][JR][2], q[AHEAD + 1][N][2];
         auto load = [&](auto B, uint32_t kc, uint32_t qc) {
 #pragma unroll
             for (int j = 0; j < JR; ++j) lds4(kc + j * 1024, k[B][j][0], k[B][j][1]);
 #pragma unroll
-            for (int i = 0; i < QL; ++i) lds4(qc + i * 4 * QROW, q[B][i][0], q[B][i][1]);
+            for (int i = 0; i < N; ++i) lds4(qc + i * 4 * QROW, q[B][i][0], q[B][i][1]);
         };
         uint32_t ka = kb + (uint32_t)rg * 128, qa = q_lane;
         if (AHEAD) load(std::integral_constant<int, 0>{}, ka + (uint32_t)(rg << 4), qa);
@@ -141,7 +150,7 @@ struct MathF32 {
                 load(std::integral_constant<int, AHEAD ? (d4 + 1) & 1 : 0>{}, ka + step * (SROWS * 128) + (uint32_t)((at ^ rg) << 4), qa + step * 128 + at * 16);
                 constexpr int use = AHEAD ? d4 & 1 : 0;
 #pragma unroll
-                for (int i = 0; i < QL; ++i) {
+                for (int i = 0; i < N; ++i) {
 #pragma unroll
                     for (int j = 0; j < JR; ++j) s2[i][j] = fma2(q[use][i][0], k[use][j][0], s2[i][j]);
 #pragma unroll
@@ -151,9 +160,9 @@ struct MathF32 {
             ka += SROWS * 128;
             qa += 128;
         }
-        float s[QL][JR];
+        float s[N][JR];
 #pragma unroll
-        for (int i = 0; i < QL; ++i)
+        for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int j = 0; j < JR; ++j) {
                 const float2 x = halves(s2[i][j]);
@@ -161,7 +170,7 @@ struct MathF32 {
             }
         k_read();                                          // both groups have read the K rows: the weights take their place
 #pragma unroll
-        for (int i = 0; i < QL; ++i) {
+        for (int i = 0; i < N; ++i) {
 #pragma unroll
             for (int j = 0; j < JR; ++j) {
                 s[i][j] *= scale;
@@ -195,8 +204,8 @@ struct MathF32 {
 #pragma unroll
         for (int j = 0; j < JR; ++j)
 #pragma unroll
-            for (int i = 0; i < QP; i += 2)
-                asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(pw + (uint32_t)(j * 8 * PROW + i * 4)), "f"(s[i][j]), "f"(i + 1 < QL ? s[i + 1 < QL ? i + 1 : 0][j] : 0.f) : "memory");
+            for (int i = 0; i < (N + 1) / 2 * 2; i += 2)
+                asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(pw + (uint32_t)(j * 8 * PROW + i * 4)), "f"(s[i][j]), "f"(i + 1 < N ? s[i + 1 < N ? i + 1 : 0][j] : 0.f) : "memory");
         const uint32_t vb = kb + STAGE_BYTES / 2, pr = kb + p_off + (uint32_t)qg * (QP * 4);
         __syncwarp();
         // O += P V, a KV row a step.  Rows that a query row does not see can hold anything, a sibling field's infinities
@@ -205,19 +214,19 @@ struct MathF32 {
             Row x;
 #pragma unroll 1
             for (int r = 0; r < SROWS; ++r) {
-                x.load(pr, vb, rg, r);
-                x.template fma<true>(o, mk, r);
+                x.template load<N>(pr, vb, rg, r);
+                x.template fma<N, true>(o, mk, r);
             }
         } else {
             // the next row's operands are read while this one's FMAs run
             Row x, y;
-            x.load(pr, vb, rg, 0);
+            x.template load<N>(pr, vb, rg, 0);
 #pragma unroll 1
             for (int r = 0; r < SROWS; r += 2) {
-                y.load(pr, vb, rg, r + 1);
-                x.template fma<false>(o, mk, r);
-                if (r + 2 < SROWS) x.load(pr, vb, rg, r + 2);
-                y.template fma<false>(o, mk, r + 1);
+                y.template load<N>(pr, vb, rg, r + 1);
+                x.template fma<N, false>(o, mk, r);
+                if (r + 2 < SROWS) x.template load<N>(pr, vb, rg, r + 2);
+                y.template fma<N, false>(o, mk, r + 1);
             }
         }
         __syncwarp();

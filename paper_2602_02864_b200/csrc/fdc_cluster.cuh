@@ -466,7 +466,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     }
     const int mg = warp % groups, kl = warp / groups;
     const int left = M - mg * GROWS;                       // rows of this warp's group that exist (<= 0: none)
-    Math math(p, qs, qrows, left > 0 ? mg * GROWS : 0, lane);
+    Math math(p, qs, qrows, left > 0 ? mg * GROWS : 0, lane, left);
     const uint8_t* fld = bs.fld + mg * GROWS;              // fields of the group's query rows
     bool alive = true;
     int st = kl, use = 1;                                  // slot of stage `it`, and how many stages (this one included) have used it
