@@ -130,14 +130,6 @@ struct Run {
     int nx;                                   // stages of new rows, ahead of the tile parts
     int total;                                // stages
 };
-// First position of block `rank`'s run among `parts` tile parts, the first `pre` of them whole prefix.  A part beyond the
-// prefix counts half: while fields are being decoded, about half of their slots' parts hold no row yet and are left out.
-__device__ __forceinline__ int run_begin(int rank, int nblk, int parts, int pre)
-{
-    if (pre > parts) pre = parts;
-    const int x = (int)((long long)rank * (parts + pre) / nblk);
-    return x <= 2 * pre ? (x + 1) >> 1 : x - pre;
-}
 template <int SROWS>
 __device__ __forceinline__ int list_row0(const Run& r, int pos)
 {
@@ -294,8 +286,8 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     Run r;
     r.tiles = p.tiles + (size_t)s * p.ntile_max;
     r.mask = p.mask + (size_t)s * p.max_active * p.W;
-    r.h0 = run_begin(rank, nblk, PARTS * nt, PARTS * (p.P / FDC_TILE_ROWS));
-    r.h1 = run_begin(rank + 1, nblk, PARTS * nt, PARTS * (p.P / FDC_TILE_ROWS));
+    r.h0 = run_begin(rank, nblk, PARTS * nt);
+    r.h1 = run_begin(rank + 1, nblk, PARTS * nt);
     r.p0 = PARTS * (p.P / FDC_TILE_ROWS);                      // the whole tiles of the prefix come first in a list
     if (r.p0 < r.h0) r.p0 = r.h0;
     if (r.p0 > r.h1) r.p0 = r.h1;

@@ -72,6 +72,17 @@ struct ClusterProblem {
         return pairs == o.pairs && mmax == o.mmax && head_dim == o.head_dim && P == o.P && T == o.T && sm_count == o.sm_count;
     }
 };
+#ifdef __CUDACC__
+#define FDC_HD __host__ __device__ __forceinline__
+#else
+#define FDC_HD inline
+#endif
+// First of block `rank`'s run among a pair's `parts` tile parts (cluster kernels): equal runs.  The listed parts beyond the
+// prefix count in full: while the last fields of a template are decoded all of them hold rows.  Counted half, a block with many of them took up
+// to twice as many.  us a layer, half / full: fp32, 14/2 heads x 64, 9 fields, 4 scenes, prefix 3000, the last field 45.6 / 35.2; 4/2 x 64, 24
+// fields, 8 scenes, prefix 2048, the last field 56.9 / 39.3; bf16, 50 pairs of 50 rows x 64, prefix 2215 43.0 / 37.7; 4 pairs of 112 rows x 128, prefix
+// 707 12.9 / 11.6.  What it gained was less: fp32, 32/8 x 128, six fields at work, 8 scenes, prefix 2048 75.7 / 79.5.
+FDC_HD int run_begin(int rank, int nblk, int parts) { return (int)((long long)rank * parts / nblk); }
 ClusterShape pick_cluster(const ClusterProblem& c, float* us);      // us (may be NULL): the estimated time
 // The largest cluster of at most `nblk` blocks that the device can place (a single block always can).
 template <class F>

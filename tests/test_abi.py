@@ -82,3 +82,20 @@ def test_cluster_size_that_a_device_cannot_place(tmp_path):
     assert largest(6, [1, 2, 4, 8])[0] == 4
     assert largest(8, [])[0] == 1                             # (single blocks are not asked about)
     assert largest(1, [])[0] == 1
+
+
+def test_runs_of_a_cluster_are_equal(tmp_path):
+    """The blocks of a cluster share a pair's tile parts out evenly, whatever the parts hold, and leave none out."""
+    import subprocess
+    src = tmp_path / "runs.cpp"
+    src.write_text('#include "fdc_internal.h"\n#include <cstdio>\n'
+                   'int main() { for (int n = 1; n <= 16; ++n) for (int parts = 0; parts <= 2200; ++parts) {\n'
+                   'if (fdc::run_begin(0, n, parts) != 0 || fdc::run_begin(n, n, parts) != parts) { printf("ends %d %d\\n", n, parts); return 1; }\n'
+                   'for (int r = 0; r < n; ++r) { const int k = fdc::run_begin(r + 1, n, parts) - fdc::run_begin(r, n, parts);\n'
+                   'if (k < parts / n || k > (parts + n - 1) / n) { printf("run %d of %d: %d of %d\\n", r, n, k, parts); return 1; } } }\n'
+                   'return 0; }\n')
+    exe = tmp_path / "runs"
+    subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2602_02864_b200", "csrc"),
+                           "-I", "/usr/local/cuda/include", str(src), "-o", str(exe)])
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
