@@ -39,8 +39,7 @@ def build_bind(force: bool = False) -> str:
     return BIND
 
 
-def build(force: bool = False, verbose: bool = False) -> str:
-    build_bind(force)
+def build_lib(force: bool = False, verbose: bool = False) -> str:
     if not force and not needs_build():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -65,6 +64,17 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.check_call([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp] + objs + ["-lcudart_static", "-ldl", "-lrt", "-lpthread"])
     os.replace(tmp, LIB)
     return LIB
+
+
+def build(force: bool = False, verbose: bool = False) -> str:
+    """The library, then the binding's module.  Without that one (no C compiler, no Python.h) the library serves every caller, the
+    binding through ctypes."""
+    lib = build_lib(force, verbose)
+    try:
+        build_bind(force)
+    except (OSError, subprocess.CalledProcessError) as e:
+        sys.stderr.write(f"{os.path.basename(BIND)} could not be built ({e}): the binding goes through ctypes\n")
+    return lib
 
 
 if __name__ == "__main__":

@@ -1,6 +1,6 @@
 /* The calls of a pass (fdc_frontier, fdc_build_masks, and per layer fdc_kv_append, fdc_decode_attn) for Python without
- * ctypes.  What bounds a pass that the host issues call by call is the host: ctypes takes 2 to 3 us to convert the 8 to 13
- * arguments of a call, about as long as the launch itself; here the same arguments (integers, tensors, None) take 0.3 us.
+ * ctypes.  What bounds a pass that the host issues call by call is the host: ctypes takes 2.1 to 2.9 us to convert the 8 to 13
+ * arguments of a call, about as long as the launch itself; here the same arguments (integers, tensors, None) take 0.5 to 0.7 us.
  *
  * A function returns the library's return code, or None when an argument is of a kind that it does not convert;
  * the caller then makes the call through ctypes, which accepts and refuses what it always did. */

@@ -1,4 +1,7 @@
 """The extension module of the binding against ctypes: the same calls accepted, refused and answered alike."""
+import os
+import subprocess
+import sys
 import types
 
 import numpy as np
@@ -44,3 +47,25 @@ def test_usual_arguments_do_not_go_through_ctypes():
     assert fdc._fdc_bind.decode_attn(0, kv, 0, T, T, T, T, T, T, 0.5, None, 0, 0) == fdc.FDC_ERR_NULL
     assert fdc._fdc_bind.frontier(0, 1, T, None, T, T, T, T, T, T, 0) == fdc.FDC_ERR_NULL
     assert fdc._fdc_bind.build_masks(0, 1, T, T, T, T, T, 0) == fdc.FDC_ERR_NULL
+
+
+def test_without_the_module_every_call_goes_through_ctypes():
+    code = ("import sys; sys.modules['paper_2602_02864_b200._fdc_bind'] = None\n"       # (an import of it raises ImportError)
+            "from paper_2602_02864_b200 import fdc\n"
+            "kv = fdc.fdc_kv_desc()\n"
+            "for f in (lambda: fdc.fdc_frontier(0, 1, 0, None, 0, 0, 0, 0, 0, 0, 0), lambda: fdc.fdc_build_masks(0, 1, 0, 0, 0, 0, 0, 0),\n"
+            "          lambda: fdc.fdc_kv_append(0, kv, 0, 0, 0, 0, 0, 0), lambda: fdc.fdc_decode_attn(0, kv, 0, 0, 0, 0, 0, 0, 0, 0.5, 0, 0, 0)):\n"
+            "    try: f()\n"
+            "    except fdc.FdcError as e: print(e.code)\n")
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.split() == [str(fdc.FDC_ERR_NULL)] * 4
+
+
+def test_the_library_is_built_without_a_c_compiler(monkeypatch, tmp_path):
+    from paper_2602_02864_b200 import build
+    build.build()
+    monkeypatch.setenv("CC", str(tmp_path / "no_such_compiler"))
+    monkeypatch.setattr(build, "BIND", str(tmp_path / "_fdc_bind.so"))
+    assert build.build() == build.LIB and os.path.exists(build.LIB)
