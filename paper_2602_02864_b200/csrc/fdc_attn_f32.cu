@@ -8,15 +8,9 @@
 // share their query rows and differ in KV rows and columns.  A 16-byte read of a warp takes the port 4 cycles when the
 // lanes of a quarter differ and 2 when they agree (measured).  FMAs go two to an instruction (about 80 % of their
 // rate with three different operands), which leaves issue slots for the reads.
-// A stage keeps its slot for as long as it is worked on, so what an SM does is the number of slots (12 of 16 KB) over a
-// stage's time: small stages with one warp each, or two groups of warps on a stage, beat larger tiles per warp.
-// Measured (us a layer, 32/8 heads x 128, prefix 2000):  8 warps x 32-row stages x 24 query rows 94 at 8 scenes with
-// six fields, 12 warps in two groups on 32-row stages 83, on 16-row stages 86; eight fields at 4 scenes 100 / 70 / 66;
-// three fields at 8 scenes 66 / 85 / 63.  The kernel that ran before (one warp per query row) took 955 in the first.
-// Up to 16 query rows one group of 12 warps does (tiles of 2 and 4).  With 17 to 32, two groups would read every K and V row twice,
-// and the port (14 cycles for 6 of FMAs in the scores, 18 for 12 in the result) is what they wait for; one group of 8 warps with tiles of
-// 6 or 8 query rows a lane (20 for 12, 20 for 24) takes 75 instead of 85 us a layer at 8 scenes with six fields, and 71 with runs cut evenly and the scores'
-// operands read a step ahead.
+// A stage keeps its slot for as long as it is worked on, so what an SM does is the number of slots (10 to 12 of 16 KB with head_dim 128)
+// over a stage's time.  Which tile and how many warps: see launch_attn_f32.  The kernel that ran before this one (one warp per query
+// row) took 955 us a layer at 8 scenes with six fields, 32/8 heads x 128, prefix 2000, where this one takes 80.
 #include "fdc_cluster.cuh"
 
 using namespace fdc;
@@ -131,9 +125,9 @@ struct MathF32 {
         for (int i = 0; i < N; ++i)
 #pragma unroll
             for (int j = 0; j < JR; ++j) s2[i][j] = 0ull;
-        // S = Q K^T: columns 4 d4 .. + 3 sit in chunk d4 of their panel, XORed with the row.  With two warps per scheduler (one
-        // group) a step's operands are read a step ahead; with three that costs registers and gains nothing.
-        constexpr int AHEAD = GROUPS == 1 && QL <= 6 ? 1 : 0;
+        // S = Q K^T: columns 4 d4 .. + 3 sit in chunk d4 of their panel, XORed with the row.  With two warps per scheduler (8 warps) a
+        // step's operands are read a step ahead; with three that costs registers and gains nothing.
+        constexpr int AHEAD = NW == 8 ? 1 : 0;
         uint64_t k[AHEAD + 1][JR][2], q[AHEAD + 1][N][2];
         auto load = [&](auto B, uint32_t kc, uint32_t qc) {
 #pragma unroll
@@ -217,6 +211,13 @@ struct MathF32 {
                 x.template load<N>(pr, vb, rg, r);
                 x.template fma<N, true>(o, mk, r);
             }
+        } else if (GROUPS == 1 && NW == 12) {              // (tiles of 6 rows at 168 registers: no room for a second row's operands)
+            Row x;
+#pragma unroll 1
+            for (int r = 0; r < SROWS; ++r) {
+                x.template load<N>(pr, vb, rg, r);
+                x.template fma<N, false>(o, mk, r);
+            }
         } else {
             // the next row's operands are read while this one's FMAs run
             Row x, y;
@@ -261,10 +262,10 @@ int launch_d(const AttnParams& p, const ClusterShape& h, int ql, cudaStream_t st
     switch (ql) {
         case 2: return launch_cluster<MathF32<D, 2, 12, 2>>(attn_f32_kernel<D, 2, 12, 2>, p, room, h, st);
         case 4: return launch_cluster<MathF32<D, 4, 12, 2>>(attn_f32_kernel<D, 4, 12, 2>, p, room, h, st);
-        case 6: return launch_cluster<MathF32<D, 6, 8, 1>>(attn_f32_kernel<D, 6, 8, 1>, p, room, h, st);
-        default:
-            if constexpr (D == 64) return launch_cluster<MathF32<D, 8, 8, 1>>(attn_f32_kernel<D, 8, 8, 1>, p, room, h, st);
-            return FDC_ERR_SHAPE;
+        default: {
+            constexpr int NW = D == 64 ? 12 : 8;
+            return launch_cluster<MathF32<D, 6, NW, 1>>(attn_f32_kernel<D, 6, NW, 1>, p, room, h, st);
+        }
     }
 }
 
@@ -272,15 +273,24 @@ int launch_d(const AttnParams& p, const ClusterShape& h, int ql, cudaStream_t st
 
 namespace fdc {
 
-// fp32 only.  Clusters per pair: as many as 32 query rows each need, all of the same width; up to 8 and up to 16 query
-// rows are one group (QL 2, 4), up to 24 and 32 two (QL 3, 4): one group reads a stage once.  Blocks per cluster:
-// what keeps all clusters on the chip at once (one block per SM; clusters of 2, 4, 8 that fit a B200 at once: 74,
-// 33, 15), and no more than give every block at least two tiles (eight stages).
+// fp32 only.  Clusters per pair: as many as 32 query rows each need, all of the same width.  Blocks per cluster: what keeps all
+// clusters on the chip at once (one block per SM; clusters of 2, 3, 4, 6, 8 that fit a B200 at once: 74, 45, 33, 22, 15), and no more
+// than give every block at least two tiles (eight stages).  The tile, by a cluster's query rows:
+//   1 to 8, 9 to 16   QL 2, 4: 12 warps in one group.
+//   17 to 24          QL 6, one group: in two, every K and V row is read twice, and the shared memory port (14 cycles for 6 of FMAs in the
+//                     scores, 18 for 12 in the result, against 20 for 12 and 20 for 24) is what they wait for.  head_dim 128 has 8 warps (an
+//                     accumulator of 96 registers), 64 has 12: a pass with few fields at work has a warp per stage as its only
+//                     parallelism, and 8 of them took 73.2 -> 91.8 us a layer with 24 fields done, 48 pairs of 48 rows.  us a layer, QL 3 in two
+//                     groups of 12 warps / this: 8 scenes, 32/8 x 128, six fields, prefix 2048 88.8 / 79.6, one field left 61.8 / 58.2; 24 scenes,
+//                     prefix 256, one field left 77.3 / 80.5 (here two groups are better); 8 scenes, 4/2 x 64, 24 fields, prefix 2048 47.7 / 42.4, one
+//                     field left 36.9 / 37.3.
+//   25 to 32          QL 4 in two groups of 12 warps: one group with tiles of 8 rows is 1 to 10 % slower with head_dim 128, and with 64
+//                     slower where few fields are at work (48 pairs of 56 rows, prefix 256, one field left 40.4 / 43.3).
 int launch_attn_f32(const AttnParams& p, int head_dim, cudaStream_t st)
 {
     ClusterShape h{1, (p.mmax + 31) / 32, 1};
     const int per = (p.mmax + h.qsplit - 1) / h.qsplit;
-    const int ql = per <= 8 ? 2 : (per <= 16 ? 4 : (per <= 24 ? 6 : (head_dim == 64 && h.qsplit > 1 ? 8 : 4)));
+    const int ql = per <= 8 ? 2 : (per <= 16 ? 4 : (per <= 24 ? 6 : 4));
     if (ql == 6) h.qsplit = (p.mmax + 23) / 24;
     const long long clusters = (long long)p.batch * p.hkv * h.qsplit;
     static const int sizes[] = {2, 3, 4, 6, 8}, holds[] = {74, 45, 33, 22, 15};

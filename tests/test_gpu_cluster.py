@@ -103,6 +103,21 @@ def test_fp32_cluster_kernel_whole_schedules(head_dim, hq, hkv, fields, batch, p
     assert r["checked"] > 0
 
 
+# fp32, one query row a field, fields that end one after the other while the prefix is long enough for stages without a mask: every number of
+# rows at work from the widest down to one, half tiles and whole ones (24 rows: up to 12 / more), one group of warps and two
+# (32 rows: up to 16 / more), and clusters of a pair that run out of rows (48, 56: several clusters of 24, 32)
+@pytest.mark.parametrize("head_dim,fields,batch,hkv,prefix", [
+    (64, 24, 1, 2, 700), (64, 24, 30, 4, 130), (64, 32, 2, 2, 400), (64, 48, 1, 2, 520), (64, 56, 2, 1, 300), (128, 24, 1, 2, 700), (128, 24, 24, 4, 130),
+    (128, 20, 3, 1, 1500), (128, 32, 2, 2, 400), (128, 48, 1, 2, 520), (128, 64, 1, 1, 260)])
+def test_fp32_every_number_of_rows(head_dim, fields, batch, hkv, prefix):
+    w = wl.random_template(8500 + fields + batch, n_nodes=fields, edge_prob=0.0, cap_lo=fields + 1, cap_hi=fields + 1, batch=batch, prefix_len=prefix, fixed_hi=0,
+                           hq=hkv, hkv=hkv, head_dim=head_dim, dtype="f32")
+    w.max_active, w.lens = fields, w.lens.copy()
+    w.lens[:] = [1 + (v * 7) % fields if fields % 7 else 1 + (v * 5) % fields for v in range(fields)]
+    r = run_and_compare(w)
+    assert r["steps"] == fields and r["checked"] > 0
+
+
 # Every cut that the library takes can be launched: one kernel a call (a call that fell back would launch two).  The shapes' best cut by the
 # estimate alone, clusters of two blocks with 80 and 112 query rows and two blocks per SM, finds no room for the partials.
 @pytest.mark.parametrize("hq,hkv,fields,batch,prefix", [(20, 4, 16, 32, 1024), (28, 4, 16, 24, 2048), (128, 8, 8, 3, 512)])
