@@ -61,20 +61,27 @@ static float tc_estimate(const ClusterProblem& c)
     return fmaxf(fixed[k] + round[k] * busiest + 11.2f * fmaxf(0.f, pairs / sms - 1.f), t_mem);
 }
 
-// The cluster kernel's cut of this problem and whether it is the faster kernel (kept in the plan: both follow
-// from the shapes alone).  Where both kernels can run, the one with the lower estimate is taken.  Of 226 shapes with head_dim
-// 128 timed on both (2 to 288 pairs, prefix 256 to 32600, 4 to 128 query rows, one or more fields of the template at work), the kernel and the
-// cut taken are on average 10 % slower than the best kernel and cut, from 13 % with the line at 0.82 of the other's estimate and the
-// constants before; one shape in twenty is slower than it was by 4 % or more.  Cluster / tcgen05 kernel, us a layer: 1 scene x 7 query
-// rows, prefix 2048 6.6 / 14.5, 1 scene x 42 rows 10.1 / 18.2; 32 pairs x 20 rows, prefix 9922 33.4 / 37.0; 16 scenes x 24 rows,
-// prefix 4096 59 / 52.
+// The cluster kernel's cut of a problem, and whether it is the faster kernel for it: its estimate against the tcgen05 kernel's.  Its blocks
+// do not share work with one another beyond a pair, so with one block a pair scenes that have ended, or have few fields left, leave
+// their SMs idle, where the tcgen05 kernel deals all the work out anew: there it has to be the better one by 15 %.  Of 1110 shapes with head_dim 128
+// (2 to 500 pairs, prefix 256 to 32700, 4 to 128 query rows, any pass of their templates) the kernel and the cut taken are on average 11 % slower than the
+// best kernel and cut timed. Against the kernel with two cluster barriers in its merge, its cuts without the ring's turns and a line at 0.82,
+// 509 are faster by more than 4 % and 14 slower by more than that (7 by more than 10 %: pairs of few rows over long prefixes, and scenes that have
+// ended; 72 pairs of 8 rows, prefix 6396, most scenes at their end: 20.3 -> 29.3 us a layer).  Cluster / tcgen05 kernel, us a layer: 1 scene x 7 query rows, prefix 1024
+// 6.1 / 13.8, 1 scene x 42 rows, prefix 2048 9.8 / 17.7; 8 pairs x 7 rows, prefix 5409 13.9 / 19.9; 192 pairs x 36 rows, prefix 2168 102 / 67.
+bool route_problem(const ClusterProblem& c, ClusterShape* cut)
+{
+    float us = 0.f;
+    *cut = pick_cluster(c, &us);
+    return c.head_dim != 128 || us < (cut->nblk == 1 ? 0.85f : 1.05f) * tc_estimate(c);
+}
+
+// (kept in the plan: both follow from the shapes alone)
 static const ClusterShape& route(fdc_plan* p, const fdc_kv_desc* kv)
 {
     const ClusterProblem c{(int64_t)kv->batch * kv->hkv, p->h.max_active * (kv->hq / kv->hkv), kv->head_dim, p->h.P, p->h.T, p->sm_count};
     if (!(p->route_for == c)) {
-        float us = 0.f;
-        p->route_shape = pick_cluster(c, &us);
-        p->route_cluster = kv->head_dim != 128 || us < tc_estimate(c);
+        p->route_cluster = route_problem(c, &p->route_shape);
         p->route_for = c;
     }
     return p->route_shape;

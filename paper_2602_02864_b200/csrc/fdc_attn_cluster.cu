@@ -300,24 +300,26 @@ int get_kv_tensor_map(const void* base, const AttnParams& p, int dtype, int head
 static size_t block_room(int per_sm) { return per_sm > 1 ? 113 * 1024 : 227 * 1024; }       // two blocks per SM: 228 KB, less 1 KB each for the system
 // Stages in the ring of a block of a cluster of n with `rows` query rows; 0: it finds no room for what the other blocks send it
 // beside a ring that its own partials fit.  (With two blocks per SM and head_dim 128: more than 48 rows in clusters of several blocks.)
-template <int D>
-static int ring_of(int rows, int n, int two) { return cluster_ring_stages<MathBf16<D>>(block_room(two + 1), rows, n); }
+int cluster_ring(int head_dim, int rows, int nblk, int per_sm)
+{
+    return head_dim == 64 ? cluster_ring_stages<MathBf16<64>>(block_room(per_sm), rows, nblk) : cluster_ring_stages<MathBf16<128>>(block_room(per_sm), rows, nblk);
+}
 
 // How a launch is cut: blocks per cluster (shares of a pair's rows), clusters per pair (shares of its query
 // rows; each reads all the pair's K/V, the later ones from L2) and blocks per SM, by the lowest estimate of
-//     fixed + waves x (one block's time) + a launch that does not fit beside the one ahead + a ring that stays short
-// where a block's time is the largest of its warps' chain of stages (latency), its SM's share of the
-// arithmetic and its SM's share of the bytes, and an SM with two blocks shares the last two.  Two things decide besides:
-//  - consecutive launches overlap only where both find a place: else the later one's set-up (1 to 2 us) begins when the
-//    one ahead ends.  4 pairs, 7 query rows, prefix 1024: 7.7 us a layer with clusters of 16 and one block per SM (7 fit
-//    the chip), 6.6 with two;
-//  - with two blocks per SM the ring is half as deep, which costs where a run does not fit it.  32 pairs, 20 query rows,
-//    head_dim 128, prefix 9922: 36.3 us a layer with (3, 2, 2), 33.4 with (4, 1, 1).
-// The constants (us) are the best of a grid by the mean loss against the best of up to 60 cuts timed on a B200 for 471
-// shapes (2 to 288 pairs, prefix 256 to 32600, 2 to 128 query rows): the cut taken is on average 8 % (head_dim 64) and 11 %
-// (128) slower than the best one, from 11 and 18 % with the constants before.  Cutting the query rows pays while the chip has
-// idle SMs: one scene, 4 KV heads, 42 query rows, prefix 2048: 16.8 us a layer with one cluster of 16 blocks per KV head,
-// 10.1 us with three.
+//     fixed + waves x (one block's time) + a launch that does not fit beside the one ahead
+// where a block's time is the largest of its warps' chain of stages (latency), its SM's share of the arithmetic and its SM's share
+// of the bytes (an SM with two blocks shares the last two), and its ring's turns.  Two things decide besides the work:
+//  - consecutive launches overlap only where both find a place: else the later one's set-up begins when the one ahead ends.  4
+//    pairs, 7 query rows, prefix 1024: 7.2 us a layer with clusters of 16 and one block per SM (7 fit the chip), 6.1 with two;
+//  - a run longer than the ring gets a ring's stages per turn (a copy's latency and the stage's work: 2.5 us and 0.7 more per group of
+//    query rows), and with two blocks per SM a ring is half as deep.  56 pairs, 12 query rows, prefix 4737: 33.3 us a layer with
+//    (3, 1, 2), 25.0 with (3, 1, 1).
+// The constants (us) are the best of a grid over 1110 (head_dim 128) and 650 (64) shapes drawn over 2 to 500 pairs, prefix 256 to 32700, 2 to 128 query
+// rows, at any pass of their templates, with up to 60 cuts of each timed on a B200: the cut taken with head_dim 64 is on average 8 % slower than the
+// best one timed, 12 % without the last two terms.  562 of the 650 are faster by more than 4 % than with the cuts (and the merge) of before, 8 are slower by
+// more than that (60 pairs of 35 rows, prefix 4802: 35.0 -> 44.9 us a layer).  Cutting the query rows pays while the chip has idle SMs: one
+// scene, 4 KV heads, 42 query rows, prefix 2048: 10.8 us a layer with one cluster of 16 blocks per KV head, 9.8 with three.
 ClusterShape pick_cluster(const ClusterProblem& c, float* us)
 {
     static const int sizes[] = {1, 2, 3, 4, 6, 8, 16};
@@ -325,8 +327,8 @@ ClusterShape pick_cluster(const ClusterProblem& c, float* us)
     // (cudaOccupancyMaxActiveClusters): the SMs of a cluster share one GPC
     static const int holds[2][7] = {{148, 74, 45, 33, 22, 15, 7}, {296, 148, 93, 71, 45, 33, 14}};
     const bool d64 = c.head_dim == 64;
-    const float chain = d64 ? 0.8f : 1.06f, arith = d64 ? 0.08f : 0.16f;       // per stage of a warp; per stage and group of an SM
-    const float merge = d64 ? 1.f : 2.f, late = 0.7f, shallow = d64 ? 0.f : 4.f;
+    const float chain = d64 ? 0.65f : 1.2f, arith = d64 ? 0.11f : 0.21f;       // per stage of a warp; per stage and group of an SM
+    const float merge = 1.f, late = 0.7f;
     const int groups_all = (c.mmax + 15) / 16;
     const float rows = (float)c.P + 0.5f * (float)c.T, pairs = (float)c.pairs, stages = rows / 32.f;
     ClusterShape best{1, 1, 2};
@@ -341,14 +343,15 @@ ClusterShape pick_cluster(const ClusterProblem& c, float* us)
             for (int two = 0; two < 2; ++two) {
                 const float n = (float)sizes[i], clusters = pairs * (float)q, hold = (float)holds[two][i] * (float)c.sm_count / 148.f;
                 if (sizes[i] > 1 && stages < 2.f * n) continue;
-                const int ring = d64 ? ring_of<64>(gl * 16, sizes[i], two) : ring_of<128>(gl * 16, sizes[i], two);
+                const int ring = cluster_ring(c.head_dim, gl * 16, sizes[i], two + 1);
                 if (ring == 0) continue;                   // (no room for the partials)
                 const float waves = clusters > hold ? clusters / hold + 0.4f : 1.f;
                 const float share = two ? fminf(2.f, fmaxf(1.f, clusters * n / (float)c.sm_count)) : 1.f;
                 const float sb = ceilf(stages / n);
-                const float body = fmaxf(ceilf(sb / (float)lanes) * chain, sb * share * fmaxf((float)gl * arith, (float)(c.head_dim * 128) * 1e-3f / 56.f));
-                const float over = fminf(fmaxf((2.f * clusters - hold) / hold, 0.f), 1.f), past = two ? fminf(fmaxf((sb - (float)ring) / (float)ring, 0.f), 1.f) : 0.f;
-                const float t = fmaxf(3.2f + (body + (sizes[i] > 1 ? merge : 0.f) + 4.2f * (float)gl) * waves + late * over + shallow * past, t_mem);
+                const float turns = sb > (float)ring ? (sb - (float)ring) / (float)ring * (2.5f + 0.7f * (float)gl) + chain : 0.f;
+                const float body = fmaxf(fmaxf(ceilf(sb / (float)lanes) * chain, turns), sb * share * fmaxf((float)gl * arith, (float)(c.head_dim * 128) * 1e-3f / 56.f));
+                const float over = fminf(fmaxf((2.f * clusters - hold) / hold, 0.f), 1.f);
+                const float t = fmaxf(3.2f + (body + (sizes[i] > 1 ? merge : 0.f) + 4.2f * (float)gl) * waves + late * over, t_mem);
                 if (t < t_best * 0.995f) {
                     t_best = t;
                     best = ClusterShape{sizes[i], q, two + 1};

@@ -84,6 +84,8 @@ struct ClusterProblem {
 // 707 12.9 / 11.6.  What it gained was less: fp32, 32/8 x 128, six fields at work, 8 scenes, prefix 2048 75.7 / 79.5.
 FDC_HD int run_begin(int rank, int nblk, int parts) { return (int)((long long)rank * parts / nblk); }
 ClusterShape pick_cluster(const ClusterProblem& c, float* us);      // us (may be NULL): the estimated time
+bool route_problem(const ClusterProblem& c, ClusterShape* cut);     // the cut, and whether the cluster kernel is the one to take (head_dim 64: always)
+int cluster_ring(int head_dim, int rows, int nblk, int per_sm);     // stages of a block's ring (bf16); 0: no room for the partials beside it
 // The largest cluster of at most `nblk` blocks that the device can place (a single block always can).
 template <class F>
 int largest_placeable(int nblk, F&& placeable)
