@@ -188,14 +188,22 @@ __device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, const flo
 // Chunk k (query row k / (D / 16), columns 16 (k mod D / 16) ..) belongs to block k mod nblk and is its (k / nblk)-th.
 constexpr int CHUNK_BYTES = 16 * 4 + 8;
 __host__ __device__ __forceinline__ int chunks_of_block(int chunks, int nblk) { return (chunks + nblk - 1) / nblk; }
-// The wait for them.  A block that gives up elsewhere still sends what it has, after a second or so; the limit here is
-// several times that, so that nobody leaves while bytes for it are under way.
+// The wait for them: false where it ran out (nothing of them may then be read).  A sender whose own wait runs out still sends what it
+// has, after its limit (a second or so) and what its earlier waits took.  This wait is flagged after eight such limits and then goes on as long
+// again, so that bytes still under way find the block's memory in place.  That is an assumption, not a guarantee: a sender can be later than
+// both if many of its waits end just short of their limits, in a launch that is lost already; its bytes would then fall into memory that may be another
+// block's.  (A barrier of the cluster that every thread passes before it leaves would rule that out; it costs 1 % on average, and
+// 6.13 -> 6.57 us a layer at 4 pairs x 7 query rows, prefix 1024.)
+constexpr uint32_t PUSHED_FLAG = SPIN_LIMIT * 8, PUSHED_LEAVE = PUSHED_FLAG * 2;
 static __device__ __noinline__ bool wait_pushed_slow(uint32_t bar, volatile int* abort_flag, int32_t* status)
 {
-    for (uint32_t i = 0; i < SPIN_LIMIT * 8; ++i)
+    for (uint32_t i = 0; i < PUSHED_LEAVE; ++i) {
         if (mbar_try(bar, 0)) return true;
-    *abort_flag = 1;
-    atomicOr(status, FDC_DEV_TIMEOUT);
+        if (i + 1 == PUSHED_FLAG) {
+            *abort_flag = 1;
+            atomicOr(status, FDC_DEV_TIMEOUT);
+        }
+    }
     return false;
 }
 // Merge over the lanes of a block, for every (query row, 4 columns): `rows` = query rows of a lane's partial;
@@ -583,8 +591,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
         }
     if (nblk == 1) return;
     // ---- cluster: every block finishes its chunks once all blocks' partials of them are there
-    if (!mbar_try(pushed, 0)) wait_pushed_slow(pushed, abortp, p.status);
-    __syncwarp();
+    if (!__all_sync(0xffffffffu, mbar_try(pushed, 0) || wait_pushed_slow(pushed, abortp, p.status))) return;       // (flagged: no output)
     {
         // Four threads per item (4 columns), each with every fourth block (at most four), summed by shuffles.
         const float4* ro = reinterpret_cast<const float4*>(recv);
