@@ -18,6 +18,7 @@ void note_launch() { g_launch_counter.fetch_add(1, std::memory_order_relaxed); }
 int set_cuda_error(cudaError_t e)
 {
     snprintf(g_cuda_msg, sizeof(g_cuda_msg), "%s: %s", cudaGetErrorName(e), cudaGetErrorString(e));
+    cudaGetLastError();                                    // reported here: the next call's check must not find it again
     return FDC_ERR_CUDA;
 }
 

@@ -88,3 +88,27 @@ def test_loop_limit_stops_the_loop_and_is_flagged():
     w = wl.cfg2_batched(layers=1, batch=2)
     passes, status, n = _play_on_device(w, False, max_passes=5)
     assert n > 5 and passes == 5 and status == fdc.FDC_DEV_LOOP_LIMIT
+
+
+def test_a_failed_launch_is_not_reported_again_by_the_next_call():
+    """The launch of frontier fails on a stream whose capture has become invalid (a copy to the host's stack and a
+    synchronisation cannot be captured); that is reported by the call itself, and the next call on another stream starts afresh."""
+    from paper_2602_02864_b200 import fdc
+    from paper_2602_02864_b200.device_loop import _ok, _rt
+    sess = fdc.DecodeSession(2, [(0, 1)], [4, 4], None, 8, 1, 1)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    raw = _rt.cudaStream_t(stream.cuda_stream)
+    _ok(_rt.cudaStreamBeginCapture(raw, _rt.cudaStreamCaptureMode.cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture")
+    try:
+        with pytest.raises(fdc.FdcError):
+            fdc.fdc_status(sess.plan, stream=stream)
+        with pytest.raises(fdc.FdcError) as e:
+            sess.frontier(stream=stream)
+        assert e.value.code == fdc.FDC_ERR_CUDA
+    finally:
+        assert int(_rt.cudaStreamEndCapture(raw)[0]) != 0
+    sess.init(None)
+    sess.frontier()
+    assert sess.n_active.item() == 1 and sess.status() == 0
+    sess.close()
