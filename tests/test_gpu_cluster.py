@@ -118,20 +118,72 @@ def test_fp32_every_number_of_rows(head_dim, fields, batch, hkv, prefix):
     assert r["steps"] == fields and r["checked"] > 0
 
 
-# Every cut that the library takes can be launched: one kernel a call (a call that fell back would launch two).  The shapes' best cut by the
-# estimate alone, clusters of two blocks with 80 and 112 query rows and two blocks per SM, finds no room for the partials.
-@pytest.mark.parametrize("hq,hkv,fields,batch,prefix", [(20, 4, 16, 32, 1024), (28, 4, 16, 24, 2048), (128, 8, 8, 3, 512)])
+# Sequential decoding of one or two query rows a pair over a long prefix: clusters of 16 blocks, of which 8 or 12 own no part of the result (4 or 8
+# chunks of 16 columns); several layers a pass, append apart and inside
+@pytest.mark.parametrize("fused", [False, True], ids=["append_kernel", "append_inside_attention"])
+@pytest.mark.parametrize("head_dim,hq,hkv,prefix", [(64, 2, 2, 2000), (64, 4, 2, 2000), (128, 4, 4, 2000)])
+def test_blocks_that_own_no_part_of_the_result(head_dim, hq, hkv, prefix, fused):
+    w = wl.random_template(9100 + hq, n_nodes=3, edge_prob=1.0, cap_lo=4, cap_hi=8, batch=1, prefix_len=prefix, fixed_hi=1, hq=hq, hkv=hkv, head_dim=head_dim, dtype="bf16")
+    w.max_active, w.layers = 1, 3
+    r = run_and_compare(w, kernel=2, fused_append=fused)
+    assert r["checked"] > 0
+
+
+# head_dim 64 and fp32 serve a tile list in any order (head_dim 128 in bf16 reports one that does not begin with the prefix): a prefix tile and one beyond
+# the prefix change places, and first and last.  Several layers, so that the later ones read the list ahead of the dependency wait.
+@pytest.mark.parametrize("dtype,head_dim,hq,hkv,prefix", [("bf16", 64, 14, 2, 1000), ("f32", 64, 4, 2, 1000), ("f32", 128, 8, 2, 1000)])
+def test_lists_in_any_order(dtype, head_dim, hq, hkv, prefix):
+    from paper_2602_02864_b200 import fdc
+    fields, batch, layers, passes, slot = 3, 2, 3, 30, 40
+    dt = torch.float32 if dtype == "f32" else torch.bfloat16
+    sess = fdc.DecodeSession(fields, [], [slot] * fields, None, prefix, fields, batch)
+    g = torch.Generator(device="cuda").manual_seed(12)
+    k, v = (torch.randn(batch, layers, hkv, prefix + slot * fields, head_dim, generator=g, device="cuda").to(dt) for _ in range(2))
+    q = torch.randn(layers, batch, fields, hq, head_dim, generator=g, device="cuda").to(dt)
+    sess.bind_cache(k, v, hq)
+    sess.init(None)
+    for _ in range(passes):
+        sess.frontier()
+    npre = prefix // 64
+    outs = []
+    for swap in ([], [(3, npre)], [(0, npre + 1), (npre - 1, npre)]):
+        sess.build_masks()
+        assert int(sess.ntiles.min()) >= npre + 2
+        for i, j in swap:
+            sess.tiles[:, [i, j]] = sess.tiles[:, [j, i]]
+        out = torch.zeros_like(q)
+        for l in range(layers):
+            sess.decode_attn(l, q[l], out[l], head_dim ** -0.5)
+        outs.append(out.double())
+    assert sess.status() == 0
+    # (another order of the same sums: fp32 rounding, and weights and outputs rounded to bf16, 2^-9 each, against other maxima)
+    tol = 2e-6 if dtype == "f32" else 2 ** -7
+    for o in outs[1:]:
+        assert (o - outs[0]).norm() <= tol * outs[0].norm()
+    sess.close()
+
+
+# Every cut that the library takes can be launched: one kernel a call (a call that fell back would launch two).  Clusters with 80 and
+# 112 query rows and two blocks per SM find no room for the partials (that none is taken at any shape: test_routes.py); the output of the first and
+# the last scene against the checker.
+@pytest.mark.parametrize("hq,hkv,fields,batch,prefix", [(20, 4, 16, 32, 1024), (28, 4, 16, 24, 2048), (128, 8, 8, 3, 512), (28, 4, 15, 35, 6166), (32, 8, 18, 38, 3980)])
 def test_the_cut_leaves_room_for_the_partials(hq, hkv, fields, batch, prefix):
+    from harness import check_close, f32
+    from oracle import attention
     from paper_2602_02864_b200 import fdc
     sess = fdc.DecodeSession(fields, [], [16] * fields, None, prefix, fields, batch)
-    k, v = (torch.randn(batch, 1, hkv, prefix + 16 * fields, 128, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    k, v = (torch.randn(batch, 1, hkv, prefix + 16 * fields, 128, device="cuda").mul_(0.5).to(torch.bfloat16) for _ in range(2))
     q = torch.randn(batch, fields, hq, 128, device="cuda", dtype=torch.bfloat16)
     sess.bind_cache(k, v, hq)
     fdc.fdc_set_attn_kernel(sess.plan, 2)
     sess.init(None)
     sess.frontier()
     sess.build_masks()
-    before = fdc.fdc_launch_count()
-    sess.decode_attn(0, q, torch.empty_like(q), 128 ** -0.5)
+    before, out = fdc.fdc_launch_count(), torch.empty_like(q)
+    sess.decode_attn(0, q, out, 128 ** -0.5)
     assert fdc.fdc_launch_count() == before + 1 and sess.status() == 0
+    for s in (0, batch - 1):
+        vis = torch.ones(fields, prefix + 16 * fields, dtype=torch.bool)
+        vis[:, prefix:] = torch.eye(fields, dtype=torch.bool).repeat_interleave(16, 1) & (torch.arange(16 * fields) % 16 == 0)      # its own first row
+        check_close(f32(out[s]), attention.attention(f32(q[s]), f32(k[s, 0]), f32(v[s, 0]), vis.numpy(), 128 ** -0.5), "bf16", f"scene {s}")
     sess.close()
