@@ -7,7 +7,7 @@
 // -> softmax -> output -> merge -> end of the grid).  This kernel is made for a short chain: no TMEM, no
 // arrival counters, no partials in global memory, no second kernel and no split table.  The blocks
 // of a pair take equal runs of its 32-row half tiles; everything of the prefix that fits the ring is
-// requested before the dependency wait; the merge is two trips inside the cluster.  The tensor work
+// requested before the dependency wait; the merge is one one-way trip inside the cluster (fdc_cluster.cuh).  The tensor work
 // is small here (a pair has 1 to 128 query rows), so it is done by mma.sync from registers, which
 // needs no hand-over between issuing thread, tensor memory and softmax threads.
 //
@@ -15,8 +15,8 @@
 // per cluster where the query rows are cut, see pick_cluster).
 //
 // Measured (a layer, graphs of whole passes, against the kernels that served these shapes before): 1 scene, 28/4
-// heads x 128, prefix 1024, one field: 14.6 -> 8.0 us; prefix 2048, six fields: 19.3 -> 11.9; 1 scene, 14/2 heads x
-// 64, prefix 1531, six fields, append apart: 56.2 -> 16.1; 16 scenes, 14/2 x 64, prefix 4096: 56.4 -> 19.4.
+// heads x 128, prefix 1024, one field: 14.6 -> 6.1 us; prefix 2048, six fields: 19.3 -> 9.8; 1 scene, 14/2 heads x
+// 64, prefix 1531, six fields, append apart and issued by the host: 56.2 -> 12.4; 16 scenes, 14/2 x 64, prefix 4096: 56.4 -> 18.4.
 //
 // Block = 8 warps, two blocks per SM (128 registers a thread: the accumulators of 16 query rows take
 // half of them).  A stage is 32 KV rows of K and V (TMA, 128-byte swizzle).  The query rows form 1, 2, 4
@@ -30,7 +30,7 @@
 // Half tiles without any visible row are not loaded at all.
 // Fused append: the pass's new K/V rows are a stage of their own, filled straight from k_new / v_new by the
 // first block of the cluster; in the stages of the cache the same rows count as unseen.  The block whose
-// run holds a row's half tile writes it to the cache after its last stage, while it waits for the cluster.
+// run holds a row's half tile writes it to the cache after it has sent its partials.
 #include <cudaTypedefs.h>
 
 #include <cmath>
