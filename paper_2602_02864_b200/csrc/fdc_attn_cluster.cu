@@ -220,9 +220,9 @@ struct MathBf16 {
 template <int D>
 __global__ void __launch_bounds__(MathBf16<D>::NW * 32, 2)
 attn_cluster_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
-                    const int nstage, const int nblk, const int qsplit, const int qrows)
+                    const __grid_constant__ ClusterArgs args)
 {
-    attn_cluster_body<MathBf16<D>>(p, tm_k, tm_v, nstage, nblk, qsplit, qrows);
+    attn_cluster_body<MathBf16<D>>(p, tm_k, tm_v, args);
 }
 
 // ---------------------------------------------------------------- host side

@@ -249,10 +249,10 @@ struct MathF32 {
 
 template <int D, int QL, int NW, int GROUPS>
 __global__ void __launch_bounds__(NW * 32, 1)
-attn_f32_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const int nstage,
-                const int nblk, const int qsplit, const int qrows)
+attn_f32_kernel(const __grid_constant__ AttnParams p, const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v,
+                const __grid_constant__ ClusterArgs args)
 {
-    attn_cluster_body<MathF32<D, QL, NW, GROUPS>>(p, tm_k, tm_v, nstage, nblk, qsplit, qrows);
+    attn_cluster_body<MathF32<D, QL, NW, GROUPS>>(p, tm_k, tm_v, args);
 }
 
 template <int D>

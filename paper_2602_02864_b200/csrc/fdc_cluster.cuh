@@ -105,17 +105,16 @@ struct __align__(16) BlockState {
     int used[MAX_STAGES];                     // groups that have finished with the stage
     int asked[MAX_STAGES];                    // requests made for the stage so far
     int abort_flag;                           // a bounded wait ran out somewhere in the block
-    int first_beyond;                         // first part of the run that reaches beyond the prefix
-    int n_kept;                               // entries of kept[]
-    int pad;
+    int beyond[NW];                           // first part of the run that reaches beyond the prefix, among those a warp looked at
     float2 wml[NW * GROWS];                   // (m, l) per warp and row of its group ([lane][query row])
     uint64_t pushed;                          // the cluster's partials of this block's chunks have arrived
     uint64_t pad2;
     uint8_t fld[MAX_QROWS];                   // field of every query row of the cluster (0xff: a row past the last)
     int app_row[FDC_MAX_NODES];               // fused append: cache row of every field's new K/V vector, -1: not written
     uint32_t newbits[2 * FDC_MAX_NODES];      // [new rows 0-31, 32-63][field] the new rows that the field sees
-    uint32_t seen[MASK_HALVES];               // rows of a tile part that some field sees
-    uint8_t kept[MASK_HALVES];                // those of them that hold a visible row, in order
+    uint32_t seen[MASK_HALVES];               // rows of a tile part that some field sees and whose values come from the cache
+    uint8_t holds[MASK_HALVES];               // the part holds a visible row
+    uint8_t kept[MASK_HALVES];                // the parts that do, in order
     uint32_t bits[MASK_WORDS];                // [part][field] the rows that the field sees
     int row0[ROW0S];                          // first KV row of the run's parts
 };
@@ -129,6 +128,7 @@ struct Run {
     int h0, h1, p0, np;
     int nx;                                   // stages of new rows, ahead of the tile parts
     int total;                                // stages
+    int n_kept;                               // entries of kept[]
 };
 template <int SROWS>
 __device__ __forceinline__ int list_row0(const Run& r, int pos)
@@ -146,7 +146,7 @@ __device__ __forceinline__ int stage_pos(const Run& r, const Block& bs, int it)
 {
     const int i = it - r.nx - (r.p0 - r.h0);
     if (i < 0) return r.h0 + it - r.nx;
-    return i < bs.n_kept ? r.p0 + bs.kept[i] : r.p0 + r.np + (i - bs.n_kept);
+    return i < r.n_kept ? r.p0 + bs.kept[i] : r.p0 + r.np + (i - r.n_kept);
 }
 // Rows of the tile part that some field sees (whole warp).
 template <int SROWS>
@@ -257,16 +257,28 @@ __device__ __forceinline__ void merge_lanes(int lanes, int tid, int M, int rows,
     }
 }
 
-// The kernel (two blocks' worth of arguments beyond AttnParams: ring slots, blocks per cluster, clusters per
-// pair, query rows per cluster).
+// What a launch's blocks need besides AttnParams.
+struct ClusterArgs {
+    int nstage, nblk, qsplit, qrows;           // ring slots, blocks per cluster, clusters per pair, query rows per cluster
+    uint32_t by_nblk, by_qsplit, by_group;     // div_inverse of nblk, qsplit and the query heads of a KV head
+};
+
+// The kernel.  Grid: x = (KV head, share of the query rows, block of the cluster), y = scene.
+//
+// The set-up is on the path of every launch whose blocks find no place beside the launch ahead (and of the first of a pass), and
+// it is a chain of trips to memory (counts -> tile list -> bitmaps), fences and, more than both, of instructions that are fetched for one
+// execution.  So: the barriers and the prefix's first stages are warp 0's alone, which needs no barrier of the block for it; the
+// other warps prepare the visibility meanwhile, a warp per tile part, a lane per field; one barrier of the block ends it; and
+// nothing is divided.  Cycles from the block's first instruction to its dependency wait, all warps going through every step with three barriers of the
+// block and a releasing arrival at the cluster's (1000 cycles by itself) / now: see the figures at launch_cluster.
 template <class Math>
-__device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const int nstage, const int nblk,
-                                                  const int qsplit, const int qrows)
+__device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const ClusterArgs& ca)
 {
     constexpr int D = Math::D, GROWS = Math::GROWS, STAGE_BYTES = Math::STAGE_BYTES, NW = Math::NW, THREADS = NW * 32, SROWS = Math::SROWS;
     constexpr int PARTS = FDC_TILE_ROWS / SROWS;           // stages of a tile
     constexpr int CHUNK = 16 / sizeof(typename Math::Elem);         // elements of a 16-byte chunk
     extern __shared__ unsigned char smem_dyn[];
+    const int nstage = ca.nstage, nblk = ca.nblk, qrows = ca.qrows;
     unsigned char* ring = reinterpret_cast<unsigned char*>(((uintptr_t)smem_dyn + 1023) & ~(uintptr_t)1023);
     unsigned char* qs = ring + (size_t)nstage * STAGE_BYTES;
     unsigned char* recv = qs + Math::q_bytes(qrows);       // partials of this block's chunks, from all blocks of the cluster
@@ -274,58 +286,42 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     __shared__ BlockState<NW, GROWS> bs;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int rank = blockIdx.x % nblk;                    // = rank in the cluster (the grid is cut into runs of nblk blocks)
-    const int cluster = blockIdx.x / nblk;
-    const int pair = cluster / qsplit, m0 = (cluster - pair * qsplit) * qrows;      // this cluster: query rows m0 .. m0 + qrows - 1 of the pair
-    const int s = pair / p.hkv, g = pair - s * p.hkv;
+    const int s = blockIdx.y, cluster = (int)div_by(blockIdx.x, ca.by_nblk), rank = (int)blockIdx.x - cluster * nblk;      // rank in the cluster
+    const int g = (int)div_by((uint32_t)cluster, ca.by_qsplit), m0 = (cluster - g * ca.qsplit) * qrows;      // this cluster: query rows m0 .. m0 + qrows - 1 of the pair
     // Programmatic dependent launch: as in the tcgen05 kernel (fdc_attn_tc_kernel.cuh).  With p.early the pass
-    // tables and the prefix rows may be read ahead of the wait; every thread passes the wait.
+    // tables and the prefix rows may be read ahead of the wait.
     if (!p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // (the launch may be ahead of whatever writes the new rows' numbers: what is read here is checked after the wait)
-    int ar0 = p.app_row && tid < p.max_active ? p.app_row[(size_t)s * p.max_active + tid] : -1;
     const int A = p.n_active[s], nt = p.ntiles[s];
-    if (A * p.group <= m0 || nt <= 0) {                    // nothing to do (all blocks of the cluster agree)
-        if (p.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+    // (the launch may be ahead of whatever writes the new rows' numbers: what is read here is checked after the wait)
+    const int32_t* app = p.app_row ? p.app_row + (size_t)s * p.max_active : nullptr;
+    int ar[2];                                             // lane: of fields lane and lane + 32
+#pragma unroll
+    for (int j = 0; j < 2; ++j) ar[j] = app && lane + 32 * j < p.max_active ? app[lane + 32 * j] : -1;
+    if (A * p.group <= m0 || nt <= 0) {
+        // Nothing to do (all blocks of the cluster agree).  Such blocks leave at once: their places go to the next launch's blocks, which set
+        // themselves up meanwhile.  One block of the grid waits for the launch ahead, so that grids still complete in stream order.
+        // us a layer, all of them waiting / this: 3 scenes, 28/4 heads, one of five fields left, prefix 1000: 10.7 / 7.
+        if (p.early && blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }
     const int M = A * p.group - m0 < qrows ? A * p.group - m0 : qrows;
     const int groups = Math::GROUPS == 1 || M <= GROWS ? 1 : (Math::GROUPS == 2 || M <= 2 * GROWS ? 2 : (M <= 4 * GROWS ? 4 : 8)), lanes = NW / groups;
+    auto by_nblk = [&](uint32_t x) { return div_by(x, ca.by_nblk); };
     Run r;
     r.tiles = p.tiles + (size_t)s * p.ntile_max;
     r.mask = p.mask + (size_t)s * p.max_active * p.W;
-    r.h0 = run_begin(rank, nblk, PARTS * nt);
-    r.h1 = run_begin(rank + 1, nblk, PARTS * nt);
-    r.p0 = PARTS * (p.P / FDC_TILE_ROWS);                      // the whole tiles of the prefix come first in a list
+    r.h0 = run_begin(rank, nblk, PARTS * nt, by_nblk);
+    r.h1 = run_begin(rank + 1, nblk, PARTS * nt, by_nblk);
+    const int whole = p.P / FDC_TILE_ROWS;                     // the whole tiles of the prefix come first in a list
+    r.p0 = PARTS * whole;
     if (r.p0 < r.h0) r.p0 = r.h0;
     if (r.p0 > r.h1) r.p0 = r.h1;
     r.np = r.h1 - r.p0;
-    if (r.np > MASK_WORDS / A) r.np = MASK_WORDS / A;
+    if (r.np * A > MASK_WORDS) r.np = (int)__fdividef((float)MASK_WORDS, (float)A);       // (any number will do that is not too high)
     if (r.np > MASK_HALVES) r.np = MASK_HALVES;
-    const int chunks = M * (D / 16), slots = chunks_of_block(chunks, nblk);     // chunks of the result, of one block at most
-    // ---- set-up: barriers, the prefix's first stages, the run's rows, the fields' visibility beyond the prefix
-    r.nx = p.app_row && rank == 0 ? (A + SROWS - 1) / SROWS : 0;
-    if (tid < nstage) {
-        bs.used[tid] = 0;
-        bs.asked[tid] = tid < r.nx ? 1 : 0;
-        mbar_init(smem_u32(&bs.full[tid]), 1);
-        if (Math::K_REUSED) mbar_init(smem_u32(&bs.k_read[tid]), groups);
-        if (tid == 0) {
-            bs.abort_flag = 0;
-            bs.first_beyond = r.h1 - r.h0;
-            mbar_init(smem_u32(&bs.pushed), 1);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_async_smem();
-        if (tid == 0 && nblk > 1) mbar_expect_tx(smem_u32(&bs.pushed), nblk * ((chunks - rank + nblk - 1) / nblk) * CHUNK_BYTES);
-        if (tid < r.nx) mbar_arrive(smem_u32(&bs.full[tid]));         // filled by this block itself, ahead of the main loop
-    }
-    if (tid < MASK_HALVES) bs.seen[tid] = 0u;
-    if (tid < MAX_QROWS) bs.fld[tid] = tid < M ? (uint8_t)((m0 + tid) / p.group) : (uint8_t)0xff;
-    __syncthreads();
-    // (the barrier of the partials is there: the other blocks may send once they have seen this)
-    if (nblk > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-    volatile int* abortp = &bs.abort_flag;
+    const int chunks = M * (D / 16), slots = (int)by_nblk((uint32_t)(chunks + nblk - 1));     // chunks of the result, of one block at most
+    r.nx = app && rank == 0 ? (A + SROWS - 1) / SROWS : 0;
     const uint32_t full0 = smem_u32(bs.full), ring0 = smem_u32(ring);
     auto request_rows = [&](int row0, int st, int n) {     // one thread: the copies of a stage, the n-th to use slot st
         const uint32_t bar = full0 + 8 * st, dst = ring0 + (uint32_t)st * STAGE_BYTES;
@@ -338,75 +334,113 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
         __threadfence_block();
         *(volatile int*)&bs.asked[st] = n;
     };
-    // The first stages (warp w requests w, w + NW, ..): those of the prefix right away, so that they are on their way while
-    // the rest is set up; stages fb1.. may hold rows beyond the prefix and wait for the kernel ahead.
-    int fb1 = r.nx + r.p0 - r.h0;
+    // The first stages: those of the prefix right away, by warp 0; stages fb1.. may hold rows beyond the prefix and wait for the kernel ahead.
+    int fb1 = r.nx + r.p0 - r.h0, first0 = 0;              // lane: first KV row of part h0 + lane
     if (!Math::PREFIX_FIRST) {                             // (any order of the list is served)
         const int pos = r.h0 + lane;
-        const unsigned beyond = __ballot_sync(0xffffffffu, pos < r.p0 && r.tiles[pos / PARTS] * FDC_TILE_ROWS + pos % PARTS * SROWS + SROWS > p.P);
+        first0 = pos < r.p0 ? list_row0<SROWS>(r, pos) : 0;
+        const unsigned beyond = __ballot_sync(0xffffffffu, pos < r.p0 && first0 + SROWS > p.P);
         if (beyond) fb1 = r.nx + __ffs(beyond) - 1;
     }
-    if (lane == 0)
-        for (int it = warp; it < nstage && it < fb1; it += NW)
-            if (it >= r.nx) {
-                const int pos = r.h0 + it - r.nx;
-                request_rows((Math::PREFIX_FIRST ? pos / PARTS : r.tiles[pos / PARTS]) * FDC_TILE_ROWS + pos % PARTS * SROWS, it, 1);
+    if (warp == 0) {
+        const int ask = nstage < fb1 ? nstage : fb1;
+        if (lane < nstage) {
+            bs.used[lane] = 0;
+            bs.asked[lane] = lane < r.nx ? 1 : 0;
+            mbar_init(full0 + 8 * lane, 1);
+            if (Math::K_REUSED) mbar_init(smem_u32(&bs.k_read[lane]), groups);
+            if (lane == 0) {
+                bs.abort_flag = 0;
+                mbar_init(smem_u32(&bs.pushed), 1);
             }
-    __syncwarp();
-    bool off_list = false;
-    int beyond = 0x7fffffff;                               // first part of this thread's that reaches beyond the prefix
-    for (int i = tid; i < r.h1 - r.h0; i += THREADS) {
-        const int pos = r.h0 + i, row0 = list_row0<SROWS>(r, pos);
-        if (i < ROW0S) bs.row0[i] = row0;
-        if (row0 + SROWS > p.P && beyond == 0x7fffffff) beyond = i;
-        off_list |= pos < PARTS * (p.P / FDC_TILE_ROWS) && row0 != pos * SROWS;
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+            fence_async_smem();
+            if (lane == 0 && nblk > 1) mbar_expect_tx(smem_u32(&bs.pushed), nblk * (int)by_nblk((uint32_t)(chunks - rank + nblk - 1)) * CHUNK_BYTES);
+            if (lane < r.nx) mbar_arrive(full0 + 8 * lane);               // filled by this block itself, ahead of the main loop
+        }
+        __syncwarp();
+        const int from = Math::PREFIX_FIRST ? (r.h0 + lane - r.nx) * SROWS : __shfl_sync(0xffffffffu, first0, lane >= r.nx ? lane - r.nx : 0);
+        if (lane >= r.nx && lane < ask) request_rows(from, lane, 1);
+        __syncwarp();
     }
-    if (beyond != 0x7fffffff) atomicMin(&bs.first_beyond, beyond);
+    // (the barrier of the partials is there, made known by the fence: the other blocks may send once they have seen all of this arrive)
+    if (nblk > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+    volatile int* abortp = &bs.abort_flag;
+    bool off_list = false;
+    {
+        int beyond = 0x7fffffff;                           // first part of this thread's that reaches beyond the prefix
+        for (int i = tid; i < r.h1 - r.h0; i += THREADS) {
+            const int pos = r.h0 + i, row0 = list_row0<SROWS>(r, pos);
+            if (i < ROW0S) bs.row0[i] = row0;
+            if (row0 + SROWS > p.P && beyond == 0x7fffffff) beyond = i;
+            off_list |= pos < PARTS * whole && row0 != pos * SROWS;
+        }
+        beyond = __reduce_min_sync(0xffffffffu, beyond);
+        if (lane == 0) bs.beyond[warp] = beyond;
+    }
+    if (tid < MAX_QROWS) bs.fld[tid] = tid < M ? (uint8_t)div_by((uint32_t)(m0 + tid), ca.by_group) : (uint8_t)0xff;
+    // Visibility of the run's parts from position p0 on: a warp per part (from the last warp down: warp 0 has the barriers), a lane per
+    // field.  Fused append: the new rows count as unseen there (their values come from the stage of new rows).
+    auto written = [&](int row) { return row >= p.P && row < p.rows; };
     auto cache_bits = [&]() {
-        for (int i = tid; i < r.np * A; i += THREADS) {
-            const int h = i / A, b = i - h * A;
-            const uint32_t x = part_bits<SROWS>(r.mask + (size_t)b * p.W, p.W, p.P, list_row0<SROWS>(r, r.p0 + h));
-            bs.bits[i] = x;
-            if (x) atomicOr(&bs.seen[h], x);
+        for (int h = NW - 1 - warp; h < r.np; h += NW) {
+            const int row0 = list_row0<SROWS>(r, r.p0 + h);
+            uint32_t x[2] = {0u, 0u}, fresh = 0u;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int b = lane + 32 * j, i = ar[j] - row0;
+                if (b < A) {
+                    x[j] = part_bits<SROWS>(r.mask + (size_t)b * p.W, p.W, p.P, row0);
+                    if (written(ar[j]) && i >= 0 && i < SROWS) fresh |= 1u << i;
+                }
+            }
+            if (app) fresh = __reduce_or_sync(0xffffffffu, fresh);
+            const uint32_t any = __reduce_or_sync(0xffffffffu, x[0] | x[1]);
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (lane + 32 * j < A) bs.bits[h * A + lane + 32 * j] = x[j] & ~fresh;
+            if (lane == 0) {
+                bs.seen[h] = any & ~fresh;
+                bs.holds[h] = any != 0u;               // (the new rows' numbers may still change)
+            }
         }
     };
-    // Fused append, from the new rows' places (bs.app_row): which of them every field sees, and their rows
-    // taken out of the tables of the cache's tile parts.
+    // ... and which of the new rows every field sees (block 0)
     auto new_bits = [&]() {
-        for (int i = tid; i < r.np * A; i += THREADS) {
-            const int h = i / A, b = i - h * A, x = bs.app_row[b] - part_row0<SROWS>(r, bs, r.p0 + h);
-            if (x >= 0 && x < SROWS) {
-                atomicAnd(&bs.seen[h], ~(1u << x));
-                for (int b2 = 0; b2 < A; ++b2) atomicAnd(&bs.bits[h * A + b2], ~(1u << x));
-            }
-        }
         for (int i = warp; i < r.nx * A; i += NW) {
-            const int x = i / A, b = i - x * A, j = x * SROWS + lane;
-            const int ar = j < A ? bs.app_row[j] : -1, t = ar - p.P;
-            const bool on = ar >= 0 && (t >> 6) < p.W && ((r.mask[(size_t)b * p.W + (t >> 6)] >> (t & 63)) & 1ull);
+            static_assert(!Math::FUSES || SROWS == 32, "a lane's two fields are in two stages");
+            const int x = i >= A ? 1 : 0, b = i - x * A, row = x * 32 + lane < A ? (x ? ar[1] : ar[0]) : -1, t = row - p.P;
+            const bool on = written(row) && (t >> 6) < p.W && ((r.mask[(size_t)b * p.W + (t >> 6)] >> (t & 63)) & 1ull);
             const uint32_t bits = __ballot_sync(0xffffffffu, on);
             if (lane == 0) bs.newbits[x * FDC_MAX_NODES + b] = bits;
         }
+        if (warp == NW - 1)
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+                if (lane + 32 * j < A) bs.app_row[lane + 32 * j] = written(ar[j]) ? ar[j] : -1;
     };
-    if (tid < A) bs.app_row[tid] = ar0 >= p.P && ar0 < p.rows ? ar0 : -1;
     cache_bits();
+    if (app) new_bits();
     __syncthreads();
-    if (warp == 0) {
-        // the parts that hold a visible row, in order
+    // The parts that hold a visible row, in order (every warp makes the whole list: the same values).
+    auto keep_parts = [&]() {
         int n = 0;
         for (int h0 = 0; h0 < r.np; h0 += 32) {
-            const bool keep = h0 + lane < r.np && bs.seen[h0 + lane] != 0u;
+            const bool keep = h0 + lane < r.np && bs.holds[h0 + lane] != 0;
             const uint32_t ball = __ballot_sync(0xffffffffu, keep);
             if (keep) bs.kept[n + __popc(ball & ((1u << lane) - 1u))] = (uint8_t)(h0 + lane);
             n += __popc(ball);
         }
-        if (lane == 0) bs.n_kept = n;
-    }
-    __syncthreads();
-    if (p.app_row) new_bits();                             // (read after the block's next barrier)
-    r.total = r.nx + (r.h1 - r.h0) - (r.np - bs.n_kept);
+        __syncwarp();
+        return n;
+    };
+    r.n_kept = keep_parts();
+    int first_beyond = lane < NW ? bs.beyond[lane] : 0x7fffffff;
+    first_beyond = __reduce_min_sync(0xffffffffu, first_beyond);
+    if (first_beyond > r.h1 - r.h0) first_beyond = r.h1 - r.h0;
+    r.total = r.nx + (r.h1 - r.h0) - (r.np - r.n_kept);
     // stages fb.. may hold rows beyond the prefix (parts ahead of p0 are never left out)
-    const int fb = r.nx + (bs.first_beyond < r.p0 - r.h0 ? bs.first_beyond : r.p0 - r.h0);
+    const int fb = r.nx + (first_beyond < r.p0 - r.h0 ? first_beyond : r.p0 - r.h0);
     auto request = [&](int it, int st, int n) { request_rows(part_row0<SROWS>(r, bs, stage_pos(r, bs, it)), st, n); };
     if (p.early) {
         // The queries and the new rows may still be written by the kernel ahead: their lines are only requested into L2
@@ -423,18 +457,18 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
             }
         asm volatile("griddepcontrol.wait;" ::: "memory");
     }
+    // queries of the pair: row m = field * group + head-in-group; rows M.. up to a whole group are zero
+    for (int i = tid; i < (M + GROWS - 1) / GROWS * GROWS * (D / CHUNK); i += THREADS) {
+        const int m = i / (D / CHUNK), dc = i - m * (D / CHUNK);
+        const int b = m < M ? (int)bs.fld[m] : 0, hg = m < M ? m0 + m - b * p.group : 0;
+        cp_async16(qs + Math::q_off(qrows, m, dc),
+                   reinterpret_cast<const uint4*>(p.q) + ((((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * D) / CHUNK + dc, m < M);
+    }
     if (lane == 0) {
         for (int it = warp; it < nstage && it < r.total; it += NW)
             if (it >= fb1) request(it, it, 1);
     }
     __syncwarp();
-    // queries of the pair: row m = field * group + head-in-group; rows M.. up to a whole group are zero
-    for (int i = tid; i < (M + GROWS - 1) / GROWS * GROWS * (D / CHUNK); i += THREADS) {
-        const int m = i / (D / CHUNK), dc = i - m * (D / CHUNK);
-        const int b = m < M ? (m0 + m) / p.group : 0, hg = m < M ? m0 + m - b * p.group : 0;
-        cp_async16(qs + Math::q_off(qrows, m, dc),
-                   reinterpret_cast<const uint4*>(p.q) + ((((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * D) / CHUNK + dc, m < M);
-    }
     // the stages of new rows: row i of stage x = the new vectors of field 32 x + i (rows past the last field: zero)
     for (int i = tid; i < r.nx * SROWS * (D / CHUNK); i += THREADS) {
         const int b = i / (D / CHUNK), dc = i - b * (D / CHUNK);
@@ -446,21 +480,21 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     // (kernels for other caches have never asked for the prefix tiles to come first)
     if (Math::PREFIX_FIRST && off_list) atomicOr(p.status, FDC_DEV_TILE_LIST);
     int moved = 0;
-    if (p.app_row && tid < A) {
-        const int ar = __ldcg(p.app_row + (size_t)s * p.max_active + tid);
-        if ((ar < p.P || ar >= p.rows) && cluster == s * p.hkv * qsplit && rank == 0) atomicOr(p.status, FDC_DEV_ROW_RANGE);     // skipped and flagged
-        moved = ar != ar0;
-        ar0 = ar;
+    if (app) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (lane + 32 * j < A) {
+                const int now = __ldcg(app + lane + 32 * j);
+                if (!written(now) && warp == 0 && blockIdx.x == 0) atomicOr(p.status, FDC_DEV_ROW_RANGE);     // skipped and flagged
+                moved |= now != ar[j];
+                ar[j] = now;
+            }
     }
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-    fence_async_smem();                                    // (the next copy into the new rows' slots goes through the asynchronous proxy)
+    if (r.nx) fence_async_smem();                          // (the next copy into the new rows' slots goes through the asynchronous proxy)
     if (__syncthreads_or(moved)) {
         // the row numbers were written by the kernel ahead: the tables once more
-        if (tid < A) bs.app_row[tid] = ar0 >= p.P && ar0 < p.rows ? ar0 : -1;
-        if (tid < MASK_HALVES) bs.seen[tid] = 0u;
-        __syncthreads();
         cache_bits();
-        __syncthreads();
         new_bits();
         __syncthreads();
     }
@@ -551,19 +585,18 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     __syncthreads();
     auto store_out = [&](int mm, int c4, const float4& acc, float lt) {
         const float inv = 1.f / lt;
-        const int b = (m0 + mm) / p.group, hg = m0 + mm - b * p.group;
+        const int b = bs.fld[mm], hg = m0 + mm - b * p.group;
         Math::store(reinterpret_cast<typename Math::Elem*>(p.out) + (((size_t)s * p.max_active + b) * p.hq + (size_t)g * p.group + hg) * D + c4,
                     make_float4(acc.x * inv, acc.y * inv, acc.z * inv, acc.w * inv));
     };
     // block: merge over the warps of a group; with one block per pair that is the result, else it is sent to the chunk's block
     if (nblk > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");       // (long complete: all blocks have set up their barriers)
     const uint32_t recv0 = smem_u32(recv), recv_ml0 = recv0 + (uint32_t)(nblk * slots * 64), pushed = smem_u32(&bs.pushed);
-    const uint32_t by_nblk = 65536u / (uint32_t)nblk + 1u;                                  // k / nblk for k < 4096 by a multiplication
     merge_lanes<Math>(lanes, tid, M, groups * GROWS, bs.wml, part, [&](int mm, int c4, float mx, float lt, const float4& acc) {
         if (nblk == 1) {
             store_out(mm, c4, acc, lt);
         } else {
-            const uint32_t k = (uint32_t)(mm * (D / 16) + (c4 >> 4)), slot = (k * by_nblk) >> 16, owner = k - slot * (uint32_t)nblk;
+            const uint32_t k = (uint32_t)(mm * (D / 16) + (c4 >> 4)), slot = by_nblk(k), owner = k - slot * (uint32_t)nblk;
             const uint32_t at = (uint32_t)(rank * slots) + slot, bar = map_rank(pushed, owner);
             st_async4(map_rank(recv0 + at * 64 + (uint32_t)(c4 & 15) * 4, owner), bar, acc);
             if ((c4 & 15) == 0) st_async2(map_rank(recv_ml0 + at * 8, owner), bar, make_float2(mx, lt));
@@ -572,11 +605,11 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     // fused append: the new rows whose tile parts are in this block's run go to the cache (this block's copies
     // from there have landed; clusters with the pair's other query rows may still be reading the
     // part, but to them, too, the row counts as unseen: its bytes there do not matter)
-    if (Math::FUSES && p.app_row && m0 == 0 && bs.first_beyond < r.h1 - r.h0)
+    if (Math::FUSES && p.app_row && m0 == 0 && first_beyond < r.h1 - r.h0)
         for (int b = warp; b < A; b += NW) {
             const int ar = bs.app_row[b];
             bool here = false;
-            for (int i = bs.first_beyond + lane; i < r.h1 - r.h0; i += 32) {
+            for (int i = first_beyond + lane; i < r.h1 - r.h0; i += 32) {
                 const int x = ar - part_row0<SROWS>(r, bs, r.h0 + i);
                 here |= x >= 0 && x < SROWS;
             }
@@ -596,7 +629,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
         // Four threads per item (4 columns), each with every fourth block (at most four), summed by shuffles.
         const float4* ro = reinterpret_cast<const float4*>(recv);
         const float2* rml = reinterpret_cast<const float2*>(recv + (size_t)nblk * slots * 64);
-        const int q = tid & 3, items = (chunks - rank + nblk - 1) / nblk * 4;
+        const int q = tid & 3, items = (int)by_nblk((uint32_t)(chunks - rank + nblk - 1)) * 4;
         for (int i = tid >> 2; __any_sync(0xffffffffu, i < items); i += THREADS / 4) {
             const bool on = i < items;
             const int slot = on ? i >> 2 : 0, k = slot * nblk + rank, mm = k / (D / 16), c4 = (k - mm * (D / 16)) * 16 + (i & 3) * 4;
@@ -723,8 +756,9 @@ int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const Cluste
         return cluster_placeable(reinterpret_cast<const void*>(kernel), one, n, h.per_sm > 1, known);
     });
     at[1].val.clusterDim.x = (unsigned)nblk;
-    cfg.gridDim = dim3((unsigned)((long long)p.batch * p.hkv * h.qsplit * nblk));
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, tk, tv, nstage, nblk, h.qsplit, qrows);
+    cfg.gridDim = dim3((unsigned)(p.hkv * h.qsplit * nblk), (unsigned)p.batch);
+    const ClusterArgs args{nstage, nblk, h.qsplit, qrows, div_inverse(nblk), div_inverse(h.qsplit), div_inverse(p.group)};
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, tk, tv, args);
     if (e != cudaSuccess) return set_cuda_error(e);
     note_launch();
     return FDC_OK;

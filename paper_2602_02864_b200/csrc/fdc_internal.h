@@ -82,7 +82,22 @@ struct ClusterProblem {
 // to twice as many.  us a layer, half / full: fp32, 14/2 heads x 64, 9 fields, 4 scenes, prefix 3000, the last field 45.6 / 35.2; 4/2 x 64, 24
 // fields, 8 scenes, prefix 2048, the last field 56.9 / 39.3; bf16, 50 pairs of 50 rows x 64, prefix 2215 43.0 / 37.7; 4 pairs of 112 rows x 128, prefix
 // 707 12.9 / 11.6.  What it gained was less: fp32, 32/8 x 128, six fields at work, 8 scenes, prefix 2048 75.7 / 79.5.
-FDC_HD int run_begin(int rank, int nblk, int parts) { return (int)((long long)rank * parts / nblk); }
+// (= rank * parts / nblk; `div(x)` is x / nblk, which the kernels do without a division)
+template <class Div>
+FDC_HD int run_begin(int rank, int nblk, int parts, Div&& div)
+{
+    const int each = (int)div((uint32_t)parts);
+    return rank * each + (int)div((uint32_t)(rank * (parts - each * nblk)));
+}
+FDC_HD int run_begin(int rank, int nblk, int parts)
+{
+    return run_begin(rank, nblk, parts, [nblk](uint32_t x) { return x / (uint32_t)nblk; });
+}
+// Division of x < 2^28 by a small n (1 to 16) or of x < 2^24 by any n < 256: div_by(x, div_inverse(n)) = x / n.
+inline uint32_t div_inverse(int n) { return n > 1 ? (uint32_t)((1ull << 32) / (uint32_t)n + 1) : 0u; }
+#ifdef __CUDACC__
+__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t inverse) { return inverse ? __umulhi(x, inverse) : x; }
+#endif
 ClusterShape pick_cluster(const ClusterProblem& c, float* us);      // us (may be NULL): the estimated time
 bool route_problem(const ClusterProblem& c, ClusterShape* cut);     // the cut, and whether the cluster kernel is the one to take (head_dim 64: always)
 int cluster_ring(int head_dim, int rows, int nblk, int per_sm);     // stages of a block's ring (bf16); 0: no room for the partials beside it
