@@ -2,14 +2,28 @@
 // group of softmax warps), and the entry points that choose between the builds.
 #define FDC_TC_NGRP 1
 #define FDC_TC_NPMAX 32
+#define FDC_TC_TWO 0
 #define FDC_TC_KERNEL attn_tc_kernel
 #define FDC_TC_LAUNCH launch_tc_np32
 #include "fdc_attn_tc_kernel.cuh"
 
 namespace fdc {
 
-int launch_tc_np64(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);    // fdc_attn_tc_g2.cu
-int launch_tc_rows(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);    // fdc_attn_tc_rows.cu
+int launch_tc_np64(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);        // fdc_attn_tc_g2.cu
+int launch_tc_rows(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);        // fdc_attn_tc_rows.cu
+int launch_tc_np64_two(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);    // fdc_attn_tc_g2_two.cu
+int launch_tc_rows_two(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);    // fdc_attn_tc_rows_two.cu
+
+// Launches whose pairs come in two parts each, one per CTA, as long as no scene has ended, go to builds of their own (parts that are spread over the
+// pair's list, and that hand each other half of their results): with more than 32 query rows, from 32 tiles a pair on and while the shares are short enough
+// for one part per CTA (see SplitFinder).  us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, 140 tiles 59.1 / 56.6.  With
+// 16 tiles a pair the start of the CTAs two by two costs more than that gains (64 pairs, 35 rows 21.7 / 23.7), with equal shares nothing is
+// handed over (128 rows, 544 tiles 213.3 / 216.0).
+static bool pairs_in_two_parts(const AttnParams& p)
+{
+    const long long pairs = (long long)p.batch * p.hkv;
+    return p.pair_cnt && p.n_cta % 2 == 0 && 2 * pairs <= p.n_cta && 3 * pairs > p.n_cta && p.ntile_max >= 32 && p.ntile_max * pairs < (p.mmax > 64 ? 100 : 200) * (long long)p.n_cta;
+}
 
 // More than 64 query rows go to the row form.  Measured on both sides of the line (us a layer, transposed / row
 // form): 128 rows, 8 scenes, prefix 1024 / 4096 / 32768: 56.6 / 40.7, 90.8 / 61.1, 336 / 212; 84 rows, 8 scenes, prefix
@@ -17,6 +31,10 @@ int launch_tc_rows(const AttnParams& p, int head_dim, cudaStream_t st, int split
 // scenes, prefix 4096: 53.3 / 59.5; 16 rows, 64 scenes, prefix 16384: 629 / 732.
 static int launch_tc(const AttnParams& p, int head_dim, cudaStream_t st, int split_only)
 {
+    if (p.mmax > 32 && pairs_in_two_parts(p)) {
+        const int rc = p.mmax > 64 ? launch_tc_rows_two(p, head_dim, st, split_only) : launch_tc_np64_two(p, head_dim, st, split_only);
+        if (rc != FDC_ERR_SHAPE) return rc;
+    }
     if (p.mmax > 64) return launch_tc_rows(p, head_dim, st, split_only);
     if (p.mmax > 32) return launch_tc_np64(p, head_dim, st, split_only);
     return launch_tc_np32(p, head_dim, st, split_only);

@@ -1,8 +1,8 @@
 // Split-KV pass for bf16 caches (head_dim 128) on the 5th-generation tensor cores (tcgen05 + TMEM).
-// This file is the whole kernel and its launcher, for pairs of up to 64 query rows; it is compiled twice, by the two translation
+// This file is the whole kernel and its launcher, for pairs of up to 64 query rows; it is compiled by the translation
 // units that include it with FDC_TC_NGRP = 1 and 2 (the number of groups the softmax warps work
-// in, see softmax_segment), so that each build holds only its own inner loop and gets its own
-// register allocation.
+// in, see softmax_segment), and for two groups once more with FDC_TC_TWO (pairs in two parts, fdc_tc_common.cuh), so that each
+// build holds only its own inner loop and gets its own register allocation.
 //
 // Sec. 3.3: the queries of all parallel fields of a scene, times the GQA heads of a KV head,
 // share ONE read of the KV rows.  The kernel is written in the transposed form, with the KV
@@ -37,7 +37,7 @@
 // flagged.  Sums and accumulator use the same reference and the same rounded P^T, so the result
 // is exact up to the rounding of P^T.
 #if !defined(FDC_TC_NGRP) || !defined(FDC_TC_NPMAX)
-#error "include from a translation unit that defines FDC_TC_NGRP (1 or 2), FDC_TC_NPMAX (32 or 64), FDC_TC_KERNEL and FDC_TC_LAUNCH"
+#error "include from a translation unit that defines FDC_TC_NGRP (1 or 2), FDC_TC_NPMAX (32 or 64), FDC_TC_TWO (0 or 1), FDC_TC_KERNEL and FDC_TC_LAUNCH"
 #endif
 #include "fdc_tc_common.cuh"
 
@@ -143,6 +143,7 @@ struct Ctx : Split {
     __device__ __forceinline__ uint32_t q_ready() const { return bar0 + 32 * MAXST + 96; }
     __device__ __forceinline__ uint32_t o_free() const { return bar0 + 32 * MAXST + 104; }
     __device__ __forceinline__ uint32_t app_done() const { return bar0 + 32 * MAXST + 112; }
+    __device__ __forceinline__ uint32_t peer_done() const { return bar0 + 32 * MAXST + 120; }
     int ns, s_stride;                // S^T buffers in TMEM (4 of 64 columns) and their distance
     uint32_t tmem;
     unsigned char *kring, *vring, *qs, *ps, *ones;
@@ -695,7 +696,11 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, const Ctx& 
     int t = 0;                                    // round within the segment
     for (int jb = 0; jb < ntile; jb += 32) {
         const int jn = ntile - jb < 32 ? ntile - jb : 32;
+#if FDC_TC_TWO
+        const int my_tile = lane < jn ? p.tiles[(size_t)sg.s * p.ntile_max + tile_entry(sg, jb + lane)] : 0;
+#else                                             // (the same thing; by way of tile_entry the build for 32 rows spills)
         const int my_tile = lane < jn ? p.tiles[(size_t)sg.s * p.ntile_max + sg.j0 + jb + lane] : 0;
+#endif
         for (int k = 0; k < jn; k += 2, ++g, ++t) {
             const int nt = jn - k < 2 ? 1 : 2;
             const uint32_t b = g & 1;
@@ -851,7 +856,7 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, const Ctx& 
 #pragma unroll
                 for (int i = 0; i < 4; ++i) st4 |= (none || ((seen >> (16 * i)) & 0xffffull)) ? (1u << i) : 0u;
                 // the whole tiles of the prefix come first in a tile list (entry j = tile j): the producer relies on it
-                if (col0r == 0 && (q4 & 1) == 0 && lane == 0 && sg.j0 + jb + k + ti < p.P / TILE) atomicOr(p.status, FDC_DEV_TILE_LIST);
+                if (col0r == 0 && (q4 & 1) == 0 && lane == 0 && tile_entry(sg, jb + k + ti) < p.P / TILE) atomicOr(p.status, FDC_DEV_TILE_LIST);
             }
             if (col0r == 0 && (q4 & 1) == 0 && lane == 0) cx.v_steps[b * 2 + ti] = (int)st4;
             if (++vst == cx.nv) {
@@ -915,6 +920,7 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, const Ctx& 
     const int pair = sg.s * p.hkv + sg.g;
     const int slot = blockIdx.x + pair;
     const bool whole = sg.j0 == 0 && sg.j1 == sg.nt;       // this CTA saw every tile of the pair
+    if (TWO && half_of_pair(cx, sg, p.hkv) >= 0) return;   // (one part a CTA: the run's only segment; finish_in_two)
     if (p.pair_cnt && whole) {
         // no other partial exists: normalise and write the output directly
         if (tid < np) cx.alpha[tid] = 1.f / ((cx.lred[tid] + cx.lred[128 + tid]) + (cx.lred[256 + tid] + cx.lred[384 + tid]));
@@ -983,6 +989,78 @@ __device__ __forceinline__ void softmax_segment(const AttnParams& p, const Ctx& 
     tc_fence_before();
     __syncwarp();
     if (!dead && lane == 0) mbar_arrive(cx.o_free());
+}
+
+// The end of a CTA that has one part of a pair in two (half_of_pair; all softmax warps; the partial sums are in lred).  Half 0 finishes the pair's query columns of
+// column parts 0 and 1, half 1 those of 2 and 3, each with what the other CTA hands over through the workspace.
+__device__ __forceinline__ void finish_in_two(const AttnParams& p, const Ctx& cx, const Segment& sg, const int nph, const int half, const bool dead, const int warp, const int lane)
+{
+    const int tid = threadIdx.x, q4 = warp & 3, part = warp >> 2, krow = q4 * 32 + lane;
+    const int nch = nph >> 3, col0 = part * nph, G = p.group, M = cx.nact[sg.s] * G;
+    const uint32_t o_addr = cx.tmem + ((uint32_t)(q4 * 32) << 16) + TM_O + col0;
+    const size_t slot = blockIdx.x + sg.s * p.hkv + sg.g, peer = half ? slot - 1 : slot + 1;
+    const bool mine = part >> 1 == half;
+    float m = -INFINITY, l = 0.f;                          // (thread = query column)
+    if (tid < M) {
+        const float mn = cx.mneg[tid];
+        m = mn == UNSET ? -INFINITY : -mn;
+        l = (cx.lred[tid] + cx.lred[128 + tid]) + (cx.lred[256 + tid] + cx.lred[384 + tid]);
+        if (!dead) *reinterpret_cast<float2*>(p.ws_ml + (slot * p.mmax + tid) * 2) = make_float2(m, l);
+    }
+    if (!mine && !dead) {
+        // O^T: lane = head_dim index, column = query row; partials are stored [query row][head_dim]
+        float* wo = p.ws_o + slot * p.mmax * D + krow;
+#pragma unroll 1
+        for (int ch = 0; ch < nch; ++ch) {
+            uint32_t ov[8];
+            tmem_ld<8>(o_addr + ch * 8, ov);
+            tmem_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (col0 + ch * 8 + i < M) wo[(size_t)(col0 + ch * 8 + i) * D] = __uint_as_float(ov[i]);
+        }
+    }
+    __threadfence();
+    soft_sync();
+    if (tid == 0 && !dead) arrive_at_peer(cx.peer_done());
+    const bool ok = !dead && wait_for_peer(cx.peer_done(), cx.abortp, p.status);         // (else: flagged, no output)
+    // the other CTA's values of this thread's columns, all on their way before the first is used
+    constexpr int PER = NP_MAX / NPART;
+    float z[PER];
+    const float* po = p.ws_o + peer * p.mmax * D + krow;
+    if (mine && ok)
+#pragma unroll
+        for (int i = 0; i < PER; ++i) z[i] = i < nph && col0 + i < M ? __ldcg(po + (size_t)(col0 + i) * D) : 0.f;
+    if (tid < M && ok) {
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(p.ws_ml + (peer * p.mmax + tid) * 2));
+        const float nm = fmaxf(m, v.x), ms = nm == -INFINITY ? 0.f : nm, a = fast_exp2(m - ms), w = fast_exp2(v.x - ms);      // (a part that saw nothing: 0)
+        const float inv = 1.f / fmaf(v.y, w, l * a);
+        cx.alpha[tid] = a * inv;
+        cx.lred[tid] = w * inv;
+    }
+    soft_sync();
+    if (mine && ok) {
+        __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out);
+#pragma unroll
+        for (int ch = 0; ch < PER / 8; ++ch)
+            if (ch < nch) {
+                uint32_t ov[8];
+                tmem_ld<8>(o_addr + ch * 8, ov);
+                tmem_wait_ld();
+                int b = (col0 + ch * 8) / G, hg = (col0 + ch * 8) - b * G;
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int n = col0 + ch * 8 + i;
+                    if (n < M)
+                        out[(((size_t)sg.s * p.max_active + b) * p.hq + (size_t)sg.g * G + hg) * D + krow] =
+                            __float2bfloat16_rn(fmaf(z[ch * 8 + i], cx.lred[n], __uint_as_float(ov[i]) * cx.alpha[n]));
+                    if (++hg == G) {
+                        hg = 0;
+                        ++b;
+                    }
+                }
+            }
+    }
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -1058,6 +1136,7 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
         mbar_init(cx.q_ready(), NSOFT);
         mbar_init(cx.o_free(), NSOFT);
         mbar_init(cx.app_done(), 1);
+        if (TWO) mbar_init(cx.peer_done(), 1);
         mbar_init(smem_u32(&cta_flags.raise_bar), NSOFT);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
@@ -1069,6 +1148,7 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
     }
     tc_fence_before();
     __syncthreads();
+    if (TWO) cluster_arrive();
     tc_fence_after();
     const uint32_t tmem = split_only ? 0u : *reinterpret_cast<volatile uint32_t*>(tmem_holder);
     cx.tmem = tmem;
@@ -1086,6 +1166,7 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
     if (!p.early) split.issue(p);
     long long lo = 0, hi = 0;
     bool active = split.find(p, cx, split_only, lo, hi);
+    if (TWO) cluster_wait();
     // Two roles run ahead of the dependency wait (with p.early): the TMA producer, which takes the wait
     // itself once nothing more of the prefix can be requested, and the softmax warps, which first stage
     // the first pair's bitmaps.
@@ -1122,6 +1203,12 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
             ++seg;
             u = sg.next_u;
         }
+        if (TWO) {
+            s = 0;
+            const Segment sg = decode_segment(lo, hi, cx.pre, p.hkv, s);
+            const int half = half_of_pair(cx, sg, p.hkv);
+            if (half >= 0) finish_in_two(p, cx, sg, ((NP_MAX == 32 || cx.nact[sg.s] * p.group <= 32) ? 32 : 64) / NPART, half, dead, warp, lane);
+        }
     }
     // ---- teardown: everybody is done with TMEM before it is freed
     tc_fence_before();
@@ -1135,6 +1222,10 @@ FDC_TC_KERNEL(const AttnParams p, const __grid_constant__ CUtensorMap tm_k, cons
             for (int i = 0; i < 100; ++i) __nanosleep(1000);
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+    }
+    if (TWO) {
+        cluster_arrive();
+        cluster_wait();
     }
 }
 
@@ -1153,16 +1244,22 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     const int p_buf = ((np_max + 63) / 64) * PANEL;
     if (np_max != NP_MAX) return FDC_ERR_SHAPE;   // another build's launches
     const int npb = 2;
+    int rc = FDC_OK;
     const size_t fixed = 1024 + (size_t)npb * p_buf + (size_t)(D / 64) * np_max * 128 + ONES_BYTES + 8 * (5 * MAXST + 16) + 16 +
                          4 * (128 + 128 + 512 + 128 + 12) + sizeof(int) * (3 * p.batch + 2) + 8 * (2 * MBUF + 2 * UW + 2) + 64;
     int stages = (int)((227 * 1024 - 256 - fixed) / STAGE);
     if (stages > 2 * MAXST) stages = 2 * MAXST;
     if (stages < 4) return FDC_ERR_SHAPE;
+    if (TWO) {
+        static PairsPlaceable placeable;
+        rc = placeable.all(reinterpret_cast<const void*>(FDC_TC_KERNEL), THREADS, fixed + (size_t)stages * STAGE, p.n_cta);
+        if (rc) return rc;
+    }
     if (split_only) stages = 0;
     const int nk = stages / 2, nv = stages - nk;
     const size_t smem = fixed + (size_t)stages * STAGE;
     alignas(64) CUtensorMap tk, tv;
-    int rc = get_kv_tensor_map(p.k, p, FDC_BF16, D, TILE, &tk);
+    rc = get_kv_tensor_map(p.k, p, FDC_BF16, D, TILE, &tk);
     if (rc) return rc;
     rc = get_kv_tensor_map(p.v, p, FDC_BF16, D, TILE, &tv);
     if (rc) return rc;
@@ -1175,11 +1272,12 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
         cfg.blockDim = dim3(THREADS);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
-        cudaLaunchAttribute at[1];
+        cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = at;
         cfg.numAttrs = split_only ? 0 : 1;
+        if (TWO && !split_only) at[cfg.numAttrs++] = cluster_of_two();
         cudaError_t e = cudaLaunchKernelEx(&cfg, FDC_TC_KERNEL, p, tk, tv, nk, nv, split_only);
         if (e != cudaSuccess) return set_cuda_error(e);
     }

@@ -269,8 +269,9 @@ struct ClusterArgs {
 // it is a chain of trips to memory (counts -> tile list -> bitmaps), fences and, more than both, of instructions that are fetched for one
 // execution.  So: the barriers and the prefix's first stages are warp 0's alone, which needs no barrier of the block for it; the
 // other warps prepare the visibility meanwhile, a warp per tile part, a lane per field; one barrier of the block ends it; and
-// nothing is divided.  Cycles from the block's first instruction to its dependency wait, all warps going through every step with three barriers of the
-// block and a releasing arrival at the cluster's (1000 cycles by itself) / now: see the figures at launch_cluster.
+// nothing is divided.  From a block's first instruction to its dependency wait (traced): 3.3 us with all warps going through every step, three barriers of
+// the block and a releasing arrival at the cluster's (1000 cycles by itself), 2.1 us now.  us a layer: one scene, 28/4 heads x 128, six fields, prefix
+// 2048 9.9 / 8.8; one field, prefix 1024 6.2 / 5.8; 14/2 x 64, 41 scenes, prefix 281, one field left 14.1 / 12.2.
 template <class Math>
 __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUtensorMap& tm_k, const CUtensorMap& tm_v, const ClusterArgs& ca)
 {
@@ -300,8 +301,8 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     for (int j = 0; j < 2; ++j) ar[j] = app && lane + 32 * j < p.max_active ? app[lane + 32 * j] : -1;
     if (A * p.group <= m0 || nt <= 0) {
         // Nothing to do (all blocks of the cluster agree).  Such blocks leave at once: their places go to the next launch's blocks, which set
-        // themselves up meanwhile.  One block of the grid waits for the launch ahead, so that grids still complete in stream order.
-        // us a layer, all of them waiting / this: 3 scenes, 28/4 heads, one of five fields left, prefix 1000: 10.7 / 7.
+        // themselves up meanwhile (3 scenes, 28/4 heads, one of five fields left, 144 of 216 blocks idle: a launch's last blocks began 0.5 us before the launch ahead
+        // ended, now 15 us).  One block of the grid waits for the launch ahead, so that grids still complete in stream order.
         if (p.early && blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }

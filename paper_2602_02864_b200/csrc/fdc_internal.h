@@ -12,11 +12,13 @@
 // nothing else, before the pass's first attention launch) and kept here with the counts it was
 // computed from; the attention launches only check that the counts are unchanged.  Layout, in
 // int32: [0..15] header, [16..) n_active[FDC_MEMO_BATCH], tiles[FDC_MEMO_BATCH],
-// prev[FDC_MEMO_BATCH + 1], [FDC_MEMO_ENTRIES..) first and last unit of each CTA (2 x int64).
+// prev[FDC_MEMO_BATCH + 1], [FDC_MEMO_ENTRIES..) first and last unit of each CTA (2 x int64), [FDC_MEMO_SPREAD..) how each
+// CTA's part is spread over its pair's list (4 each).
 #define FDC_MEMO_BATCH 256
 #define FDC_MEMO_CTAS 256
 #define FDC_MEMO_ENTRIES 800
-#define FDC_MEMO_INTS (FDC_MEMO_ENTRIES + 4 * FDC_MEMO_CTAS)
+#define FDC_MEMO_SPREAD (FDC_MEMO_ENTRIES + 4 * FDC_MEMO_CTAS)
+#define FDC_MEMO_INTS (FDC_MEMO_SPREAD + 4 * FDC_MEMO_CTAS)
 
 namespace fdc {
 

@@ -5,6 +5,7 @@
 
 #include <cudaTypedefs.h>
 
+#include <atomic>
 #include <climits>
 
 #include "fdc_attn_common.cuh"
@@ -18,6 +19,10 @@ constexpr int TILE = FDC_TILE_ROWS;          // rows per entry of the visited-ti
 constexpr int W_PREFIX = 4;       // cost of a tile inside the prefix (the unit of the weighted work split is a quarter of it)
 constexpr int W_MASKED = 6;       // cost of a tile beyond the prefix (bitmap selects, V clean-up): measured about 1.5 prefix tiles
 constexpr int W_PAIR = 32;           // cost of finishing a (scene, KV head) pair (drain, partial write, next queries)
+#if !defined(FDC_TC_TWO)
+#error "FDC_TC_TWO: 1 for the build that launches whose pairs are cut in two parts are given (pairs_in_two_parts), else 0"
+#endif
+constexpr bool TWO = FDC_TC_TWO != 0;
 constexpr int UW = 64;                       // words of a scene's union bitmap kept in shared memory (when W <= UW)
 constexpr int MIN_TILES = 8;                 // tiles per CTA below which fewer CTAs are used (small problems)
 constexpr int MIN_UNITS = MIN_TILES * W_PREFIX;   // the same as a weighted length
@@ -136,6 +141,35 @@ __device__ __forceinline__ int tile_of_vt(const Split& cx, int nt, int r)
     const int j = r <= np * W_PREFIX ? (r + W_PREFIX - 1) / W_PREFIX : np + (r - np * W_PREFIX + W_MASKED - 1) / W_MASKED;
     return j > nt ? nt : j;
 }
+// Spread parts (the builds for pairs in two parts).  Where a pair is cut for one part per CTA and every part gets at least SPREAD tiles beyond the prefix, a part
+// has its share of the prefix AND its share of what lies beyond (the units of such a pair are counted part by part): all parts begin with tiles that
+// can be requested ahead of the dependency wait and that cover the append, which the tiles beyond the prefix wait for (a part of those alone idled for
+// 4.4 us), and they are equal whatever the two kinds of tile cost.  With fewer of them, and with many parts, a part's few masked tiles and two
+// roundings cost more than that (us a pass, one scene, prefix 18250, 126 rows beyond it, 18 parts of a pair: 606 without, 627 spread).
+// (In static shared memory: registers held for it cost the kernels that sit at their limit spills, and local memory is far away beside 217 KB of shared
+// memory: up to 11 % on passes with short parts.)
+constexpr int SPREAD = 4;
+__device__ __forceinline__ bool spread_parts(int nt, int np, int k) { return k > 1 && nt - np >= SPREAD * k; }
+struct Spread {
+    int na, a0, b0;                  // na >= 0: this CTA's part is spread (tiles of the prefix, the first of them, the first beyond)
+};
+__device__ __forceinline__ Spread& spread_of_cta()
+{
+    __shared__ Spread x;
+    return x;
+}
+// List entry of the segment's tile t, and how many of its tiles are whole tiles of the prefix (they come first).
+__device__ __forceinline__ int tile_entry(const Segment& sg, int t)
+{
+    if (!TWO) return sg.j0 + t;
+    const Spread& x = spread_of_cta();
+    return x.na < 0 ? sg.j0 + t : (t < x.na ? x.a0 + t : x.b0 + t - x.na);
+}
+__device__ __forceinline__ int prefix_tiles(const Segment& sg, int npre)
+{
+    const int na = TWO ? spread_of_cta().na : -1;
+    return na >= 0 ? na : (npre <= sg.j0 ? 0 : (npre < sg.j1 ? npre : sg.j1) - sg.j0);
+}
 // First unit whose weighted start is >= x.
 __device__ __forceinline__ long long unit_of_virt(const AttnParams& p, const Split& cx, long long x)
 {
@@ -180,15 +214,15 @@ __device__ __forceinline__ void pair_ctas(const AttnParams& p, const Split& cx, 
 // issue() is called there, and the trip hides behind the set-up.
 template <int THREADS>
 struct SplitFinder {
-    static constexpr int MEMO_MAGIC = 0x5D180000 | (W_PREFIX << 12) | (W_MASKED << 8) | W_PAIR;
+    static constexpr int MEMO_MAGIC = 0x5D180000 | (TWO ? 0x02000000 : 0) | (W_PREFIX << 12) | (W_MASKED << 8) | W_PAIR;
     const int32_t* mrd;
-    int4 mh0, mh1, mh2, me;
+    int4 mh0, mh1, mh2, me, msp;
     int m_na, m_nt, m_prev;
     int na[4], nt[4];
 
     __device__ __forceinline__ SplitFinder(const AttnParams& p, int split_only) : mrd((p.split_memo && !split_only) ? p.split_memo : nullptr)
     {
-        mh0 = mh1 = mh2 = me = make_int4(0, 0, 0, 0);
+        mh0 = mh1 = mh2 = me = msp = make_int4(0, 0, 0, 0);
         m_na = m_nt = -1;
         m_prev = 0;
     }
@@ -199,6 +233,7 @@ struct SplitFinder {
             mh1 = __ldcg(reinterpret_cast<const int4*>(mrd) + 1);
             mh2 = __ldcg(reinterpret_cast<const int4*>(mrd) + 2);
             me = __ldcg(reinterpret_cast<const int4*>(mrd + FDC_MEMO_ENTRIES) + blockIdx.x);
+            if (TWO && threadIdx.x == 0) msp = __ldcg(reinterpret_cast<const int4*>(mrd + FDC_MEMO_SPREAD) + blockIdx.x);
             if ((int)threadIdx.x < p.batch) {
                 m_na = __ldcg(mrd + 16 + threadIdx.x);
                 m_nt = __ldcg(mrd + 16 + FDC_MEMO_BATCH + threadIdx.x);
@@ -252,6 +287,7 @@ struct SplitFinder {
             cx.n_cta = mh1.w;
             cx.vtot = ((long long)mh2.y << 32) | (uint32_t)mh2.x;
             if ((int)threadIdx.x <= p.batch) cx.prev[threadIdx.x] = m_prev;
+            if (TWO && threadIdx.x == 0) spread_of_cta() = Spread{msp.x, msp.y, msp.z};
             __syncthreads();
             lo = ((long long)me.y << 32) | (uint32_t)me.x;
             hi = ((long long)me.w << 32) | (uint32_t)me.z;
@@ -360,8 +396,13 @@ struct SplitFinder {
                     const int k = cx.prev[sl + 1] - cx.prev[sl], nt = cx.pre[sl + 1] - cx.pre[sl];
                     const uint32_t idx = (uint32_t)(c - cx.prev[sl] * p.hkv), g = idx / (uint32_t)k, i = idx - g * (uint32_t)k;
                     const uint32_t V = (uint32_t)vt_of(cx, nt, nt);       // part i: tiles whose weighted start lies in [i V / k, (i + 1) V / k)
-                    const int j0 = tile_of_vt(cx, nt, (int)((i * V + k - 1) / (uint32_t)k));
-                    const int j1 = tile_of_vt(cx, nt, (int)(((i + 1) * V + k - 1) / (uint32_t)k));
+                    int j0 = tile_of_vt(cx, nt, (int)((i * V + k - 1) / (uint32_t)k));
+                    int j1 = tile_of_vt(cx, nt, (int)(((i + 1) * V + k - 1) / (uint32_t)k));
+                    const int np = cx.npre < nt ? cx.npre : nt;
+                    if (TWO && spread_parts(nt, np, k)) {
+                        j0 = np * (int)i / k + (nt - np) * (int)i / k;
+                        j1 = np * ((int)i + 1) / k + (nt - np) * ((int)i + 1) / k;
+                    }
                     lo = (long long)cx.pre[sl] * p.hkv + (long long)g * nt + j0;
                     hi = lo + (j1 - j0);
                 }
@@ -378,12 +419,32 @@ struct SplitFinder {
             hi = cta_first_unit(blockIdx.x + 1, U, cx.n_cta);
         }
         if (lo >= hi || (int)blockIdx.x >= cx.n_cta) active = false;
+        if (TWO && !hit) {
+            if (threadIdx.x == 0) {
+                Spread& x = spread_of_cta();
+                x = Spread{-1, 0, 0};
+                if (active && cx.tpart && p.W >= 2 * SPREAD - 1) {       // (else no pair has that many tiles beyond the prefix)
+                    int s = 0;
+                    const Segment sg = decode_segment(lo, hi, cx.pre, p.hkv, s);
+                    const int np = cx.npre < sg.nt ? cx.npre : sg.nt, k = cx.prev[s + 1] - cx.prev[s];
+                    if (spread_parts(sg.nt, np, k)) {
+                        const int i = (int)blockIdx.x - (cx.prev[s] * p.hkv + sg.g * k);
+                        x.a0 = np * i / k;
+                        x.na = np * (i + 1) / k - x.a0;
+                        x.b0 = np + (sg.nt - np) * i / k;
+                    }
+                }
+            }
+            __syncthreads();
+        }
         if (split_only) {
             // this launch only computes the split and leaves it to the attention launches of the pass
             int32_t* mwr = p.split_memo;
             if (threadIdx.x == 0)
                 reinterpret_cast<int4*>(mwr + FDC_MEMO_ENTRIES)[blockIdx.x] =
                     active ? make_int4((int)(uint32_t)lo, (int)(lo >> 32), (int)(uint32_t)hi, (int)(hi >> 32)) : make_int4(0, 0, 0, 0);
+            if (TWO && threadIdx.x == 0)
+                reinterpret_cast<int4*>(mwr + FDC_MEMO_SPREAD)[blockIdx.x] = make_int4(spread_of_cta().na, spread_of_cta().a0, spread_of_cta().b0, 0);
             if (blockIdx.x == 0) {
                 if (threadIdx.x == 0) {
                     reinterpret_cast<int4*>(mwr)[0] = make_int4(MEMO_MAGIC, (int)p.seq, p.hkv, p.n_cta);
@@ -402,11 +463,41 @@ struct SplitFinder {
     }
 };
 
+// ---- pairs in two parts -----------------------------------------------------------------------
+// The launch's CTAs come in clusters of two, so the two CTAs of a pair that is cut in two (consecutive, the first one even) are on the chip
+// together and may wait for one another: each hands the other one half of its partial result through the workspace, finishes the other half itself
+// and no CTA merges alone.  Every thread of the launch arrives at the cluster's barrier when its block's barriers stand, and waits there ahead of its role; and
+// again at the very end, so that no block leaves while the other one may still signal it.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// One arrival at the other block's barrier at the same place; everything the thread has written or seen written is known to who sees it.
+__device__ __forceinline__ void arrive_at_peer(uint32_t bar)
+{
+    asm volatile(
+        "{\n\t.reg .b32 r, a;\n\tmov.u32 r, %cluster_ctarank;\n\txor.b32 r, r, 1;\n\tmapa.shared::cluster.u32 a, %0, r;\n\t"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n\t}" ::"r"(bar)
+        : "memory");
+}
+// (bounded like every in-kernel wait; the outcome is the warp's)
+__device__ __forceinline__ bool wait_for_peer(uint32_t bar, volatile int* abort_flag, int32_t* status)
+{
+    bool ok = mbar_wait_warp(bar, 0, abort_flag, status);
+    asm volatile("fence.acq_rel.cluster;" ::: "memory");
+    return ok;
+}
+// This CTA's place in a pair cut in two: 0 or 1; -1: not such a pair, or not in one cluster.
+__device__ __forceinline__ int half_of_pair(const Split& cx, const Segment& sg, int hkv)
+{
+    if (!cx.tpart || cx.prev[sg.s + 1] - cx.prev[sg.s] != 2) return -1;
+    const int c_first = cx.prev[sg.s] * hkv + sg.g * 2;
+    return (c_first & 1) ? -1 : (int)blockIdx.x - c_first;
+}
+
 // Position of one ring's producer in the CTA's unit sequence.
 struct Cursor {
     long long u;                 // first unit of the current segment
     Segment sg;
-    int s, jb, jn, k, my_tile;   // scene hint; batch of up to 32 tile ids (one per lane) and the position inside it
+    int s, jb, jn, k, my_tile;   // scene hint; batch of up to 32 tile ids (one per lane; jb: the segment's tiles ahead of it) and the position inside it
     uint32_t g;                  // round
     int st;                      // ring stage of round g
     uint32_t ph;                 // ring phase of round g
@@ -414,9 +505,10 @@ struct Cursor {
 };
 __device__ __forceinline__ void cursor_batch(Cursor& c, const AttnParams& p, int lane)
 {
-    c.jn = c.sg.j1 - c.jb < 32 ? c.sg.j1 - c.jb : 32;
+    const int n = c.sg.j1 - c.sg.j0;
+    c.jn = n - c.jb < 32 ? n - c.jb : 32;
     // entry j of a tile list is tile j for every whole tile of the prefix: no need to read those
-    const int j = c.jb + lane;
+    const int j = tile_entry(c.sg, c.jb + lane);
     c.my_tile = lane < c.jn ? (j < p.P / TILE ? j : p.tiles[(size_t)c.sg.s * p.ntile_max + j]) : 0;
     c.k = 0;
 }
@@ -425,7 +517,7 @@ __device__ __forceinline__ void cursor_open(Cursor& c, const AttnParams& p, cons
     c.live = c.u < hi;
     if (!c.live) return;
     c.sg = decode_segment(c.u, hi, cx.pre, p.hkv, c.s);
-    c.jb = c.sg.j0;
+    c.jb = 0;
     cursor_batch(c, p, lane);
 }
 template <int TPS>
@@ -439,7 +531,7 @@ __device__ __forceinline__ void cursor_next(Cursor& c, const AttnParams& p, cons
     }
     if (c.k < c.jn) return;
     c.jb += 32;
-    if (c.jb < c.sg.j1) {
+    if (c.jb < c.sg.j1 - c.sg.j0) {
         cursor_batch(c, p, lane);
     } else {
         c.u = c.sg.next_u;
@@ -580,7 +672,13 @@ __device__ __noinline__ void append_rows(char* kc, char* vc, long long stride_sc
     while (u < hi) {
         const Segment sg = decode_segment(u, hi, pre, hkv, s);
         const int A = nact[sg.s];
-        const int t_first = tiles[(size_t)sg.s * ntile_max + sg.j0], t_last = tiles[(size_t)sg.s * ntile_max + sg.j1 - 1];
+        int j0 = sg.j0, j1 = sg.j1;
+        if (TWO) {                                     // (a new row is in no whole tile of the prefix)
+            const int n = sg.j1 - sg.j0, na = prefix_tiles(sg, P / TILE);
+            j0 = na < n ? tile_entry(sg, na) : 0;
+            j1 = na < n ? tile_entry(sg, n - 1) + 1 : 1;
+        }
+        const int t_first = tiles[(size_t)sg.s * ntile_max + j0], t_last = tiles[(size_t)sg.s * ntile_max + j1 - 1];
         for (int b0 = 0; b0 < A; b0 += 32) {
             const int b = b0 + lane;
             const int r = b < A ? app_row[(size_t)sg.s * max_active + b] : P;
@@ -631,5 +729,43 @@ __device__ __noinline__ uint64_t tile_seen_rows(const uint64_t* un, const uint64
     const uint32_t uh = __reduce_or_sync(0xffffffffu, (uint32_t)(um >> 32));
     return ((uint64_t)uh << 32) | ul;
 }
+
+inline cudaLaunchAttribute cluster_of_two()
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = 2;
+    a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    return a;
+}
+// Whether the device holds n_cta blocks of a kernel in clusters of two at once (asked once per device): FDC_OK, or FDC_ERR_SHAPE (another build's launch).
+struct PairsPlaceable {
+    std::atomic<int> known[kMaxDevices] = {};         // 0: not asked; n + 1: that many clusters
+    int all(const void* kernel, int threads, size_t smem, int n_cta)
+    {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return FDC_ERR_SHAPE;
+        int n = known[dev].load(std::memory_order_relaxed);
+        if (n == 0) {
+            static size_t attr_smem[kMaxDevices] = {};
+            const int rc = raise_dynamic_smem(kernel, smem, attr_smem);
+            if (rc) return rc;
+            cudaLaunchConfig_t one = {};
+            cudaLaunchAttribute at = cluster_of_two();
+            one.gridDim = dim3((unsigned)n_cta);
+            one.blockDim = dim3((unsigned)threads);
+            one.dynamicSmemBytes = smem;
+            one.attrs = &at;
+            one.numAttrs = 1;
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &one) != cudaSuccess) {
+                cudaGetLastError();
+                clusters = 0;
+            }
+            known[dev].store(n = clusters + 1, std::memory_order_relaxed);
+        }
+        return 2 * (n - 1) >= n_cta ? FDC_OK : FDC_ERR_SHAPE;
+    }
+};
 
 }  // namespace
