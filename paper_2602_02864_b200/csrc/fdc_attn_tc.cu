@@ -18,7 +18,8 @@ int launch_tc_rows_two(const AttnParams& p, int head_dim, cudaStream_t st, int s
 // pair's list, and that hand each other half of their results): with more than 32 query rows, from 32 tiles a pair on and while the shares are short enough
 // for one part per CTA (see SplitFinder).  us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, 140 tiles 59.1 / 56.6.  With
 // 16 tiles a pair the start of the CTAs two by two costs more than that gains (64 pairs, 35 rows 21.7 / 23.7), with equal shares nothing is
-// handed over (128 rows, 544 tiles 213.3 / 216.0).
+// handed over (128 rows, 544 tiles 213.3 / 216.0), and up to 32 rows are merged as fast by the CTA that comes last (64 pairs, 24 rows, prefix 4096 34.4 / 34.8;
+// 28 rows, 2048 23.3 / 24.2).
 static bool pairs_in_two_parts(const AttnParams& p)
 {
     const long long pairs = (long long)p.batch * p.hkv;
