@@ -15,15 +15,16 @@ int launch_tc_np64_two(const AttnParams& p, int head_dim, cudaStream_t st, int s
 int launch_tc_rows_two(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);    // fdc_attn_tc_rows_two.cu
 
 // Launches whose pairs come in two parts each, one per CTA, as long as no scene has ended, go to builds of their own (parts that are spread over the
-// pair's list, and that hand each other half of their results): with more than 32 query rows, from 32 tiles a pair on and while the shares are short enough
-// for one part per CTA (see SplitFinder).  us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, 140 tiles 59.1 / 56.6.  With
+// pair's list, and that hand each other half of their results): with more than 32 query rows, from 32 tiles a pair on and while all tiles of a
+// template, listed at once, still make one part per CTA (equal_shares, as the kernels split them).  us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, 140 tiles 59.1 / 56.6.  With
 // 16 tiles a pair the start of the CTAs two by two costs more than that gains (64 pairs, 35 rows 21.7 / 23.7), with equal shares nothing is
-// handed over (128 rows, 544 tiles 213.3 / 216.0), and up to 32 rows are merged as fast by the CTA that comes last (64 pairs, 24 rows, prefix 4096 34.4 / 34.8;
-// 28 rows, 2048 23.3 / 24.2).
-static bool pairs_in_two_parts(const AttnParams& p)
+// handed over (128 rows, 208 tiles, 32 of them beyond the prefix 93.4 / 95.9; 231 tiles, 96 beyond 117.3 / 128.1), and up to 32 rows are merged as fast by the
+// CTA that comes last (64 pairs, 24 rows, prefix 4096 34.4 / 34.8; 28 rows, 2048 23.3 / 24.2).
+bool pairs_in_two_parts(int64_t pairs, int mmax, int P, int ntile_max, int n_cta)
 {
-    const long long pairs = (long long)p.batch * p.hkv;
-    return p.pair_cnt && p.n_cta % 2 == 0 && 2 * pairs <= p.n_cta && 3 * pairs > p.n_cta && p.ntile_max >= 32 && p.ntile_max * pairs < (p.mmax > 64 ? 100 : 200) * (long long)p.n_cta;
+    if (mmax <= 32 || n_cta % 2 || 2 * pairs > n_cta || 3 * pairs <= n_cta || ntile_max < 32) return false;
+    const int length = weighted_tiles(P / FDC_TILE_ROWS, ntile_max);
+    return !equal_shares(pairs * (length + W_PAIR), (length + 1) / 2, n_cta, mmax);
 }
 
 // More than 64 query rows go to the row form.  Measured on both sides of the line (us a layer, transposed / row
@@ -32,7 +33,7 @@ static bool pairs_in_two_parts(const AttnParams& p)
 // scenes, prefix 4096: 53.3 / 59.5; 16 rows, 64 scenes, prefix 16384: 629 / 732.
 static int launch_tc(const AttnParams& p, int head_dim, cudaStream_t st, int split_only)
 {
-    if (p.mmax > 32 && pairs_in_two_parts(p)) {
+    if (p.pair_cnt && pairs_in_two_parts((int64_t)p.batch * p.hkv, p.mmax, p.P, p.ntile_max, p.n_cta)) {
         const int rc = p.mmax > 64 ? launch_tc_rows_two(p, head_dim, st, split_only) : launch_tc_np64_two(p, head_dim, st, split_only);
         if (rc != FDC_ERR_SHAPE) return rc;
     }

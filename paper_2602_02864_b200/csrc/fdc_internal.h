@@ -100,6 +100,27 @@ inline uint32_t div_inverse(int n) { return n > 1 ? (uint32_t)((1ull << 32) / (u
 #ifdef __CUDACC__
 __device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t inverse) { return inverse ? __umulhi(x, inverse) : x; }
 #endif
+// Weights of the tcgen05 kernels' work split (the unit is a quarter of a tile inside the prefix).
+constexpr int W_PREFIX = 4;
+constexpr int W_MASKED = 6;          // a tile beyond the prefix (bitmap selects, V clean-up): measured about 1.5 prefix tiles
+constexpr int W_PAIR = 32;           // finishing a (scene, KV head) pair (drain, partial write, next queries)
+// Weighted length of a pair's first `nt` tiles, of which the first `np` are whole tiles of the prefix.
+FDC_HD int weighted_tiles(int np, int nt) { return nt <= np ? nt * W_PREFIX : np * W_PREFIX + (nt - np) * W_MASKED; }
+// One part per CTA leaves CTAs idle when the parts per pair do not divide the CTAs evenly
+// (64 pairs on 148 CTAs: 2 or 3 parts, a CTA carries up to 16 % more than the average).  Where the
+// shares are long enough for a pair boundary inside a CTA to cost less than that, equal shares of the
+// weighted length win after all: from about 200 prefix tiles per CTA, half of that with more than 64 query
+// rows (the row form), whose tiles take longer.  Measured there, us a layer one part / equal shares, 32 / 8
+// heads x 128, 32 fields: 26 tiles per CTA (8 scenes, prefix 3840) 57 / 65, 60 tiles 85.9 / 85.1, 100 tiles
+// 121 / 116, 150 tiles 165 / 158; 100 tiles in 5 scenes (40 pairs) 124 / 116, in 12 scenes (96 pairs) 153 /
+// 125; where the parts divide well (48 pairs in 144 parts) 103 / 107.
+// length: of all pairs, W_PAIR for each included; part: the longest part of a cut for one part per CTA.
+FDC_HD bool equal_shares(long long length, int part, int n_cta, int mmax)
+{
+    const long long avg = length / n_cta;
+    return avg * (mmax > 64 ? 2 : 1) >= 200 * W_PREFIX && (long long)part * 100 > avg * 108;
+}
+bool pairs_in_two_parts(int64_t pairs, int mmax, int P, int ntile_max, int n_cta);      // fdc_attn_tc.cu
 ClusterShape pick_cluster(const ClusterProblem& c, float* us);      // us (may be NULL): the estimated time
 bool route_problem(const ClusterProblem& c, ClusterShape* cut);     // the cut, and whether the cluster kernel is the one to take (head_dim 64: always)
 int cluster_ring(int head_dim, int rows, int nblk, int per_sm);     // stages of a block's ring (bf16); 0: no room for the partials beside it

@@ -16,9 +16,6 @@ namespace {
 
 constexpr int D = 128;                       // head_dim handled by these kernels
 constexpr int TILE = FDC_TILE_ROWS;          // rows per entry of the visited-tile list
-constexpr int W_PREFIX = 4;       // cost of a tile inside the prefix (the unit of the weighted work split is a quarter of it)
-constexpr int W_MASKED = 6;       // cost of a tile beyond the prefix (bitmap selects, V clean-up): measured about 1.5 prefix tiles
-constexpr int W_PAIR = 32;           // cost of finishing a (scene, KV head) pair (drain, partial write, next queries)
 #if !defined(FDC_TC_TWO)
 #error "FDC_TC_TWO: 1 for the build that launches whose pairs are cut in two parts are given (pairs_in_two_parts), else 0"
 #endif
@@ -131,8 +128,7 @@ struct Split {
 // start falls into its share, so shares always cut the unit sequence into consecutive runs.
 __device__ __forceinline__ int vt_of(const Split& cx, int nt, int j)
 {
-    const int np = cx.npre < nt ? cx.npre : nt;
-    return j <= np ? j * W_PREFIX : np * W_PREFIX + (j - np) * W_MASKED;
+    return weighted_tiles(cx.npre < nt ? cx.npre : nt, j);
 }
 // First tile of a pair of nt tiles whose weighted start is >= r (nt if there is none).
 __device__ __forceinline__ int tile_of_vt(const Split& cx, int nt, int r)
@@ -342,21 +338,12 @@ struct SplitFinder {
             }
             __syncthreads();
             if (one_part && threadIdx.x == 0) {
-                // One part per CTA leaves CTAs idle when the parts per pair do not divide the CTAs evenly
-                // (64 pairs on 148 CTAs: 2 or 3 parts, a CTA carries up to 16 % more than the average).  Where the
-                // shares are long enough for a pair boundary inside a CTA to cost less than that, equal shares of the
-                // weighted length win after all: from about 200 prefix tiles per CTA, half of that with more than 64 query
-                // rows (the row form), whose tiles take longer.  Measured there, us a layer one part / equal shares, 32 / 8
-                // heads x 128, 32 fields: 26 tiles per CTA (8 scenes, prefix 3840) 57 / 65, 60 tiles 85.9 / 85.1, 100 tiles
-                // 121 / 116, 150 tiles 165 / 158; 100 tiles in 5 scenes (40 pairs) 124 / 116, in 12 scenes (96 pairs) 153 /
-                // 125; where the parts divide well (48 pairs in 144 parts) 103 / 107.
                 long long tot = 0;
                 for (int i = 0; i < p.batch; ++i) {
                     const int nt = cx.pre[i + 1] - cx.pre[i];
                     if (nt > 0) tot += vt_of(cx, nt, nt) + W_PAIR;
                 }
-                const long long avg = tot * p.hkv / p.n_cta;
-                if (avg * (p.mmax > 64 ? 2 : 1) >= 200 * W_PREFIX && (long long)split_tpart * 100 > avg * 108) split_tpart = 0;
+                if (equal_shares(tot * p.hkv, split_tpart, p.n_cta, p.mmax)) split_tpart = 0;
             }
             __syncthreads();
             if (threadIdx.x < 32) {

@@ -69,3 +69,55 @@ def test_every_cut_has_room_for_the_partials(route):
     assert len(got) == len(shapes)
     assert all(g[4] > 0 for g in got)
     assert any(g[1] > 1 and g[3] == 2 for g in got) and any(g[1] > 1 and g[3] == 1 for g in got)
+
+
+TWO_PARTS = """#include "fdc_internal.h"
+#include <cstdio>
+int main() {
+    long long pairs; int mmax, P, nt;
+    while (scanf("%lld %d %d %d", &pairs, &mmax, &P, &nt) == 4) printf("%d\\n", fdc::pairs_in_two_parts(pairs, mmax, P, nt, 148));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def two_parts(tmp_path_factory):
+    """shapes (pairs, query rows, prefix, tiles a pair at most) -> the launch goes to the builds for pairs in two parts (148 CTAs)"""
+    from paper_2602_02864_b200 import build
+    lib = build.build()
+    d = tmp_path_factory.mktemp("two")
+    (d / "two.cpp").write_text(TWO_PARTS)
+    subprocess.check_call(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2602_02864_b200", "csrc"),
+                           "-I", "/usr/local/cuda/include", str(d / "two.cpp"), "-o", str(d / "two"), lib, "-Wl,-rpath," + os.path.dirname(lib)])
+
+    def ask(shapes):
+        out = subprocess.run([str(d / "two")], input="\n".join(" ".join(str(x) for x in s) for s in shapes), capture_output=True, text=True, check=True).stdout
+        return [x == "1" for x in out.split()]
+    return ask
+
+
+def split_of_whole_lists(scenes, hkv, mmax, P, nt, n_cta=148):
+    """Parts of a pair when every scene lists `nt` tiles, as the tcgen05 kernels cut them (0: equal shares)."""
+    prefix = min(P // 64, nt)
+    length = 4 * prefix + 6 * (nt - prefix)
+    part = next(t for t in range(min(length, 32), length + 1) if scenes * -(-length // t) <= n_cta // hkv)
+    avg = scenes * hkv * (length + 32) // n_cta
+    return 0 if avg * (2 if mmax > 64 else 1) >= 800 and part * 100 > avg * 108 else -(-length // part)
+
+
+# us a layer, plain build / build for pairs in two parts
+@pytest.mark.parametrize("shape,two", [
+    ((64, 128, 1024, 48), True),              # 38.6 / 34.0
+    ((64, 128, 176 * 64, 208), False),        # 93.4 / 95.9: equal shares
+    ((64, 128, 80 * 64, 176), False),         # 99.2 / 103.5: equal shares
+    ((64, 128, 135 * 64, 231), False)])       # 117.3 / 128.1: equal shares
+def test_pairs_in_two_parts(two_parts, shape, two):
+    assert two_parts([shape])[0] == two
+
+
+def test_pairs_in_two_parts_are_cut_in_two(two_parts):
+    shapes = [(scenes, hkv, mmax, P, P // 64 + beyond) for hkv in (1, 2, 4, 5, 8) for scenes in range(-(-50 // hkv), 74 // hkv + 1) for mmax in (36, 64, 72, 128)
+              for P in (0, 500, 1024, 2048, 5120, 8192, 13312, 20480, 28672) for beyond in (3, 16, 32, 48, 96)]
+    got = two_parts([(s * h, m, P, nt) for s, h, m, P, nt in shapes])
+    assert any(got) and not all(got)
+    assert all(split_of_whole_lists(*x) == 2 for x, g in zip(shapes, got) if g)
