@@ -15,15 +15,26 @@ int launch_tc_np64_two(const AttnParams& p, int head_dim, cudaStream_t st, int s
 int launch_tc_rows_two(const AttnParams& p, int head_dim, cudaStream_t st, int split_only);    // fdc_attn_tc_rows_two.cu
 
 // Launches whose pairs come in two parts each, one per CTA, as long as no scene has ended, go to builds of their own (parts that are spread over the
-// pair's list, and that hand each other half of their results): with more than 32 query rows, from 32 tiles a pair on and while all tiles of a
-// template, listed at once, still make one part per CTA (equal_shares, as the kernels split them).  us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, 140 tiles 59.1 / 56.6.  With
-// 16 tiles a pair the start of the CTAs two by two costs more than that gains (64 pairs, 35 rows 21.7 / 23.7), with equal shares nothing is
+// pair's list, and that hand each other half of their results): with more than 32 query rows, from 32 tiles a pair on, while all tiles of a
+// template, listed at once, still make one part per CTA (equal_shares, as the kernels split them), and where a template as a whole gains by it.
+//
+// That is where the tiles beyond the prefix are at least half of the list's length, so that the plain builds' second part has nothing that it could
+// load ahead of the append, or where a merge by one CTA is long (120 query rows and more).  CTAs that start two by two cost 1 us a launch (blocks that wait for a
+// place for both), which passes with few fields at work, as most templates have them at one end, do not win back.  Whole templates, plain build / these (the time of every 8th or 16th
+// pass, fan, diamond, wide and free, fields of equal and of drawn lengths, 50 to 74 pairs, prefix 512 to 16384): half and more beyond 1.054 (181 templates, the
+// worst 0.984), 120 rows and more otherwise 1.028 (81, 0.990), 65 to 119 rows 1.009 (195, 0.974, 18 of them below 0.985), 33 to 64 rows 0.999 (190,
+// 0.957, 42 below 0.985; 8 scenes, 16 fields x 4 heads, prefix 8192: widest passes 1.02, later ones 0.98).  Within these lines single passes lie between 0.90 (most scenes
+// ended) and 1.2.
+//
+// us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, prefix 1024, 32 tiles 32.6 / 27.1.  With
+// 16 tiles a pair that start costs more than this gains (64 pairs, 35 rows 21.7 / 23.7), with equal shares nothing is
 // handed over (128 rows, 208 tiles, 32 of them beyond the prefix 93.4 / 95.9; 231 tiles, 96 beyond 117.3 / 128.1), and up to 32 rows are merged as fast by the
 // CTA that comes last (64 pairs, 24 rows, prefix 4096 34.4 / 34.8; 28 rows, 2048 23.3 / 24.2).
 bool pairs_in_two_parts(int64_t pairs, int mmax, int P, int ntile_max, int n_cta)
 {
     if (mmax <= 32 || n_cta % 2 || 2 * pairs > n_cta || 3 * pairs <= n_cta || ntile_max < 32) return false;
     const int length = weighted_tiles(P / FDC_TILE_ROWS, ntile_max);
+    if (mmax < 120 && 2 * W_PREFIX * (P / FDC_TILE_ROWS) > length) return false;
     return !equal_shares(pairs * (length + W_PAIR), (length + 1) / 2, n_cta, mmax);
 }
 

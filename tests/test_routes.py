@@ -108,6 +108,12 @@ def split_of_whole_lists(scenes, hkv, mmax, P, nt, n_cta=148):
 # us a layer, plain build / build for pairs in two parts
 @pytest.mark.parametrize("shape,two", [
     ((64, 128, 1024, 48), True),              # 38.6 / 34.0
+    ((72, 128, 5632, 120), True),             # 69.3 / 65.0: 128 rows
+    ((64, 64, 1024, 32), True),               # 32.6 / 27.1
+    ((64, 36, 2048, 41), False),              # 25.6 / 26.7
+    ((68, 63, 2048, 41), False),              # 9 fields x 7 heads, fan, the whole template 0.957
+    ((64, 64, 8192, 142), False),             # 16 fields x 4 heads, wide, 55.1 / 55.9 in its later passes, the whole template 0.999
+    ((72, 91, 2048, 47), False),              # 13 fields x 7 heads, wide, the whole template 0.974
     ((64, 128, 176 * 64, 208), False),        # 93.4 / 95.9: equal shares
     ((64, 128, 80 * 64, 176), False),         # 99.2 / 103.5: equal shares
     ((64, 128, 135 * 64, 231), False)])       # 117.3 / 128.1: equal shares
