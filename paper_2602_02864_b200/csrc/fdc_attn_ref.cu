@@ -241,8 +241,8 @@ int launch_ref_t(const AttnParams& p, cudaStream_t st)
     size_t smem = sizeof(float) * ((size_t)64 * (D + 1) + 64 * D + 2 * (size_t)p.mmax * D + kWarps * 64 + 2 * p.mmax) +
                   sizeof(int) * (p.batch + 1);
     if (smem > 227 * 1024) return FDC_ERR_SHAPE;
-    static size_t attr_smem[kMaxDevices] = {};
-    const int rcs = raise_dynamic_smem(reinterpret_cast<const void*>(attn_ref_kernel<T, D>), smem, attr_smem);
+    static SmemLimit limit;
+    const int rcs = raise_dynamic_smem(reinterpret_cast<const void*>(attn_ref_kernel<T, D>), smem, limit);
     if (rcs) return rcs;
     attn_ref_kernel<T, D><<<p.n_cta, kThreads, smem, st>>>(p);
     note_launch();

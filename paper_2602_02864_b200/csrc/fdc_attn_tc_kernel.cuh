@@ -1244,6 +1244,7 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     const int p_buf = ((np_max + 63) / 64) * PANEL;
     if (np_max != NP_MAX) return FDC_ERR_SHAPE;   // another build's launches
     const int npb = 2;
+    static SmemLimit limit;
     int rc = FDC_OK;
     const size_t fixed = 1024 + (size_t)npb * p_buf + (size_t)(D / 64) * np_max * 128 + ONES_BYTES + 8 * (5 * MAXST + 16) + 16 +
                          4 * (128 + 128 + 512 + 128 + 12) + sizeof(int) * (3 * p.batch + 2) + 8 * (2 * MBUF + 2 * UW + 2) + 64;
@@ -1252,7 +1253,7 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     if (stages < 4) return FDC_ERR_SHAPE;
     if (TWO) {
         static PairsPlaceable placeable;
-        rc = placeable.all(reinterpret_cast<const void*>(FDC_TC_KERNEL), THREADS, fixed + (size_t)stages * STAGE, p.n_cta);
+        rc = placeable.all(reinterpret_cast<const void*>(FDC_TC_KERNEL), THREADS, fixed + (size_t)stages * STAGE, p.n_cta, limit);
         if (rc) return rc;
     }
     if (split_only) stages = 0;
@@ -1263,8 +1264,7 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     if (rc) return rc;
     rc = get_kv_tensor_map(p.v, p, FDC_BF16, D, TILE, &tv);
     if (rc) return rc;
-    static size_t attr_smem[kMaxDevices] = {};
-    rc = raise_dynamic_smem(reinterpret_cast<const void*>(FDC_TC_KERNEL), smem, attr_smem);
+    rc = raise_dynamic_smem(reinterpret_cast<const void*>(FDC_TC_KERNEL), smem, limit);
     if (rc) return rc;
     {
         cudaLaunchConfig_t cfg = {};

@@ -946,10 +946,11 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     int stages = (int)((227 * 1024 - 256 - fixed) / STAGE);
     if (stages > 2 * MAXST) stages = 2 * MAXST;
     if (stages < 2 * NBUF) return FDC_ERR_SHAPE;  // (a V stage's use before is known to be over when its next one is waited for: NBUF of them at least)
+    static SmemLimit limit;
     int rc = FDC_OK;
     if (TWO) {
         static PairsPlaceable placeable;
-        rc = placeable.all(reinterpret_cast<const void*>(FDC_TC_KERNEL), THREADS, fixed + (size_t)stages * STAGE, p.n_cta);
+        rc = placeable.all(reinterpret_cast<const void*>(FDC_TC_KERNEL), THREADS, fixed + (size_t)stages * STAGE, p.n_cta, limit);
         if (rc) return rc;
     }
     if (split_only) stages = 0;
@@ -960,8 +961,7 @@ int FDC_TC_LAUNCH(const AttnParams& p, int head_dim, cudaStream_t st, int split_
     if (rc) return rc;
     rc = get_kv_tensor_map(p.v, p, FDC_BF16, D, TILE, &tv);
     if (rc) return rc;
-    static size_t attr_smem[kMaxDevices] = {};
-    rc = raise_dynamic_smem(reinterpret_cast<const void*>(FDC_TC_KERNEL), smem, attr_smem);
+    rc = raise_dynamic_smem(reinterpret_cast<const void*>(FDC_TC_KERNEL), smem, limit);
     if (rc) return rc;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p.n_cta);

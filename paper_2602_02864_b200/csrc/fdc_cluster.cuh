@@ -724,8 +724,8 @@ int launch_cluster(Kernel kernel, const AttnParams& p, size_t room, const Cluste
     if (nstage == 0) return FDC_ERR_SHAPE;
     size_t smem = cluster_smem_fixed<Math>(qrows, h.nblk) + (size_t)nstage * Math::STAGE_BYTES;
     if (h.per_sm <= 1 && smem < 120 * 1024) smem = 120 * 1024;        // (more than half of an SM's: no second block beside this one)
-    static size_t attr_smem[kMaxDevices] = {};
-    int rc = raise_dynamic_smem(reinterpret_cast<const void*>(kernel), smem, attr_smem);
+    static SmemLimit limit;
+    int rc = raise_dynamic_smem(reinterpret_cast<const void*>(kernel), smem, limit);
     if (rc) return rc;
     static PlaceableClusters known;
     alignas(64) CUtensorMap tk, tv;

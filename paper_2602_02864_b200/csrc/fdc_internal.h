@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "fdc.h"
 
 #define FDC_PAIR_COUNTERS 65536
@@ -217,21 +219,69 @@ int  launch_kv_append(fdc_plan* plan, const fdc_kv_desc* kv, int32_t layer, cons
                       const void* d_k_new, const void* d_v_new, void* stream);
 int  flush_pending_append(fdc_plan* plan);     // launches a recorded append on its own (no-op when there is none)
 
-// cudaFuncAttributeMaxDynamicSharedMemorySize is kept by the runtime per device: `set` remembers,
-// per device ordinal, what this process has already asked for on behalf of one kernel.
+// cudaFuncAttributeMaxDynamicSharedMemorySize is kept by the runtime per kernel and device, and the last call wins.  So every call sets the
+// same value, all that a block can have: threads that launch with different sizes cannot lower it for one another, in whatever order
+// they come.  One SmemLimit per kernel remembers the devices that have been told.
 constexpr int kMaxDevices = 64;
-inline int raise_dynamic_smem(const void* kernel, size_t bytes, size_t (&set)[kMaxDevices])
+struct SmemLimit {
+    std::atomic<size_t> set[kMaxDevices] = {};
+};
+inline int raise_dynamic_smem(const void* kernel, size_t bytes, SmemLimit& limit)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return set_cuda_error(e);
     const bool known = dev >= 0 && dev < kMaxDevices;
-    if (known && bytes <= set[dev]) return FDC_OK;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (known && bytes <= limit.set[dev].load(std::memory_order_acquire)) return FDC_OK;
+    int block = 0;
+    cudaFuncAttributes own;
+    e = cudaDeviceGetAttribute(&block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&own, kernel);
     if (e != cudaSuccess) return set_cuda_error(e);
-    if (known) set[dev] = bytes;
+    const size_t room = (size_t)block > own.sharedSizeBytes ? (size_t)block - own.sharedSizeBytes : 0;
+    const size_t most = bytes > room ? bytes : room;            // (more than there is: refused here)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) return set_cuda_error(e);
+    if (known) limit.set[dev].store(most, std::memory_order_release);
     return FDC_OK;
 }
+
+inline cudaLaunchAttribute cluster_of_two()
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = 2;
+    a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    return a;
+}
+// Whether the device holds n_cta blocks of a kernel in clusters of two at once (asked once per device): FDC_OK, or FDC_ERR_SHAPE (another build's launch).
+struct PairsPlaceable {
+    std::atomic<int> known[kMaxDevices] = {};         // 0: not asked; n + 1: that many clusters
+    int all(const void* kernel, int threads, size_t smem, int n_cta, SmemLimit& limit)
+    {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return FDC_ERR_SHAPE;
+        int n = known[dev].load(std::memory_order_relaxed);
+        if (n == 0) {
+            const int rc = raise_dynamic_smem(kernel, smem, limit);
+            if (rc) return rc;
+            cudaLaunchConfig_t one = {};
+            cudaLaunchAttribute at = cluster_of_two();
+            one.gridDim = dim3((unsigned)n_cta);
+            one.blockDim = dim3((unsigned)threads);
+            one.dynamicSmemBytes = smem;
+            one.attrs = &at;
+            one.numAttrs = 1;
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &one) != cudaSuccess) {
+                cudaGetLastError();
+                clusters = 0;
+            }
+            known[dev].store(n = clusters + 1, std::memory_order_relaxed);
+        }
+        return 2 * (n - 1) >= n_cta ? FDC_OK : FDC_ERR_SHAPE;
+    }
+};
 
 // ----------------------------------------------------------------------------------
 // device helpers

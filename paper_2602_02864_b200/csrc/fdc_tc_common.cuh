@@ -5,7 +5,6 @@
 
 #include <cudaTypedefs.h>
 
-#include <atomic>
 #include <climits>
 
 #include "fdc_attn_common.cuh"
@@ -716,43 +715,5 @@ __device__ __noinline__ uint64_t tile_seen_rows(const uint64_t* un, const uint64
     const uint32_t uh = __reduce_or_sync(0xffffffffu, (uint32_t)(um >> 32));
     return ((uint64_t)uh << 32) | ul;
 }
-
-inline cudaLaunchAttribute cluster_of_two()
-{
-    cudaLaunchAttribute a;
-    a.id = cudaLaunchAttributeClusterDimension;
-    a.val.clusterDim.x = 2;
-    a.val.clusterDim.y = a.val.clusterDim.z = 1;
-    return a;
-}
-// Whether the device holds n_cta blocks of a kernel in clusters of two at once (asked once per device): FDC_OK, or FDC_ERR_SHAPE (another build's launch).
-struct PairsPlaceable {
-    std::atomic<int> known[kMaxDevices] = {};         // 0: not asked; n + 1: that many clusters
-    int all(const void* kernel, int threads, size_t smem, int n_cta)
-    {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return FDC_ERR_SHAPE;
-        int n = known[dev].load(std::memory_order_relaxed);
-        if (n == 0) {
-            static size_t attr_smem[kMaxDevices] = {};
-            const int rc = raise_dynamic_smem(kernel, smem, attr_smem);
-            if (rc) return rc;
-            cudaLaunchConfig_t one = {};
-            cudaLaunchAttribute at = cluster_of_two();
-            one.gridDim = dim3((unsigned)n_cta);
-            one.blockDim = dim3((unsigned)threads);
-            one.dynamicSmemBytes = smem;
-            one.attrs = &at;
-            one.numAttrs = 1;
-            int clusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &one) != cudaSuccess) {
-                cudaGetLastError();
-                clusters = 0;
-            }
-            known[dev].store(n = clusters + 1, std::memory_order_relaxed);
-        }
-        return 2 * (n - 1) >= n_cta ? FDC_OK : FDC_ERR_SHAPE;
-    }
-};
 
 }  // namespace
