@@ -187,7 +187,6 @@ __device__ __forceinline__ void st_async2(uint32_t addr, uint32_t bar, const flo
 // Where the partials of a block's chunks arrive: [block of the cluster][chunk][16 columns], then [block][chunk] (m, l).
 // Chunk k (query row k / (D / 16), columns 16 (k mod D / 16) ..) belongs to block k mod nblk and is its (k / nblk)-th.
 constexpr int CHUNK_BYTES = 16 * 4 + 8;
-__host__ __device__ __forceinline__ int chunks_of_block(int chunks, int nblk) { return (chunks + nblk - 1) / nblk; }
 // The wait for them: false where it ran out (nothing of them may then be read).  A sender whose own wait runs out still sends what it
 // has, after its limit (a second or so) and what its earlier waits took.  This wait is flagged after eight such limits and then goes on as long
 // again, so that bytes still under way find the block's memory in place.  That is an assumption, not a guarantee: a sender can be later than

@@ -93,15 +93,16 @@ FDC_HD int run_begin(int rank, int nblk, int parts, Div&& div)
     const int each = (int)div((uint32_t)parts);
     return rank * each + (int)div((uint32_t)(rank * (parts - each * nblk)));
 }
-FDC_HD int run_begin(int rank, int nblk, int parts)
-{
-    return run_begin(rank, nblk, parts, [nblk](uint32_t x) { return x / (uint32_t)nblk; });
-}
 // Division of x < 2^28 by a small n (1 to 16) or of x < 2^24 by any n < 256: div_by(x, div_inverse(n)) = x / n.
 inline uint32_t div_inverse(int n) { return n > 1 ? (uint32_t)((1ull << 32) / (uint32_t)n + 1) : 0u; }
-#ifdef __CUDACC__
-__device__ __forceinline__ uint32_t div_by(uint32_t x, uint32_t inverse) { return inverse ? __umulhi(x, inverse) : x; }
+FDC_HD uint32_t div_by(uint32_t x, uint32_t inverse)
+{
+#ifdef __CUDA_ARCH__
+    return inverse ? __umulhi(x, inverse) : x;
+#else
+    return inverse ? (uint32_t)(((uint64_t)x * inverse) >> 32) : x;
 #endif
+}
 // Weights of the tcgen05 kernels' work split (the unit is a quarter of a tile inside the prefix).
 constexpr int W_PREFIX = 4;
 constexpr int W_MASKED = 6;          // a tile beyond the prefix (bitmap selects, V clean-up): measured about 1.5 prefix tiles

@@ -90,8 +90,9 @@ def test_runs_of_a_cluster_are_equal(tmp_path):
     src = tmp_path / "runs.cpp"
     src.write_text('#include "fdc_internal.h"\n#include <cstdio>\n'
                    'int main() { for (int n = 1; n <= 16; ++n) for (int parts = 0; parts <= 2200; ++parts) {\n'
-                   'if (fdc::run_begin(0, n, parts) != 0 || fdc::run_begin(n, n, parts) != parts) { printf("ends %d %d\\n", n, parts); return 1; }\n'
-                   'for (int r = 0; r < n; ++r) { const int k = fdc::run_begin(r + 1, n, parts) - fdc::run_begin(r, n, parts);\n'
+                   'const uint32_t inv = fdc::div_inverse(n); auto begin = [&](int r) { return fdc::run_begin(r, n, parts, [&](uint32_t x) { return fdc::div_by(x, inv); }); };\n'
+                   'if (begin(0) != 0 || begin(n) != parts) { printf("ends %d %d\\n", n, parts); return 1; }\n'
+                   'for (int r = 0; r < n; ++r) { const int k = begin(r + 1) - begin(r);\n'
                    'if (k < parts / n || k > (parts + n - 1) / n) { printf("run %d of %d: %d of %d\\n", r, n, k, parts); return 1; } } }\n'
                    'return 0; }\n')
     exe = tmp_path / "runs"

@@ -8,7 +8,7 @@ PROGRAM = """#include "fdc_internal.h"
 int main() {
     for (uint32_t n = 1; n < 256; ++n) {
         const uint32_t inv = fdc::div_inverse((int)n), top = n <= 16 ? 1u << 28 : 1u << 24;
-        auto by = [&](uint32_t x) { return inv ? (uint32_t)(((uint64_t)x * inv) >> 32) : x; };      // __umulhi
+        auto by = [&](uint32_t x) { return fdc::div_by(x, inv); };
         for (uint32_t k = 0; k < 20000; ++k)
             for (uint32_t x : {k, k * n, k * n + n - 1, top - 1 - k, (top - 1) / n * n - k % 2})
                 if (x < top && by(x) != x / n) { printf("%u / %u\\n", x, n); return 1; }
