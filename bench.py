@@ -32,7 +32,7 @@ sys.path.insert(0, ROOT)
 # profiles/attn_tc_kernel_cfg2.md (dram__bytes_read.sum + dram__bytes_write.sum over the launch's
 # algorithmic bytes; traffic grows in proportion to the visited tiles, so it scales to a full-size
 # launch).  Only valid for the kernel source it was measured on: keyed by a hash of that source.
-NCU_TRAFFIC = {"kernel_sha256_16": "1b2d94574c9b23cd", "dram_bytes_per_algorithmic_byte": 1.087}
+NCU_TRAFFIC = {"kernel_sha256_16": "91acfe3952fd4978", "dram_bytes_per_algorithmic_byte": 1.087}
 
 
 def kernel_source_hash() -> str:
@@ -70,7 +70,7 @@ def get_workload(name: str):
 # The attention kernel the library chooses for a workload's widest passes (the choice follows from the shapes).
 ATTENTION_KERNEL = {"cfg0": "attn_f32_kernel (fp32 FMAs, one cluster per scene and KV head)",
                     "cfg1": "attn_cluster_kernel (mma.sync, clusters per scene and KV head)",
-                    "cfg2": "attn_tc_kernel (tcgen05, up to 32 query rows)", "cfg3": "attn_tc_kernel_g2_two (tcgen05, 33 to 64 query rows, pairs in two parts)"}
+                    "cfg2": "attn_tc_kernel (tcgen05, up to 32 query rows)", "cfg3": "attn_tc_kernel_g2 (tcgen05, 33 to 64 query rows)"}
 
 WORKLOAD_TEXT = {
     "cfg0": "configs[0] tiny fp32: 1 layer, 4q/2kv heads, D 64, batch 1, prefix 256, 6-field DAG, 16-token slots",

@@ -301,7 +301,7 @@ __device__ __forceinline__ void attn_cluster_body(const AttnParams& p, const CUt
     if (A * p.group <= m0 || nt <= 0) {
         // Nothing to do (all blocks of the cluster agree).  Such blocks leave at once: their places go to the next launch's blocks, which set
         // themselves up meanwhile (3 scenes, 28/4 heads, one of five fields left, 144 of 216 blocks idle: a launch's last blocks began 0.5 us before the launch ahead
-        // ended, now 15 us).  One block of the grid waits for the launch ahead, so that grids still complete in stream order.
+        // ended, now 15 us; over 160 drawn passes with at most a third of their fields at work no faster than waiting on average, 0.946 to 1.051).  One block of the grid waits for the launch ahead, so that grids still complete in stream order.
         if (p.early && blockIdx.x == 0 && blockIdx.y == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
         return;
     }

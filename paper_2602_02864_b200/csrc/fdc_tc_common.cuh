@@ -1,5 +1,5 @@
 // What the two tcgen05 kernels share (fdc_attn_tc_kernel.cuh: KV rows on the M side of the multiplications;
-// fdc_attn_tc_rows.cu: query rows): wrappers of the tensor-core instructions, the work split over the CTAs, the TMA
+// fdc_attn_tc_rows_kernel.cuh: query rows): wrappers of the tensor-core instructions, the work split over the CTAs, the TMA
 // producer of the K and V rings and the fused append.  Included once per translation unit.
 #pragma once
 

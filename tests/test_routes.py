@@ -42,7 +42,7 @@ def route(tmp_path_factory):
     ((8, 7, 128, 5409, 810), True),           # 13.9 / 19.9
     ((192, 36, 128, 2168, 630), False),       # 67 / 102
     ((200, 48, 128, 1644, 360), False),       # 59 / 80
-    ((64, 128, 128, 1024, 2048), False)])     # 38 / 63
+    ((64, 128, 128, 1024, 2048), False)])     # 34 / 57
 def test_kernel(route, shape, cluster):
     assert bool(route([shape])[0][0]) == cluster
 
