@@ -24,7 +24,8 @@ int launch_tc_rows_two(const AttnParams& p, int head_dim, cudaStream_t st, int s
 // pass, fan, diamond, wide and free, fields of equal and of drawn lengths, 50 to 74 pairs, prefix 512 to 16384): half and more beyond 1.054 (181 templates, the
 // worst 0.984), 120 rows and more otherwise 1.028 (81, 0.990), 65 to 119 rows 1.009 (195, 0.974, 18 of them below 0.985), 33 to 64 rows 0.999 (190,
 // 0.957, 42 below 0.985; 8 scenes, 16 fields x 4 heads, prefix 8192: widest passes 1.02, later ones 0.98).  Within these lines single passes lie between 0.90 (most scenes
-// ended) and 1.2.
+// ended) and 1.2.  Up to 100 tiles per CTA (row form) and 200: longer lists in one part per CTA (70 to 74 pairs) gain 1.008 (72 templates, prefix 12288 to 24576, 120 rows and
+// more), single passes 0.95 to 1.045.
 //
 // us a layer, without / with: 64 pairs, 128 rows, 48 tiles 38.6 / 34.0; 64 rows, prefix 1024, 32 tiles 32.6 / 27.1.  With
 // 16 tiles a pair that start costs more than this gains (64 pairs, 35 rows 21.7 / 23.7), with equal shares nothing is
@@ -35,6 +36,7 @@ bool pairs_in_two_parts(int64_t pairs, int mmax, int P, int ntile_max, int n_cta
     if (mmax <= 32 || n_cta % 2 || 2 * pairs > n_cta || 3 * pairs <= n_cta || ntile_max < 32) return false;
     const int length = weighted_tiles(P / FDC_TILE_ROWS, ntile_max);
     if (mmax < 120 && 2 * W_PREFIX * (P / FDC_TILE_ROWS) > length) return false;
+    if (ntile_max * pairs >= (mmax > 64 ? 100 : 200) * (int64_t)n_cta) return false;
     return !equal_shares(pairs * (length + W_PAIR), (length + 1) / 2, n_cta, mmax);
 }
 

@@ -109,6 +109,7 @@ def split_of_whole_lists(scenes, hkv, mmax, P, nt, n_cta=148):
 @pytest.mark.parametrize("shape,two", [
     ((64, 128, 1024, 48), True),              # 38.6 / 34.0
     ((72, 128, 5632, 120), True),             # 69.3 / 65.0: 128 rows
+    ((74, 128, 24576, 416), False),           # 100 tiles per CTA and more: the whole template 1.00 to 1.01
     ((64, 64, 1024, 32), True),               # 32.6 / 27.1
     ((64, 36, 2048, 41), False),              # 25.6 / 26.7
     ((68, 63, 2048, 41), False),              # 9 fields x 7 heads, fan, the whole template 0.957
